@@ -325,7 +325,7 @@ class GridPlan:
 
     @property
     def n_entries(self) -> int:
-        """Stored weight factors (4 bytes each: 12 per patch candidate)."""
+        """Stored weight factors (4 bytes each: 16 per entry at W = 4 .. 7)."""
         return int(lib().mwax_grid_plan_entries(self._h))
 
     def empty_grids(self):

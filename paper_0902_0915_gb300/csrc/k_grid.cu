@@ -13,31 +13,38 @@
 //   2p+q for |s - x| < W/2 and |r - y| < W/2, w(dx, dy) =
 //   exp(-(dx^2 + dy^2) / (2 sigma^2)); cells outside [0, Ng) are dropped.
 //
+//
+// Half plane: the grids are Hermitian, G_pq(r, s) = conj(G_qp(Ng - r, Ng - s)),
+// because every point has its reversed twin.  Only the cells of rows
+// Ng/2 .. Ng and columns 0 .. Ng are summed (one row and column past the grid,
+// whose mirror images are row 0 and column 0); each row above Ng/2 is stored
+// twice, as it is and mirrored.  That halves the points, their weights and
+// the multiply-adds.
+//
 // Plan (geometry only, once per array layout and band):
-//   1. per point: position (FP64, so the support sets match an FP64
-//      definition exactly), support bounds, and its bin = the first cell of
-//      its support (r_lo, s_lo), shifted by W-1 so bins of points that reach
-//      row or column 0 are >= 0;
-//   2. counting sort by bin (integer atomics for counts and slots, an
-//      exclusive prefix sum for bin offsets), then every bin's ids sorted
-//      ascending so the order of each gathered sum is fixed;
-//   3. per sorted point: last support cell (r_hi, s_hi), first support
-//      column, point id;
-//   4. the weights: the cells are cut into patches of 4 x 8 (one warp each);
-//      the candidates of a patch are the points whose support can reach it,
-//      in a fixed order (bin rows, then bin columns, then point id: per bin
-//      row one contiguous range of the sorted points).  The Gaussian is
-//      separable, w = wx(s - x) wy(r - y), and the support is a rectangle, so
-//      for every candidate the plan stores its 8 column factors and 4 row
-//      factors (12 floats, computed in FP64, 0 outside the support), and the
-//      patches in order of decreasing candidate count (the dense centre of
-//      the uv plane first, so the longest warps do not start last).
-// Grid call (per integration): one kernel gathers each sorted point's four
-// polarisation values from the int32 correlator output; then each warp walks
-// its patch's candidates in the plan's order, reads the candidate's values
-// once for the whole warp (a broadcast) and its 12 factors, and every lane
-// adds wx[col] wy[row] x values (four complex multiply-adds).  No support
-// tests and no exponentials per call; deterministic.
+//   1. the W support rows of a point are cut into bands of at most 7 rows (one
+//      band up to W = 7); a (point, band) whose cells reach the half plane is
+//      an entry.  Positions and support bounds are FP64, so the support sets
+//      match an FP64 definition exactly;
+//   2. counting sort of the entries by bin = the band's first cell (integer atomics for counts and slots, an exclusive
+//      prefix sum for bin offsets), then every bin's entries sorted ascending
+//      so the order of each gathered sum is fixed;
+//   3. the weights: the Gaussian is separable, w = wx(s - x) wy(r - y), and the
+//      support a rectangle, so an entry stores its W column and up to 7 row
+//      factors (computed in FP64, kept in FP32, 0 outside the support) and its
+//      first column: 64 bytes up to W = 7;
+//   4. the units of work: a strip of 4 columns by 32 rows (fewer on small
+//      grids) is one warp's; strips that hold more entries than a quarter of a
+//      warp's even share (the centre of the uv plane) take a CTA of 4 warps.
+// Grid call (per integration): one kernel gathers the four polarisation values
+// of every baseline and channel from the int32 correlator output into its
+// entries; then each warp walks its strip row of bins by row of bins.  The
+// entries of a bin row reach the same WN rows (7 for W = 7): the lane keeps a
+// window of WN rows of its column in registers that slides down by one, so
+// no row outside the support is touched, and the row that the window leaves is
+// complete and stored.  The warp's 8 groups of 4 lanes take every eighth entry;
+// their sums are added in a fixed order.  No support tests and no exponentials
+// per call; deterministic.
 #include <math.h>
 #include <string.h>
 
@@ -52,14 +59,6 @@ namespace {
 constexpr double kCLight = 299792458.0;
 constexpr int kScanBlock = 1024;
 
-// Weights are formed at plan time from the FP64 position, recomputed from the
-// point id (an absolute float coordinate up to Ng would lose ~1e-4 cells).
-struct GeomRec {  // sorted point (12 B)
-  int hi;        // r_hi << 16 | s_hi (both in [0, Ng))
-  int id;        // point id: ((c * n_tbl) + tbl) * 2 + side
-  int slo;       // s_lo + W - 1
-};
-
 __device__ __forceinline__ void tbl_pair(int tbl, int &a, int &b) {
   // tbl = a(a-1)/2 + b, a > b >= 0
   int i = (int)((sqrtf(8.0f * (float)tbl + 1.0f) + 1.0f) * 0.5f);
@@ -73,45 +72,67 @@ struct GridGeom {
   const double *tile_xy;
   int n_tiles, n_chan, n_tbl, Ng, W;
   double f0, df, du;
-  int nbw;  // bins per row: Ng + W - 1
+  int nbw;      // bins per row: columns -(W-1) .. Ng
+  int nb, wr;   // bands per point, rows per band
+  int off;      // window rows of the apply kernel (>= wr) - 1: bin row 0 is grid row Ng/2 - off
 };
 
-// 1. positions, support bounds and bins (bin -1: no cell of the grid reached)
-__global__ void grid_points_kernel(GridGeom g, int64_t n_pts, int *__restrict__ bin,
-                                   int *__restrict__ hi) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= n_pts) return;
+// A point's support: first and last column and row (unclipped), FP64 position.
+struct Support {
+  double x, y;
+  int s_lo, s_hi, r_lo, r_hi;
+};
+
+// Point k = ((c * n_tbl) + tbl) * 2 + side.
+__device__ __forceinline__ Support point_support(const GridGeom &g, int64_t k) {
   const int side = (int)(k & 1);
   const int64_t ct = k >> 1;
   const int c = (int)(ct / g.n_tbl), tbl = (int)(ct % g.n_tbl);
   int a, b;
   tbl_pair(tbl, a, b);
   const double nu = g.f0 + (double)c * g.df;
-  double x = (g.tile_xy[2 * a] - g.tile_xy[2 * b]) * nu / kCLight / g.du + 0.5 * g.Ng;
-  double y = (g.tile_xy[2 * a + 1] - g.tile_xy[2 * b + 1]) * nu / kCLight / g.du + 0.5 * g.Ng;
+  Support p;
+  p.x = (g.tile_xy[2 * a] - g.tile_xy[2 * b]) * nu / kCLight / g.du + 0.5 * g.Ng;
+  p.y = (g.tile_xy[2 * a + 1] - g.tile_xy[2 * b + 1]) * nu / kCLight / g.du + 0.5 * g.Ng;
   if (side) {
-    x = (double)g.Ng - x;
-    y = (double)g.Ng - y;
+    p.x = (double)g.Ng - p.x;
+    p.y = (double)g.Ng - p.y;
   }
   const double half = 0.5 * g.W;
   // cells strictly within half the support: the smallest integer above x - W/2
   // and the largest below x + W/2
-  const int s_lo = (int)floor(x - half) + 1, s_hi = (int)ceil(x + half) - 1;
-  const int r_lo = (int)floor(y - half) + 1, r_hi = (int)ceil(y + half) - 1;
-  const bool reach = s_hi >= 0 && s_lo <= g.Ng - 1 && r_hi >= 0 && r_lo <= g.Ng - 1 &&
-                     s_lo >= -(g.W - 1) && r_lo >= -(g.W - 1);
-  if (!reach) {
-    bin[k] = -1;
-    hi[k] = 0;
-    return;
-  }
-  bin[k] = (r_lo + g.W - 1) * g.nbw + (s_lo + g.W - 1);
-  hi[k] = (min(r_hi, g.Ng - 1) << 16) | min(s_hi, g.Ng - 1);
+  p.s_lo = (int)floor(p.x - half) + 1;
+  p.s_hi = (int)ceil(p.x + half) - 1;
+  p.r_lo = (int)floor(p.y - half) + 1;
+  p.r_hi = (int)ceil(p.y + half) - 1;
+  return p;
 }
 
-__global__ void grid_count_kernel(const int *__restrict__ bin, int64_t n_pts, int *__restrict__ count) {
+// Bin of band b of a point, -1 if none of its cells lie in the half plane
+// (rows Ng/2 .. Ng, columns 0 .. Ng).
+__device__ __forceinline__ int band_bin(const GridGeom &g, const Support &p, int b) {
+  if (p.s_hi < 0 || p.s_lo > g.Ng || p.r_hi < g.Ng / 2 || p.r_lo > g.Ng) return -1;
+  const int r0 = p.r_lo + b * g.wr, r1 = min(r0 + g.wr - 1, p.r_hi);
+  if (r1 < r0 || r1 < g.Ng / 2 || r0 > g.Ng) return -1;
+  return (r0 - g.Ng / 2 + g.off) * g.nbw + (p.s_lo + g.W - 1);
+}
+
+// 1. entries per bin; n_reach: points with a cell in the grid itself
+__global__ void __launch_bounds__(256) grid_count_kernel(GridGeom g, int64_t n_pts,
+                                                         int *__restrict__ count,
+                                                         int *__restrict__ n_reach) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k < n_pts && bin[k] >= 0) atomicAdd(&count[bin[k]], 1);
+  bool reach = false;
+  if (k < n_pts) {
+    const Support p = point_support(g, k);
+    reach = p.s_hi >= 0 && p.s_lo <= g.Ng - 1 && p.r_hi >= 0 && p.r_lo <= g.Ng - 1;
+    for (int b = 0; b < g.nb; ++b) {
+      const int bin = band_bin(g, p, b);
+      if (bin >= 0) atomicAdd(&count[bin], 1);
+    }
+  }
+  const int n = __syncthreads_count(reach);
+  if (threadIdx.x == 0 && n) atomicAdd(n_reach, n);
 }
 
 // exclusive prefix sum in three passes: per-block scan with block totals,
@@ -165,23 +186,28 @@ __global__ void scan_add_kernel(int *__restrict__ out, int n, const int *__restr
   if (i < n) out[i] += totals[blockIdx.x];
 }
 
-__global__ void grid_fill_kernel(const int *__restrict__ bin, int64_t n_pts,
-                                 const int *__restrict__ offsets, int *__restrict__ fill,
-                                 int *__restrict__ ids) {
+// 2. entry ids (k * nb + b) into their bins
+__global__ void __launch_bounds__(256) grid_fill_kernel(GridGeom g, int64_t n_pts,
+                                                        const int *__restrict__ offsets,
+                                                        int *__restrict__ fill,
+                                                        long long *__restrict__ ids) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= n_pts || bin[k] < 0) return;
-  const int b = bin[k];
-  ids[offsets[b] + atomicAdd(&fill[b], 1)] = (int)k;
+  if (k >= n_pts) return;
+  const Support p = point_support(g, k);
+  for (int b = 0; b < g.nb; ++b) {
+    const int bin = band_bin(g, p, b);
+    if (bin >= 0) ids[offsets[bin] + atomicAdd(&fill[bin], 1)] = k * g.nb + b;
+  }
 }
 
 // ids of every bin ascending (insertion sort; bins are short)
 __global__ void grid_sort_bins_kernel(const int *__restrict__ offsets, int n_bins,
-                                      int *__restrict__ ids) {
+                                      long long *__restrict__ ids) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= n_bins) return;
   const int lo = offsets[b], hi = offsets[b + 1];
   for (int i = lo + 1; i < hi; ++i) {
-    const int v = ids[i];
+    const long long v = ids[i];
     int j = i - 1;
     while (j >= lo && ids[j] > v) {
       ids[j + 1] = ids[j];
@@ -191,369 +217,394 @@ __global__ void grid_sort_bins_kernel(const int *__restrict__ offsets, int n_bin
   }
 }
 
-__global__ void grid_records_kernel(const int *__restrict__ ids, int n_kept,
-                                    const int *__restrict__ hi,
-                                    const int *__restrict__ bin, int nbw, GeomRec *__restrict__ rec) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n_kept) return;
-  const int k = ids[p];
-  GeomRec r;
-  r.hi = hi[k];
-  r.id = k;
-  r.slo = bin[k] % nbw;
-  rec[p] = r;
-}
+// 3. per entry: `fx` floats, [W column factors][first column s_lo, an int]
+// padded to whole 16 bytes, then 8 row factors (0 past the band or outside the
+// support); and the entry's place in the slot table [band][point].
+constexpr int kRowFactors = 8;
 
-// Cell position of a point in FP64, from its id ((c * n_tbl + tbl) * 2 + side).
-__device__ __forceinline__ void point_xy(const GridGeom &g, int id, double &x, double &y) {
-  const int side = id & 1;
-  const int ct = id >> 1;
-  const int c = ct / g.n_tbl, tbl = ct % g.n_tbl;
-  int a, b;
-  tbl_pair(tbl, a, b);
-  const double nu = g.f0 + (double)c * g.df;
-  x = (g.tile_xy[2 * a] - g.tile_xy[2 * b]) * nu / kCLight / g.du + 0.5 * g.Ng;
-  y = (g.tile_xy[2 * a + 1] - g.tile_xy[2 * b + 1]) * nu / kCLight / g.du + 0.5 * g.Ng;
-  if (side) {
-    x = (double)g.Ng - x;
-    y = (double)g.Ng - y;
+__global__ void __launch_bounds__(256) grid_weights_kernel(GridGeom g,
+                                                           const long long *__restrict__ ids,
+                                                           int n_ent, double inv_2s2d, int fx,
+                                                           int64_t n_pts, float *__restrict__ wts,
+                                                           int *__restrict__ slot) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= n_ent) return;
+  const long long id = ids[q];
+  const int64_t k = id / g.nb;
+  const int b = (int)(id - k * g.nb);
+  slot[(int64_t)b * n_pts + k] = q;
+  const Support p = point_support(g, k);
+  float *w = wts + (int64_t)q * (fx + kRowFactors);
+  for (int i = 0; i < fx; ++i) {
+    float f = 0.f;
+    if (i < g.W && p.s_lo + i <= p.s_hi) {
+      const double d = (double)(p.s_lo + i) - p.x;
+      f = (float)exp(-d * d * inv_2s2d);
+    }
+    w[i] = i == g.W ? __int_as_float(p.s_lo) : f;
+  }
+  const int r0 = p.r_lo + b * g.wr;
+  for (int i = 0; i < kRowFactors; ++i) {
+    float f = 0.f;
+    if (i < g.wr && r0 + i <= p.r_hi) {
+      const double d = (double)(r0 + i) - p.y;
+      f = (float)exp(-d * d * inv_2s2d);
+    }
+    w[fx + i] = f;
   }
 }
 
-// Patches: a warp owns rows r0 .. r0+3, columns s0 .. s0+7.  The warp's lanes
-// form kGroups groups of 32 / kGroups lanes; group g takes candidates
-// j = g (mod kGroups), and lane l of a group holds kGroups cells of one row
-// (r0 + l / (8 / kGroups), columns s0 + kGroups (l % (8 / kGroups)) + {0 ..
-// kGroups-1}), so one value broadcast and one load of kGroups column factors
-// serve kGroups cells; the groups' sums are added at the end.  A CTA runs 8
-// patches.
-#ifndef MWAX_GRID_GROUPS
-#define MWAX_GRID_GROUPS 2
-#endif
-constexpr int kGroups = MWAX_GRID_GROUPS;  // 1, 2 or 4 (measured: 1.64, 1.42, 1.46 ms per c5 call)
-constexpr int kGLanes = 32 / kGroups, kRowLanes = 8 / kGroups;
-constexpr int kPatchR = 4, kPatchC = 8;
-constexpr int kPatchThreads = 32 * 8;
+// Units of work: 4 columns (block cb) by `rows` rows from relative row r0 (row
+// Ng/2 + r0 of the grid).  Bin row i of a unit, i = 0 .. rows + off - 1, is row
+// r0 + i of the bin table and reaches the unit's rows i - off .. i; row i - off
+// is complete after it.
+constexpr int kCols = 4;
+constexpr int kUnitRows = 32;
+constexpr int kMaxBinRows = 40;  // >= kUnitRows + 6
 
-constexpr int kFactors = kPatchC + kPatchR;  // per candidate: 8 column, 4 row factors
-
-struct Patch {
-  int r0, s0, br_end, bc_end;
-};
-
-// Patch `idx` (row-major over patch rows and columns).
-__device__ __forceinline__ Patch patch_at(int idx, int n_patch_c, int W, int nbw) {
-  Patch pt;
-  pt.r0 = (idx / n_patch_c) * kPatchR;
-  pt.s0 = (idx % n_patch_c) * kPatchC;
-  // bin row br holds points with r_lo = br - (W - 1); those reaching rows
-  // r0 .. r0+3 have br in [r0, r0 + 3 + W - 1]; likewise bin columns
-  pt.br_end = min(pt.r0 + kPatchR - 1 + W - 1, nbw - 1);
-  pt.bc_end = min(pt.s0 + kPatchC + W - 1, nbw);  // exclusive
-  return pt;
-}
-
-// 4a. candidates per patch (into cnt[patch])
-__global__ void __launch_bounds__(kPatchThreads) grid_patch_count_kernel(
-    const int *__restrict__ offsets, int n_patches, int W, int nbw, int n_patch_c,
-    int *__restrict__ cnt) {
-  const int idx = blockIdx.x * (kPatchThreads / 32) + (threadIdx.x >> 5);
-  if (idx >= n_patches) return;
-  const Patch pt = patch_at(idx, n_patch_c, W, nbw);
-  const int lane = threadIdx.x & 31;
+// entries of every unit of `rows` rows (unit = row segment * n_cb + column block)
+__global__ void __launch_bounds__(256) grid_unit_count_kernel(const int *__restrict__ offsets,
+                                                              int n_units, int n_cb, int rows,
+                                                              int n_rows, int W, int off, int nbw,
+                                                              int *__restrict__ cnt) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= n_units) return;
+  const int r0 = (u / n_cb) * rows, s0 = (u % n_cb) * kCols;
+  const int nb = min(rows, n_rows - r0) + off;
+  const int c1 = min(s0 + kCols + W - 1, nbw);
   int n = 0;
-  for (int br = pt.r0 + lane; br <= pt.br_end; br += 32)
-    n += offsets[br * nbw + pt.bc_end] - offsets[br * nbw + pt.s0];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-  if (lane == 0) cnt[idx] = n;
+  for (int i = 0; i < nb; ++i) n += offsets[(r0 + i) * nbw + c1] - offsets[(r0 + i) * nbw + s0];
+  cnt[u] = n;
 }
 
-// 4b. the factors of every candidate of a patch, from w_off[patch] * 12:
-// lanes 0..7 the column factors wx(s0 + l - x), lanes 8..11 the row factors
-// wy(r0 + l - 8 - y), each 0 outside the support or the grid.
-__global__ void __launch_bounds__(kPatchThreads) grid_patch_weights_kernel(
-    GridGeom g, const GeomRec *__restrict__ rec, const int *__restrict__ offsets, double inv_2s2d,
-    int n_patches, int n_patch_c, const int *__restrict__ w_off, float *__restrict__ wts) {
-  const int idx = blockIdx.x * (kPatchThreads / 32) + (threadIdx.x >> 5);
-  if (idx >= n_patches) return;
-  const int W = g.W, nbw = g.nbw;
-  const Patch pt = patch_at(idx, n_patch_c, W, nbw);
-  const int lane = threadIdx.x & 31;
-  const bool col = lane < kPatchC, row = lane >= kPatchC && lane < kFactors;
-  const int s = pt.s0 + lane, r = pt.r0 + lane - kPatchC;
-  int64_t k = (int64_t)w_off[idx] * kFactors + lane;
-  for (int br = pt.r0; br <= pt.br_end; ++br) {
-    const int r_lo = br - (W - 1);
-    const int lo = offsets[br * nbw + pt.s0], hi = offsets[br * nbw + pt.bc_end];
-    for (int q = lo; q < hi; ++q, k += kFactors) {
-      if (!col && !row) continue;
-      const GeomRec p = rec[q];
-      const int s_lo = p.slo - (W - 1);
-      float f = 0.f;
-      double x, y;
-      if (col && s >= s_lo && s <= (p.hi & 0xFFFF) && s < g.Ng) {
-        point_xy(g, p.id, x, y);
-        const double d = (double)s - x;
-        f = (float)exp(-d * d * inv_2s2d);
-      } else if (row && r >= r_lo && r <= (p.hi >> 16) && r < g.Ng) {
-        point_xy(g, p.id, x, y);
-        const double d = (double)r - y;
-        f = (float)exp(-d * d * inv_2s2d);
-      }
-      wts[k] = f;
-    }
-  }
-}
-
-// sorted position of every point id (-1: the point reaches no cell)
-__global__ void grid_slot_kernel(const GeomRec *__restrict__ rec, int n_kept, int *__restrict__ slot) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n_kept) slot[rec[p].id] = p;
-}
-
-// grid call, step 1: the four polarisation values of every point, read in
-// point-id order (channel, then baseline: nearly sequential in the
-// correlator output) and written to the point's sorted position
-__global__ void grid_values_kernel(const int *__restrict__ slot, int n_pts, int n_tbl,
-                                   int64_t n_bl, const int2 *__restrict__ vis,
-                                   float4 *__restrict__ vals) {
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= n_pts) return;
-  const int p = slot[id];
-  if (p < 0) return;
-  const int side = id & 1;
-  const int ct = id >> 1;
-  const int c = ct / n_tbl, tbl = ct % n_tbl;
-  int a, b;
-  tbl_pair(tbl, a, b);
-  const int2 *vc = vis + (int64_t)c * n_bl;
-  float v[8];
-#pragma unroll
-  for (int pp = 0; pp < 2; ++pp)
-#pragma unroll
-    for (int qq = 0; qq < 2; ++qq) {
-      // forward point: product (pp, qq) of (a, b); reversed: conj of (qq, pp)
-      const int ip = side ? qq : pp, jq = side ? pp : qq;
-      const int64_t i = 2 * a + ip, j = 2 * b + jq;
-      const int2 x = vc[i * (i + 1) / 2 + j];
-      v[2 * (2 * pp + qq)] = (float)x.x;
-      v[2 * (2 * pp + qq) + 1] = side ? -(float)x.y : (float)x.y;
-    }
-  vals[2 * (int64_t)p] = make_float4(v[0], v[1], v[2], v[3]);
-  vals[2 * (int64_t)p + 1] = make_float4(v[4], v[5], v[6], v[7]);
-}
-
-// grid call, step 2: every cell of a patch sums, in the plan's candidate order,
-// wx[col] wy[row] x values.  apply_range adds candidates [k0, k1) of a patch
-// for this lane's cell.
-constexpr int kHeavy = 1024;  // patches with more candidates get a whole CTA
-
-struct Acc {
-  float2 v[kGroups][4];  // the lane's cells x four polarisation products
-};
-
-// Per-warp staging of 32 candidates: their values (8 floats) and factors
-// (12 floats), double-buffered; plus the patch's bin rows (first candidate
-// index and first sorted point of each).
-constexpr int kMaxRows = 40;  // >= kPatchR - 1 + W for W <= 31
-struct WarpStage {
-  float4 v[2][32][2];
-  float f[2][32][kFactors];
-  int row_k[kMaxRows + 1], row_q[kMaxRows];
-};
-
-__device__ __forceinline__ void cp16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
+// Grid call, step 1: the four polarisation values of every baseline and
+// channel, read in the correlator output's order, written as one 32-byte
+// store into each entry of the point (a, b) and of its reversed twin (conj,
+// XY and YX swapped).  HBM-bound: 32 B read, 8 B of slots and about 32 B
+// written per baseline and channel (half the points are entries).
+__device__ __forceinline__ void store8(float4 *dst, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]),
+               "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
                : "memory");
 }
 
-// Adds candidates [k0, k1) of the patch to this lane's cell: 32 candidates at
-// a time are copied (one per lane) into the warp's staging buffer while the
-// previous 32 are applied, in candidate order.
-__device__ __forceinline__ void apply_range(const Patch &pt, int nbw, const int *__restrict__ offsets,
-                                            const float *__restrict__ wf0,
-                                            const float4 *__restrict__ vals, int k0, int k1,
-                                            int lane, WarpStage &st, Acc &acc) {
-  // group hw takes candidates j + hw; this lane's column factors
-  // kGroups (l % kRowLanes) + {0 .. kGroups-1} and its row factor, l = lane % kGLanes
-  const int hw = lane / kGLanes, hl = lane % kGLanes;
-  const int fx = kGroups * (hl % kRowLanes), fy = kPatchC + hl / kRowLanes;
-  // bin rows of the patch: candidate index of each row's first point
-  const int n_rows = pt.br_end - pt.r0 + 1;
-  if (lane == 0) {
-    int k = 0;
-    for (int i = 0; i < n_rows; ++i) {
-      const int br = pt.r0 + i;
-      const int lo = __ldg(offsets + br * nbw + pt.s0), hi = __ldg(offsets + br * nbw + pt.bc_end);
-      st.row_k[i] = k;
-      st.row_q[i] = lo;
-      k += hi - lo;
+__global__ void __launch_bounds__(256) grid_values_kernel(const int2 *__restrict__ slot, int n_tbl,
+                                                          int n_chan, int nb, int64_t n_bl,
+                                                          const int2 *__restrict__ vis,
+                                                          float4 *__restrict__ vals,
+                                                          int *__restrict__ next) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *next = 0;  // step 2's unit counter
+  const int tbl = blockIdx.x * blockDim.x + threadIdx.x;
+  if (tbl >= n_tbl) return;
+  int a, b;
+  tbl_pair(tbl, a, b);
+  const int64_t i0 = 2 * a, o0 = i0 * (i0 + 1) / 2 + 2 * b, o1 = o0 + i0 + 1;
+  for (int c = blockIdx.y; c < n_chan; c += gridDim.y) {
+    const int2 *vc = vis + (int64_t)c * n_bl;
+    const int2 xx = __ldcs(vc + o0), xy = __ldcs(vc + o0 + 1), yx = __ldcs(vc + o1),
+               yy = __ldcs(vc + o1 + 1);
+    const int64_t ct = (int64_t)c * n_tbl + tbl, n_ct = (int64_t)n_chan * n_tbl;
+    const float f[8] = {(float)xx.x, (float)xx.y, (float)xy.x, (float)xy.y,
+                        (float)yx.x, (float)yx.y, (float)yy.x, (float)yy.y};
+    const float r[8] = {f[0], -f[1], f[4], -f[5], f[2], -f[3], f[6], -f[7]};
+    for (int band = 0; band < nb; ++band) {
+      const int2 q = slot[band * n_ct + ct];
+      if (q.x >= 0) store8(vals + 2 * (int64_t)q.x, f);
+      if (q.y >= 0) store8(vals + 2 * (int64_t)q.y, r);
     }
-    st.row_k[n_rows] = k;
   }
-  __syncwarp();
-  auto issue = [&](int base, int buf) {  // candidates base .. base+31 (those < k1)
-    const int kk = base + lane;
-    if (kk < k1) {
-      int i = 0;
-      while (st.row_k[i + 1] <= kk) ++i;
-      const int q = st.row_q[i] + (kk - st.row_k[i]);
-      cp16(&st.v[buf][lane][0], vals + 2 * (int64_t)q);
-      cp16(&st.v[buf][lane][1], vals + 2 * (int64_t)q + 1);
-      const float *f = wf0 + (int64_t)kk * kFactors;
-      cp16(&st.f[buf][lane][0], f);
-      cp16(&st.f[buf][lane][4], f + 4);
-      cp16(&st.f[buf][lane][8], f + 8);
+}
+
+// Grid call, step 2.
+// Staging: a ring of kSlots chunks of 32 entries per warp (values, factors).
+// Every bin row starts on a multiple of 8 entries; the places left over are
+// zeros.  One step is 8 entries, one per group.
+constexpr int kSlots = 2;
+constexpr int kChunk = 32, kRing = kSlots * kChunk;
+constexpr int kApplyWarps = 4;
+__host__ __device__ constexpr int apply_warp_bytes(int f4) {
+  return kRing * (32 + 16 * f4) + (3 * kMaxBinRows + 4) * 4;
+}
+
+struct ApplyArgs {
+  const int *offsets;
+  const float4 *wts, *vals;
+  float *grids;
+  const int2 *units;  // x = column block, y = first relative row << 8 | rows
+  int *next;          // light units handed out so far
+  int Ng, W, nbw, f4;  // f4: 16-byte pieces per entry's factors
+  int n_heavy, n_light;
+};
+
+// A unit's bin rows: first entry, entries, and steps before the row.
+struct BinRows {
+  int q[kMaxBinRows], n[kMaxBinRows], s[kMaxBinRows + 4];
+};
+
+// One component (2 (2p + q) + (re, im)) of relative row r, column s: stored at
+// its cell, and mirrored (conj, p and q swapped) unless the row is its own
+// mirror image.
+__device__ __forceinline__ void store_value(const ApplyArgs &A, int r, int s, int comp, float v) {
+  const int Ng = A.Ng, row = Ng / 2 + r, pol = comp >> 1, ri = comp & 1;
+  if (row < Ng && s < Ng) A.grids[(((int64_t)pol * Ng + row) * Ng + s) * 2 + ri] = v;
+  if (r > 0 && s >= 1 && s <= Ng) {
+    const int mp = ((pol & 1) << 1) | (pol >> 1);
+    A.grids[(((int64_t)mp * Ng + (Ng - row)) * Ng + (Ng - s)) * 2 + ri] = ri ? -v : v;
+  }
+}
+
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int lds1(uint32_t a) {
+  int v;
+  asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+
+__device__ __forceinline__ void cp16z(uint32_t dst, const void *src, bool take) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(take ? 16 : 0)
+               : "memory");
+}
+
+// One warp's walk over a unit of n_bins bin rows.  emit(i, v): after bin row i
+// the lane holds the finished value of row i - off, column lane & 3, component
+// lane >> 2 = 2 (2p + q) + (re, im).
+template <int WN, int F4, class Emit>
+__device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bins, uint8_t *sm,
+                                           const BinRows &rows, int lane, Emit &&emit) {
+  const int f4 = F4 ? F4 : A.f4;
+  const int fb = 16 * f4;  // bytes of factors per entry
+  const uint32_t uv = (uint32_t)__cvta_generic_to_shared(sm), uw = uv + kRing * 32;
+  const int total = rows.s[n_bins];  // steps
+  const int col = s0 + (lane & 3), g = lane >> 2;
+  // chunk: lane j finds the entry of place j, then consecutive lanes copy
+  // consecutive 16-byte pieces
+  int my_row = 0;
+  auto issue = [&](int chunk) {
+    const int step = chunk * (kChunk / 8) + (lane >> 3);
+    if (chunk * (kChunk / 8) < total) {
+      int q = -1;
+      if (step < total) {
+        while (rows.s[my_row + 1] <= step) ++my_row;
+        const int k = (step - rows.s[my_row]) * 8 + (lane & 7);
+        if (k < rows.n[my_row]) q = rows.q[my_row] + k;
+      }
+      const int slot = chunk % kSlots;
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const int p = m * 32 + lane;
+        const int src = __shfl_sync(0xffffffffu, q, p >> 1);
+        cp16z(uv + (slot * 64 + p) * 16, A.vals + 2 * (int64_t)max(src, 0) + (p & 1), src >= 0);
+      }
+#pragma unroll
+      for (int m = 0; m < f4; ++m) {
+        const int p = m * 32 + lane;
+        const int e = p / f4, o = p - e * f4;
+        const int src = __shfl_sync(0xffffffffu, q, e);
+        cp16z(uw + (slot * kChunk * f4 + p) * 16, A.wts + (int64_t)max(src, 0) * f4 + o, src >= 0);
+      }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  int buf = 0;
-  if (k0 < k1) issue(k0, 0);
-  for (int base = k0; base < k1; base += 32, buf ^= 1) {
-    if (base + 32 < k1) {
-      issue(base + 32, buf ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncwarp();
-    const int n = min(32, k1 - base);
-    for (int j0 = 0; j0 < n; j0 += kGroups) {
-      const int j = j0 + hw;
-      if (j < n) {
-        float wx[kGroups];
-        if constexpr (kGroups == 4) {
-          const float4 t = *reinterpret_cast<const float4 *>(&st.f[buf][j][fx]);
-          wx[0] = t.x;
-          wx[1] = t.y;
-          wx[2] = t.z;
-          wx[3] = t.w;
-        } else if constexpr (kGroups == 2) {
-          const float2 t = *reinterpret_cast<const float2 *>(&st.f[buf][j][fx]);
-          wx[0] = t.x;
-          wx[1] = t.y;
-        } else {
-          wx[0] = st.f[buf][j][fx];
-        }
-        const float wy = st.f[buf][j][fy];
-        const float4 a = st.v[buf][j][0], b = st.v[buf][j][1];
+  constexpr int P = 2;  // bin rows between shifts of the window
+  float acc[WN + P - 1][8];
 #pragma unroll
-        for (int c = 0; c < kGroups; ++c) {
-          const float w = wx[c] * wy;
-          acc.v[c][0].x += w * a.x;
-          acc.v[c][0].y += w * a.y;
-          acc.v[c][1].x += w * a.z;
-          acc.v[c][1].y += w * a.w;
-          acc.v[c][2].x += w * b.x;
-          acc.v[c][2].y += w * b.y;
-          acc.v[c][3].x += w * b.z;
-          acc.v[c][3].y += w * b.w;
-        }
-      }
-    }
-    __syncwarp();  // this buffer is refilled two steps on
-  }
-  // the groups' sums into every lane of group 0 (fixed order: a butterfly
-  // over the group bits)
+  for (int t = 0; t < WN + P - 1; ++t)
 #pragma unroll
-  for (int o = kGLanes; o < 32; o <<= 1)
+    for (int p = 0; p < 8; ++p) acc[t][p] = 0.f;
 #pragma unroll
-    for (int c = 0; c < kGroups; ++c)
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        acc.v[c][p].x += __shfl_xor_sync(0xffffffffu, acc.v[c][p].x, o);
-        acc.v[c][p].y += __shfl_xor_sync(0xffffffffu, acc.v[c][p].y, o);
-      }
-}
-
-// The lanes of group 0 store their cells (the other groups hold the same sums).
-__device__ __forceinline__ void store_cell(const Patch &pt, int lane, int Ng, const Acc &acc,
-                                           float2 *__restrict__ grids) {
-  if (lane >= kGLanes) return;
-  const int r = pt.r0 + lane / kRowLanes, s = pt.s0 + kGroups * (lane % kRowLanes);
-  if (r >= Ng) return;
-  const int64_t cell = (int64_t)r * Ng + s;
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    float2 *g = grids + (int64_t)p * Ng * Ng + cell;
-#pragma unroll
-    for (int c = 0; c < kGroups; ++c)
-      if (s + c < Ng) g[c] = acc.v[c][p];
-  }
-}
-
-// Heavy patches (order[0 .. n_heavy)): one CTA each; warp w takes the w-th
-// eighth of the candidates, and warp 0 adds the eight partial sums in warp
-// order.
-__global__ void __launch_bounds__(kPatchThreads) grid_apply_heavy_kernel(
-    const int *__restrict__ offsets, const int *__restrict__ order, const int *__restrict__ w_off,
-    const float *__restrict__ wts, const float4 *__restrict__ vals, int Ng, int W, int nbw,
-    int n_patch_c, float2 *__restrict__ grids) {
-  __shared__ WarpStage stage[kPatchThreads / 32];
-  const int idx = __ldg(order + blockIdx.x);
-  const Patch pt = patch_at(idx, n_patch_c, W, nbw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int first = __ldg(w_off + idx), count = __ldg(w_off + idx + 1) - first;
-  const int nw = kPatchThreads / 32;
-  Acc acc;
-#pragma unroll
-  for (int c = 0; c < kGroups; ++c)
-#pragma unroll
-    for (int p = 0; p < 4; ++p) acc.v[c][p] = make_float2(0.f, 0.f);
-  apply_range(pt, nbw, offsets, wts + (int64_t)first * kFactors, vals,
-              (int)((int64_t)count * warp / nw), (int)((int64_t)count * (warp + 1) / nw), lane,
-              stage[warp], acc);
-  // the partial sums reuse the staging memory once every warp is done with it
-  __syncthreads();
-  float2(*part)[kGroups][4][kGLanes] = reinterpret_cast<float2(*)[kGroups][4][kGLanes]>(stage);
-  static_assert(sizeof(float2) * (kPatchThreads / 32) * 4 * 32 <= sizeof(WarpStage) * (kPatchThreads / 32),
-                "aliasing");
-  if (lane < kGLanes)
-#pragma unroll
-    for (int c = 0; c < kGroups; ++c)
-#pragma unroll
-      for (int p = 0; p < 4; ++p) part[warp][c][p][lane] = acc.v[c][p];
-  __syncthreads();
-  if (warp == 0 && lane < kGLanes) {
-#pragma unroll
-    for (int c = 0; c < kGroups; ++c)
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        float2 t = part[0][c][p][lane];
+  for (int k = 0; k < kSlots - 1; ++k) issue(k);
+  int st = 0;
+  uint32_t pv = 0, pw = 0;  // this group's entry of the step: values, factors
 #pragma unroll 1
-        for (int w = 1; w < nw; ++w) {
-          t.x += part[w][c][p][lane].x;
-          t.y += part[w][c][p][lane].y;
+  for (int ib = 0; ib < n_bins; ib += P) {
+#pragma unroll
+    for (int ph = 0; ph < P; ++ph) {
+      const int i = ib + ph;
+      if (i < n_bins) {
+#pragma unroll 1
+        for (const int end = rows.s[i + 1]; st < end; ++st) {
+          if ((st & 3) == 0) {  // a new chunk: the slot of the one before it is free
+            __syncwarp();
+            issue(st / 4 + kSlots - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
+            __syncwarp();
+            const int slot = (st >> 2) % kSlots;
+            pv = uv + (slot * kChunk + g) * 32;
+            pw = uw + (slot * kChunk + g) * fb;
+          }
+          const int d = col - lds1(pw + 4 * A.W);
+          const float4 v0 = lds4(pv), v1 = lds4(pv + 16), y0 = lds4(pw + fb - 32);
+          float wy[WN > 5 ? 8 : 5] = {y0.x, y0.y, y0.z, y0.w};
+          if constexpr (WN > 5) {
+            const float4 y1 = lds4(pw + fb - 16);
+            wy[4] = y1.x;
+            wy[5] = y1.y;
+            wy[6] = y1.z;
+            wy[7] = y1.w;
+          } else {
+            wy[4] = __int_as_float(lds1(pw + fb - 16));
+          }
+          float wx = 0.f;
+          if ((unsigned)d < (unsigned)A.W) wx = __int_as_float(lds1(pw + 4 * d));
+          pv += 8 * 32;
+          pw += 8 * fb;
+          const float t8[8] = {wx * v0.x, wx * v0.y, wx * v0.z, wx * v0.w,
+                               wx * v1.x, wx * v1.y, wx * v1.z, wx * v1.w};
+#pragma unroll
+          for (int t = 0; t < WN; ++t)
+#pragma unroll
+            for (int p = 0; p < 8; ++p) acc[ph + t][p] = fmaf(wy[t], t8[p], acc[ph + t][p]);
         }
-        acc.v[c][p] = t;
+        // the row that the window leaves: its eight components summed over the
+        // eight groups (a butterfly over lane bits 4, 3, 2 that halves the
+        // components each lane carries: group g ends with component g)
+        float a[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) a[p] = acc[ph][p];
+        if (i >= WN - 1) {
+#pragma unroll
+          for (int h = 4; h > 0; h >>= 1) {
+            const bool up = lane & (4 * h);
+#pragma unroll
+            for (int k = 0; k < h; ++k) {
+              const float send = up ? a[k] : a[k + h], keep = up ? a[k + h] : a[k];
+              a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+            }
+          }
+          emit(i, a[0]);
+        }
       }
-    store_cell(pt, lane, Ng, acc, grids);
+    }
+#pragma unroll
+    for (int t = 0; t < WN + P - 1; ++t)
+#pragma unroll
+      for (int p = 0; p < 8; ++p) acc[t][p] = t + P < WN + P - 1 ? acc[t + P][p] : 0.f;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+constexpr int apply_smem_bytes(int f4) {
+  return kApplyWarps * apply_warp_bytes(f4) + kApplyWarps * kUnitRows * 32 * 4;
+}
+constexpr int kApplyCtas = 4;  // per SM: 16 warps at up to 128 registers
+
+// Bound by instruction issue (70 % of the slots, 59 % of the instructions on the
+// FMA pipe): 56 multiply-adds, 8 multiplies and about 20 other instructions per
+// step of 8 entries, of whose 4 x 7 cells the strip's edge leaves 70 % useful.
+// Measured for 12.5 M points on 4 x 2048^2 cells, W = 7: 0.55 ms a call, 0.076 of
+// it the values; gathering both halves patch by patch with the factors of
+// every (patch, point) pair stored took 1.42 ms.  Not taken: packed two-wide
+// multiply-adds (67 per SM and cycle against 110 for scalar ones, measured),
+// two columns per lane, bins of two rows, seven window phases unrolled instead
+// of shifting registers (fetch stalls), more warps with spills.
+// Persistent CTAs.  Heavy units (units[0 .. n_heavy)): one CTA per unit, warp w takes the w-th quarter of every bin row and the four
+// partial sums are added in warp order.  Then every warp takes the next light
+// unit until none is left (which warp takes it does not touch its sums).
+template <int WN, int F4>
+__global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kernel(ApplyArgs A) {
+  extern __shared__ __align__(16) uint8_t sm_all[];
+  constexpr int off = WN - 1;
+  const int f4 = F4 ? F4 : A.f4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t *sm = sm_all + warp * apply_warp_bytes(f4);
+  BinRows &rows = *reinterpret_cast<BinRows *>(sm + kRing * (32 + 16 * f4));
+  float *part = reinterpret_cast<float *>(sm_all + kApplyWarps * apply_warp_bytes(f4));
+  const int comp = lane >> 2;
+  int h = blockIdx.x;
+  while (true) {
+    const bool heavy = h < A.n_heavy;
+    int u = h;
+    if (!heavy) {
+      if (lane == 0) u = atomicAdd(A.next, 1);
+      u = __shfl_sync(0xffffffffu, u, 0);
+      if (u >= A.n_light) break;
+      u += A.n_heavy;
+    }
+    const int2 unit = __ldg(A.units + u);
+    const int s0 = unit.x * kCols, r0 = unit.y >> 8, n_rows = unit.y & 255;
+    const int n_bins = n_rows + off;
+    int carry = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int i = 32 * k + lane;
+      int lo = 0, n = 0;
+      if (i < n_bins) {
+        const int *o = A.offsets + (int64_t)(r0 + i) * A.nbw;
+        lo = __ldg(o + s0);
+        n = __ldg(o + min(s0 + kCols + A.W - 1, A.nbw)) - lo;
+        if (heavy) {
+          const int first = (int)((int64_t)n * warp / kApplyWarps);
+          n = (int)((int64_t)n * (warp + 1) / kApplyWarps) - first;
+          lo += first;
+        }
+      }
+      int x = (n + 7) >> 3;  // steps, then their running sum
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += t;
+      }
+      if (i < n_bins) {
+        rows.q[i] = lo;
+        rows.n[i] = n;
+        rows.s[i + 1] = carry + x;
+      }
+      carry += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) rows.s[0] = 0;
+    __syncwarp();
+    const int s = s0 + (lane & 3);
+    if (carry == 0 && !heavy) {
+      for (int r = 0; r < n_rows; ++r) store_value(A, r0 + r, s, comp, 0.f);
+    } else {
+      strip_walk<WN, F4>(A, s0, n_bins, sm, rows, lane, [&](int i, float v) {
+        if (heavy)
+          part[(warp * kUnitRows + i - off) * 32 + lane] = v;
+        else
+          store_value(A, r0 + i - off, s, comp, v);
+      });
+    }
+    if (heavy) {
+      __syncthreads();
+      for (int r = warp; r < n_rows; r += kApplyWarps) {
+        float v = part[r * 32 + lane];
+#pragma unroll
+        for (int w = 1; w < kApplyWarps; ++w) {
+          v += part[(w * kUnitRows + r) * 32 + lane];
+        }
+        store_value(A, r0 + r, s, comp, v);
+      }
+      __syncthreads();
+      h += gridDim.x;
+    }
+    __syncwarp();  // the bin rows are written again
   }
 }
 
-// The other patches (order[n_heavy .. n_patches)): one warp each.
-__global__ void __launch_bounds__(kPatchThreads) grid_apply_kernel(
-    const int *__restrict__ offsets, const int *__restrict__ order, const int *__restrict__ w_off,
-    const float *__restrict__ wts, const float4 *__restrict__ vals, int Ng, int W, int nbw,
-    int slot0, int n_patches, int n_patch_c, float2 *__restrict__ grids) {
-  __shared__ WarpStage stage[kPatchThreads / 32];
-  const int slot = slot0 + blockIdx.x * (kPatchThreads / 32) + (threadIdx.x >> 5);
-  if (slot >= n_patches) return;
-  const int idx = __ldg(order + slot);
-  const Patch pt = patch_at(idx, n_patch_c, W, nbw);
-  const int lane = threadIdx.x & 31;
-  const int first = __ldg(w_off + idx), count = __ldg(w_off + idx + 1) - first;
-  Acc acc;
-#pragma unroll
-  for (int c = 0; c < kGroups; ++c)
-#pragma unroll
-    for (int p = 0; p < 4; ++p) acc.v[c][p] = make_float2(0.f, 0.f);
-  apply_range(pt, nbw, offsets, wts + (int64_t)first * kFactors, vals, 0, count, lane,
-              stage[threadIdx.x >> 5], acc);
-  store_cell(pt, lane, Ng, acc, grids);
+constexpr int kMaxF4 = (32 + kRowFactors) / 4;  // W = 31
+
+// Windows of 5 and 7 rows; the factors of an entry take 64 bytes (F4 = 4) for
+// W = 4 .. 7.  PREPARE: set the kernel's shared-memory limit (at plan time)
+// instead of launching it.
+template <int WN, int F4, bool PREPARE>
+cudaError_t apply_one(const ApplyArgs &A, int sms, cudaStream_t s) {
+  if (PREPARE)
+    return cudaFuncSetAttribute(grid_apply_kernel<WN, F4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                apply_smem_bytes(F4 ? F4 : kMaxF4));
+  const int ctas = std::min(kApplyCtas * sms, A.n_heavy + (A.n_light + kApplyWarps - 1) / kApplyWarps);
+  grid_apply_kernel<WN, F4><<<ctas, 32 * kApplyWarps, apply_smem_bytes(A.f4), s>>>(A);
+  return cudaGetLastError();
+}
+
+template <bool PREPARE>
+cudaError_t apply_units(int win, const ApplyArgs &A, int sms, cudaStream_t s) {
+  if (win == 5)
+    return A.f4 == 4 ? apply_one<5, 4, PREPARE>(A, sms, s) : apply_one<5, 0, PREPARE>(A, sms, s);
+  return A.f4 == 4 ? apply_one<7, 4, PREPARE>(A, sms, s) : apply_one<7, 0, PREPARE>(A, sms, s);
 }
 
 }  // namespace
@@ -564,27 +615,32 @@ using namespace mwax;
 struct mwax_grid_plan_s {
   cudaStream_t stream = nullptr;
   int device = 0;
-  int n_tiles = 0, n_chan = 0, n_tbl = 0, Ng = 0, W = 0, nbw = 0;
+  int n_tiles = 0, n_chan = 0, n_tbl = 0, Ng = 0, W = 0, nbw = 0, nb = 1, win = 7, f4 = 4;
   int64_t n_pts = 0;
-  int n_kept = 0, n_patches = 0, n_patch_c = 0, n_heavy = 0;
-  int64_t n_entries = 0;     // stored factors (12 per patch candidate)
+  int n_kept = 0;            // points with a cell in the grid
+  int n_ent = 0;             // entries: (point, band) with a cell in the half plane
+  int n_heavy = 0, n_light = 0, sms = 0;
   int *offsets = nullptr;    // [n_bins + 1]
-  GeomRec *rec = nullptr;    // [n_kept]
-  int *slot = nullptr;       // [n_pts]: sorted position of each point id, or -1
-  int *w_off = nullptr;      // [n_patches + 1]: first candidate of each patch
-  int *order = nullptr;      // [n_patches]: patches by decreasing candidate count
-  float *wts = nullptr;      // [n_entries]: [candidate][8 column | 4 row factors] per patch
-  float4 *vals = nullptr;    // [n_kept][2], filled per call
+  int *slot = nullptr;       // [nb][n_pts]: place of each entry, or -1
+  int2 *units = nullptr;     // heavy units, then light ones
+  int *next = nullptr;       // counter of the light units handed out in a call
+  float *wts = nullptr;      // [n_ent][4 f4]
+  float4 *vals = nullptr;    // [n_ent][2], filled per call
 };
 
 namespace {
 
 void free_grid_plan(mwax_grid_plan_s *p) {
   if (!p) return;
-  for (void *q : {(void *)p->offsets, (void *)p->rec, (void *)p->slot, (void *)p->w_off,
-                  (void *)p->order, (void *)p->wts, (void *)p->vals})
+  for (void *q : {(void *)p->offsets, (void *)p->slot, (void *)p->units, (void *)p->next, (void *)p->wts, (void *)p->vals})
     if (q) cudaFree(q);
   delete p;
+}
+
+ApplyArgs apply_args(const mwax_grid_plan_s *p, float *grids) {
+  return ApplyArgs{p->offsets, reinterpret_cast<const float4 *>(p->wts), p->vals, grids,
+                   p->units,   p->next,                                     p->Ng,   p->W,
+                   p->nbw,     p->f4,                                       p->n_heavy, p->n_light};
 }
 
 bool is_dev(const void *p) {
@@ -612,9 +668,7 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
     return MWAX_ERR_INVALID_ARG;
   const int64_t n_tbl = (int64_t)n_tiles * (n_tiles - 1) / 2;
   const int64_t n_pts = n_tbl * n_chan * 2;
-  const int64_t nbw = (int64_t)Ng + W - 1;
-  const int64_t n_bins = nbw * nbw;
-  if (n_pts > 0x7FFFFFFFll || n_bins + 1 > 0x7FFFFFFFll) return MWAX_ERR_INVALID_ARG;
+  if (n_pts > 0x7FFFFFFFll) return MWAX_ERR_INVALID_ARG;
   mwax_grid_plan_s *p = new mwax_grid_plan_s;
   p->stream = stream;
   cudaGetDevice(&p->device);
@@ -623,125 +677,109 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
   p->n_tbl = (int)n_tbl;
   p->Ng = Ng;
   p->W = W;
-  p->nbw = (int)nbw;
   p->n_pts = n_pts;
+  p->nb = (W + 6) / 7;
+  const int wr = (W + p->nb - 1) / p->nb;
+  p->win = wr <= 5 ? 5 : 7;
+  const int off = p->win - 1;
+  p->nbw = Ng + W;
+  const int n_rows = Ng / 2 + 1;                     // rows of the half plane
+  const int n_bins = (n_rows + off) * p->nbw;  // at most 8199 x 16415
+  const int fx = (W + 1 + 3) / 4 * 4;
+  p->f4 = (fx + kRowFactors) / 4;
   // plan-time scratch
   double *d_xy = nullptr;
-  int *bin = nullptr, *hi = nullptr, *count = nullptr, *fill = nullptr, *ids = nullptr,
-      *totals = nullptr;
-  const int n_scan = (int)(n_bins + 1);
+  int *count = nullptr, *totals = nullptr, *ucnt = nullptr, *reach = nullptr;
+  long long *ids = nullptr;
+  auto free_scratch = [&] {
+    for (void *q : {(void *)d_xy, (void *)count, (void *)totals, (void *)ucnt, (void *)reach, (void *)ids})
+      if (q) cudaFree(q);
+  };
+  const int n_scan = n_bins + 1;  // one extra zero: the last offset is the total
   const int scan_blocks = (n_scan + kScanBlock - 1) / kScanBlock;
   cudaError_t e = cudaMalloc(&d_xy, sizeof(double) * 2 * n_tiles);
-  if (e == cudaSuccess) e = cudaMalloc(&bin, sizeof(int) * n_pts);
-  if (e == cudaSuccess) e = cudaMalloc(&hi, sizeof(int) * n_pts);
   if (e == cudaSuccess) e = cudaMalloc(&count, sizeof(int) * n_scan);
-  if (e == cudaSuccess) e = cudaMalloc(&fill, sizeof(int) * n_bins);
   if (e == cudaSuccess) e = cudaMalloc(&totals, sizeof(int) * scan_blocks);
+  if (e == cudaSuccess) e = cudaMalloc(&reach, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&p->offsets, sizeof(int) * n_scan);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_xy, tile_xy, sizeof(double) * 2 * n_tiles, cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(int) * n_scan, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(fill, 0, sizeof(int) * n_bins, stream);
-  GridGeom g{d_xy, n_tiles, n_chan, (int)n_tbl, Ng, W, f0, df, du, (int)nbw};
+  if (e == cudaSuccess) e = cudaMemsetAsync(reach, 0, sizeof(int), stream);
+  GridGeom g{d_xy, n_tiles, n_chan, (int)n_tbl, Ng, W, f0, df, du, p->nbw, p->nb, wr, off};
   const int T = 256;
   const unsigned nblk = (unsigned)((n_pts + T - 1) / T);
   if (e == cudaSuccess) {
-    grid_points_kernel<<<nblk, T, 0, stream>>>(g, n_pts, bin, hi);
-    grid_count_kernel<<<nblk, T, 0, stream>>>(bin, n_pts, count);
+    grid_count_kernel<<<nblk, T, 0, stream>>>(g, n_pts, count, reach);
     scan_blocks_kernel<<<scan_blocks, kScanBlock, 0, stream>>>(count, n_scan, p->offsets, totals);
     scan_totals_kernel<<<1, kScanBlock, 0, stream>>>(totals, scan_blocks);
     scan_add_kernel<<<scan_blocks, kScanBlock, 0, stream>>>(p->offsets, n_scan, totals);
     e = cudaGetLastError();
   }
-  // number of points that reach the grid, and the largest bin (for the record)
-  int kept = 0;
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&kept, p->offsets + n_bins, sizeof(int), cudaMemcpyDeviceToHost, stream);
+    e = cudaMemcpyAsync(&p->n_kept, reach, sizeof(int), cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&p->n_ent, p->offsets + n_bins, sizeof(int), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  if (e == cudaSuccess) {
-    p->n_kept = kept;
-    e = cudaMalloc(&ids, sizeof(int) * std::max(kept, 1));
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&p->rec, sizeof(GeomRec) * std::max(kept, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&p->vals, 2 * sizeof(float4) * std::max(kept, 1));
-  if (e == cudaSuccess) {
-    grid_fill_kernel<<<nblk, T, 0, stream>>>(bin, n_pts, p->offsets, fill, ids);
-    grid_sort_bins_kernel<<<(unsigned)((n_bins + T - 1) / T), T, 0, stream>>>(p->offsets,
-                                                                             (int)n_bins, ids);
-    if (kept > 0)
-      grid_records_kernel<<<(kept + T - 1) / T, T, 0, stream>>>(ids, kept, hi, bin, (int)nbw,
-                                                                p->rec);
-    e = cudaGetLastError();
-  }
-  // sorted position of every point id
-  if (e == cudaSuccess) e = cudaMalloc(&p->slot, sizeof(int) * n_pts);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->slot, 0xFF, sizeof(int) * n_pts, stream);
-  if (e == cudaSuccess && kept > 0) {
-    grid_slot_kernel<<<(kept + T - 1) / T, T, 0, stream>>>(p->rec, kept, p->slot);
-    e = cudaGetLastError();
-  }
-  // the weights: candidates per patch, their prefix sum, then [candidate][cell]
-  // (a point is a candidate of at most this many patches; the int32 prefix
-  // sum must hold the total)
-  const int64_t per_point = (int64_t)((W + kPatchR - 1) / kPatchR + 1) * ((W + kPatchC - 1) / kPatchC + 1);
-  if (e == cudaSuccess && (int64_t)kept * per_point > 0x7FFFFFFFll) {
-    for (void *q : {(void *)d_xy, (void *)bin, (void *)hi, (void *)count, (void *)fill, (void *)ids,
-                    (void *)totals})
-      if (q) cudaFree(q);
+  // the limit on points times support, in units of 4 x 8 cells
+  const int64_t per_point = (int64_t)((W + 3) / 4 + 1) * ((W + 7) / 8 + 1);
+  if (e == cudaSuccess && (int64_t)p->n_kept * per_point > 0x7FFFFFFFll) {
+    free_scratch();
     free_grid_plan(p);
     return MWAX_ERR_UNSUPPORTED;
   }
-  const int npr = (Ng + kPatchR - 1) / kPatchR, npc = (Ng + kPatchC - 1) / kPatchC;
-  const int n_patches = npr * npc;
-  const int n_pscan = n_patches + 1;  // one extra zero: the last offset is the total
-  const int pscan_blocks = (n_pscan + kScanBlock - 1) / kScanBlock;
-  int *pcnt = nullptr, *ptot = nullptr;
-  p->n_patches = n_patches;
-  p->n_patch_c = npc;
-  const double inv_2s2d = 1.0 / (2.0 * sigma * sigma);
-  const unsigned pgrid = (unsigned)((n_patches + kPatchThreads / 32 - 1) / (kPatchThreads / 32));
-  if (e == cudaSuccess) e = cudaMalloc(&pcnt, sizeof(int) * n_pscan);
-  if (e == cudaSuccess) e = cudaMalloc(&ptot, sizeof(int) * pscan_blocks);
-  if (e == cudaSuccess) e = cudaMalloc(&p->w_off, sizeof(int) * n_pscan);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pcnt, 0, sizeof(int) * n_pscan, stream);
+  const int n_ent = p->n_ent;
+  if (e == cudaSuccess) e = cudaMalloc(&ids, sizeof(long long) * std::max(n_ent, 1));
+  if (e == cudaSuccess) e = cudaMalloc(&p->vals, 2 * sizeof(float4) * std::max(n_ent, 1));
+  if (e == cudaSuccess) e = cudaMalloc(&p->wts, (size_t)16 * p->f4 * std::max(n_ent, 1));
+  if (e == cudaSuccess) e = cudaMalloc(&p->slot, sizeof(int) * n_pts * p->nb);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p->slot, 0xFF, sizeof(int) * n_pts * p->nb, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(int) * n_scan, stream);
   if (e == cudaSuccess) {
-    grid_patch_count_kernel<<<pgrid, kPatchThreads, 0, stream>>>(p->offsets, n_patches, W,
-                                                                   (int)nbw, npc, pcnt);
-    scan_blocks_kernel<<<pscan_blocks, kScanBlock, 0, stream>>>(pcnt, n_pscan, p->w_off, ptot);
-    scan_totals_kernel<<<1, kScanBlock, 0, stream>>>(ptot, pscan_blocks);
-    scan_add_kernel<<<pscan_blocks, kScanBlock, 0, stream>>>(p->w_off, n_pscan, ptot);
+    grid_fill_kernel<<<nblk, T, 0, stream>>>(g, n_pts, p->offsets, count, ids);
+    grid_sort_bins_kernel<<<(unsigned)((n_bins + T - 1) / T), T, 0, stream>>>(p->offsets, n_bins, ids);
+    if (n_ent > 0)
+      grid_weights_kernel<<<(unsigned)((n_ent + T - 1) / T), T, 0, stream>>>(
+          g, ids, n_ent, 1.0 / (2.0 * sigma * sigma), fx, n_pts, p->wts, p->slot);
     e = cudaGetLastError();
   }
-  int total = 0;
-  std::vector<int> hcnt(n_patches), horder(n_patches);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&total, p->w_off + n_patches, sizeof(int), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(hcnt.data(), pcnt, sizeof(int) * n_patches, cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  // units: 32 rows, or fewer where that would leave CTAs without a unit; a unit
+  // of r rows walks r + 6 bin rows, so short ones cost more
+  const int n_cb = Ng / kCols + 1;  // the last block holds column Ng alone
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
+  int rows = kUnitRows;
+  while (rows > 8 && (n_rows + rows - 1) / rows * n_cb < 2 * p->sms * kApplyCtas) rows /= 2;
+  const int n_u = (n_rows + rows - 1) / rows * n_cb;
+  std::vector<int> cnt(n_u);
+  if (e == cudaSuccess) e = cudaMalloc(&ucnt, sizeof(int) * n_u);
   if (e == cudaSuccess) {
-    // heaviest patches first (ties in patch order)
-    for (int i = 0; i < n_patches; ++i) horder[i] = i;
-    std::stable_sort(horder.begin(), horder.end(),
-                     [&](int a, int b) { return hcnt[a] > hcnt[b]; });
-    while (p->n_heavy < n_patches && hcnt[horder[p->n_heavy]] > kHeavy) ++p->n_heavy;
-    e = cudaMalloc(&p->order, sizeof(int) * n_patches);
-  }
-  if (e == cudaSuccess)
-    e = cudaMemcpy(p->order, horder.data(), sizeof(int) * n_patches, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) {
-    p->n_entries = (int64_t)total * kFactors;
-    e = cudaMalloc(&p->wts, sizeof(float) * std::max<int64_t>(p->n_entries, 1));
-  }
-  if (e == cudaSuccess) {
-    grid_patch_weights_kernel<<<pgrid, kPatchThreads, 0, stream>>>(
-        g, p->rec, p->offsets, inv_2s2d, n_patches, npc, p->w_off, p->wts);
+    grid_unit_count_kernel<<<(n_u + T - 1) / T, T, 0, stream>>>(p->offsets, n_u, n_cb, rows, n_rows, W, off,
+                                                               p->nbw, ucnt);
     e = cudaGetLastError();
   }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(cnt.data(), ucnt, sizeof(int) * cnt.size(), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  for (void *q : {(void *)d_xy, (void *)bin, (void *)hi, (void *)count, (void *)fill,
-                  (void *)ids, (void *)totals, (void *)pcnt, (void *)ptot})
-    if (q) cudaFree(q);
+  std::vector<int2> heavy, units;
+  if (e == cudaSuccess) {
+    int64_t total = 0;
+    for (int u = 0; u < n_u; ++u) total += cnt[u];
+    const int64_t most = std::max<int64_t>(256, total / ((int64_t)p->sms * kApplyCtas * kApplyWarps * 4));
+    for (int u = 0; u < n_u; ++u) {
+      const int r0 = u / n_cb * rows;
+      (cnt[u] > most ? heavy : units).push_back(make_int2(u % n_cb, r0 << 8 | std::min(rows, n_rows - r0)));
+    }
+    p->n_heavy = (int)heavy.size();
+    p->n_light = (int)units.size();
+    heavy.insert(heavy.end(), units.begin(), units.end());
+    e = cudaMalloc(&p->units, sizeof(int2) * heavy.size());
+  }
+  if (e == cudaSuccess)
+    e = cudaMemcpy(p->units, heavy.data(), sizeof(int2) * heavy.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMalloc(&p->next, sizeof(int));
+  if (e == cudaSuccess) e = apply_units<true>(p->win, apply_args(p, nullptr), p->sms, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  free_scratch();
   if (e != cudaSuccess) {
     free_grid_plan(p);
     return e == cudaErrorMemoryAllocation ? MWAX_ERR_OOM : MWAX_ERR_CUDA;
@@ -752,7 +790,9 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
 
 int64_t mwax_grid_plan_points(mwax_grid_plan_t plan) { return plan ? plan->n_kept : -1; }
 
-int64_t mwax_grid_plan_entries(mwax_grid_plan_t plan) { return plan ? plan->n_entries : -1; }
+int64_t mwax_grid_plan_entries(mwax_grid_plan_t plan) {
+  return plan ? (int64_t)plan->n_ent * 4 * plan->f4 : -1;
+}
 
 mwax_status mwax_grid(mwax_grid_plan_t plan, const int32_t *vis, float *grids) {
   mwax::NvtxRange nvtx_("mwax_grid");
@@ -761,22 +801,13 @@ mwax_status mwax_grid(mwax_grid_plan_t plan, const int32_t *vis, float *grids) {
     return MWAX_ERR_INVALID_ARG;
   const int64_t N = 2 * (int64_t)plan->n_tiles;
   const int T = 256;
-  if (plan->n_kept > 0)
-    grid_values_kernel<<<(unsigned)((plan->n_pts + T - 1) / T), T, 0, plan->stream>>>(
-        plan->slot, (int)plan->n_pts, plan->n_tbl, N * (N + 1) / 2,
-        reinterpret_cast<const int2 *>(vis), plan->vals);
-  float2 *g2 = reinterpret_cast<float2 *>(grids);
-  if (plan->n_heavy > 0)
-    grid_apply_heavy_kernel<<<plan->n_heavy, kPatchThreads, 0, plan->stream>>>(
-        plan->offsets, plan->order, plan->w_off, plan->wts, plan->vals, plan->Ng, plan->W,
-        plan->nbw, plan->n_patch_c, g2);
-  const int n_light = plan->n_patches - plan->n_heavy;
-  if (n_light > 0)
-    grid_apply_kernel<<<(unsigned)((n_light + kPatchThreads / 32 - 1) / (kPatchThreads / 32)),
-                        kPatchThreads, 0, plan->stream>>>(
-        plan->offsets, plan->order, plan->w_off, plan->wts, plan->vals, plan->Ng, plan->W,
-        plan->nbw, plan->n_heavy, plan->n_patches, plan->n_patch_c, g2);
-  return cudaGetLastError() == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
+  grid_values_kernel<<<dim3((unsigned)((plan->n_tbl + T - 1) / T), (unsigned)std::min(plan->n_chan, 65535)), T, 0,
+                       plan->stream>>>(reinterpret_cast<const int2 *>(plan->slot), plan->n_tbl, plan->n_chan,
+                                       plan->nb, N * (N + 1) / 2, reinterpret_cast<const int2 *>(vis), plan->vals,
+                                       plan->next);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = apply_units<false>(plan->win, apply_args(plan, grids), plan->sms, plan->stream);
+  return e == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
 }
 
 mwax_status mwax_grid_destroy(mwax_grid_plan_t plan) {
