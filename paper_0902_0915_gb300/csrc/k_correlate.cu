@@ -237,16 +237,19 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t addr) {
 
 // Operand tile of each sample width: its descriptor and the descriptor
 // offsets (16-byte units) of the K slices re 0, re 1, im 0, im 1.
+// (and the factor that makes an accumulator value an integer)
 template <int BITS>
 struct Op;
 template <>
 struct Op<8> {  // binary16, K-major
+  static constexpr float units = 1.f;
   static constexpr bool mn = false;
   static constexpr uint64_t re0 = 0, re1 = 2, im0 = 4, im1 = 6;
   static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return sw128_desc(addr); }
 };
 template <>
 struct Op<4> {  // E4M3, MN-major
+  static constexpr float units = kNib4Units;
   static constexpr bool mn = true;
   static constexpr uint64_t re0 = 0, re1 = 256, im0 = 512, im1 = 768;
   static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return sw128_mn_desc(addr); }
@@ -499,9 +502,9 @@ __device__ __forceinline__ void fused_store(uint8_t *tile, int ct, const uint4 (
     const int off = t * kRowBytes + ((ch ^ (t & 7)) << 4);
     const uint4 v = w[m];
     *reinterpret_cast<uint4 *>(tile + off) =
-        make_uint4(nib4_to_e4m3_f16(v.x), nib4_to_e4m3_f16(v.y), nib4_to_e4m3_f16(v.z), nib4_to_e4m3_f16(v.w));
+        make_uint4(nib4_re(v.x), nib4_re(v.y), nib4_re(v.z), nib4_re(v.w));
     *reinterpret_cast<uint4 *>(tile + 64 * kRowBytes + off) =
-        make_uint4(nib4_to_e4m3_f16(v.x >> 4), nib4_to_e4m3_f16(v.y >> 4), nib4_to_e4m3_f16(v.z >> 4), nib4_to_e4m3_f16(v.w >> 4));
+        make_uint4(nib4_im(v.x), nib4_im(v.y), nib4_im(v.z), nib4_im(v.w));
   }
 }
 
@@ -510,7 +513,12 @@ __device__ __forceinline__ void fused_store(uint8_t *tile, int ct, const uint4 (
 // two-entry flag so all eight warps take the same branch), convert, release
 // the accumulator, store the item's lower-triangle visibilities.  false: a
 // wait ran out (every warp stops).
-template <int KIND>
+template <int BITS>
+__device__ __forceinline__ int acc_int(uint32_t v) {
+  return __float2int_rn(__uint_as_float(v) * Op<BITS>::units);
+}
+
+template <int BITS, int KIND>
 __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it, uint32_t n_it,
                                            uint32_t tfull, uint32_t tempty, uint32_t tmem_base,
                                            uint8_t *stg, volatile int *abort_flag,
@@ -565,8 +573,8 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
     if constexpr (KIND == MWAX_KIND_EXACT) {
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
-        vre[k] = (uint32_t)__float2int_rn(__uint_as_float(vre[k]));
-        vim[k] = (uint32_t)__float2int_rn(__uint_as_float(vim[k]));
+        vre[k] = (uint32_t)acc_int<BITS>(vre[k]);
+        vim[k] = (uint32_t)acc_int<BITS>(vim[k]);
       }
     }
 #pragma unroll
@@ -590,12 +598,12 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
 
 // The same as a separate call (fused pair mode: the converters' state stays
 // out of the epilogue's register allocation).
-template <int KIND>
+template <int BITS, int KIND>
 __device__ __noinline__ bool drain_item_call(const KParams &p, const PairItem &it, uint32_t n_it,
                                              uint32_t tfull, uint32_t tempty, uint32_t tmem_base,
                                              uint8_t *stg, volatile int *abort_flag,
                                              volatile int *epi_flag, int warp, int lane, int epi0) {
-  return drain_item<KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag, warp,
+  return drain_item<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag, warp,
                           lane, epi0);
 }
 
@@ -798,10 +806,10 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
     uint8_t *stg = epi_smem + (warp - Sh::epi0) * kEpiStageBytes;
     auto drain = [&](const PairItem &it, uint32_t n_it) -> bool {
       if constexpr (FUSED)
-        return drain_item_call<KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag,
+        return drain_item_call<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag,
                                      epi_flag, warp, lane, Sh::epi0);
       else
-        return drain_item<KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag,
+        return drain_item<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag,
                                 warp, lane, Sh::epi0);
     };
     uint32_t n_it = 0;
@@ -1187,7 +1195,7 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
 #pragma unroll
           for (int k = 0; k < 32; ++k) {
             if constexpr (KIND == MWAX_KIND_EXACT) {
-              const int x = __float2int_rn(__uint_as_float(v[k]));
+              const int x = acc_int<BITS>(v[k]);
               tot[chunk * 32 + k] = (uint32_t)((int)tot[chunk * 32 + k] + x);
             } else {
               tot[chunk * 32 + k] = v[k];

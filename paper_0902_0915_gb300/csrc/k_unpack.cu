@@ -10,7 +10,7 @@
 //        inputs, holding [ re(t0) .. re(t0+31) | im(t0) .. im(t0+31) ]: one
 //        row of a 128-byte-swizzled K-major shared-memory tile, 16 KB per
 //        tile and time block.  The transpose goes through shared memory.
-//   4-bit samples (S = 64, FP8 E4M3, exact for |v| <= 16), MN-major:
+//   4-bit samples (S = 64, FP8 E4M3 codes of v x 2^-9, see mwax_nib4.h), MN-major:
 //        op[chan][kb][plane][s][n_rows] bytes, n_rows = 128 x tiles: row
 //        (plane 0, s) holds the re codes of every input at sample 64 kb + s
 //        (inputs contiguous, the order they arrive in), row (plane 1, s) the
@@ -234,19 +234,17 @@ __global__ void __launch_bounds__(256) unpack4_mn_kernel(const uint8_t *__restri
         const int tk = tu[k];
         uint8_t *dst = op + ((cu[k] * kb + (tk >> 6)) * 128 + (tk & 63)) * (int64_t)n_rows + (int64_t)g * VEC;
         if constexpr (VEC == 16) {
-          const uint4 re = make_uint4(nib4_to_e4m3_f16(w[k].x), nib4_to_e4m3_f16(w[k].y),
-                                      nib4_to_e4m3_f16(w[k].z), nib4_to_e4m3_f16(w[k].w));
-          const uint4 im = make_uint4(nib4_to_e4m3_f16(w[k].x >> 4), nib4_to_e4m3_f16(w[k].y >> 4),
-                                      nib4_to_e4m3_f16(w[k].z >> 4), nib4_to_e4m3_f16(w[k].w >> 4));
+          const uint4 re = make_uint4(nib4_re(w[k].x), nib4_re(w[k].y), nib4_re(w[k].z), nib4_re(w[k].w));
+          const uint4 im = make_uint4(nib4_im(w[k].x), nib4_im(w[k].y), nib4_im(w[k].z), nib4_im(w[k].w));
           *reinterpret_cast<uint4 *>(dst) = re;
           *reinterpret_cast<uint4 *>(dst + plane) = im;
         } else if constexpr (VEC == 4) {
-          *reinterpret_cast<uint32_t *>(dst) = nib4_to_e4m3_f16(w[k]);
-          *reinterpret_cast<uint32_t *>(dst + plane) = nib4_to_e4m3_f16(w[k] >> 4);
+          *reinterpret_cast<uint32_t *>(dst) = nib4_re(w[k]);
+          *reinterpret_cast<uint32_t *>(dst + plane) = nib4_im(w[k]);
         } else {
           const uint32_t b = w[k];
-          dst[0] = (uint8_t)nib4_to_e4m3_f16(b);
-          dst[plane] = (uint8_t)nib4_to_e4m3_f16(b >> 4);
+          dst[0] = (uint8_t)nib4_re(b);
+          dst[plane] = (uint8_t)nib4_im(b);
         }
       }
     }
