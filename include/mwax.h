@@ -106,9 +106,10 @@ typedef struct {
                               shared memory, so no operand buffer and no unpack pass
                               (4-bit exact samples in one exact segment with n_inputs a
                               multiple of 16 -- every job of a batch plan --, else
-                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 where it applies and
-                              n_inputs <= 256 (every job), else 3 where it applies,
-                              else 1                                                      */
+                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 where it applies and, for
+                              every job, n_inputs <= 256 or the launch's operand tiles
+                              exceed 64 MB and the integration has at least 256 samples
+                              per 128-input tile, else 3 where it applies, else 1         */
   int32_t pipeline;        /* tuning: 1 = unpack then correlate each channel group on the
                               plan's stream, 2 = unpack the next group (second stream,
                               second scratch buffer) while the current group correlates,

@@ -76,20 +76,25 @@ constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB
 // bubble in the tensor pipe, so the narrow shape takes three blocks (24
 // MMAs) per wait and per commit: two stages of 96 KB.
 // 3, fused pair: the pair mode for 4-bit samples with the unpack folded in:
-// the eight epilogue warps also convert: they read the packed samples from
-// global memory and write the E4M3 operand tiles into the stages themselves
-// (no operand buffer in HBM, no unpack pass), and drain each item's
-// accumulator after its last stage.
+// sixteen warps read the packed samples from global memory and write the E4M3
+// operand tiles into the stages themselves (no operand buffer in HBM, no unpack
+// pass), and drain each item's accumulator after its last stage.  Bound by the
+// shared memory that the MMAs' operands, 93 (N = 256) or 122 (N = 128) bytes of
+// 128 a cycle, and the converters' stores share.  256 inputs x 768 channels x
+// 20,000 samples: 1.87 ms (1.28 ms of MMA work at 2.07 GHz); eight converting
+// warps with an L2 prefetch ahead of them took 2.12, a ring of packed samples in
+// shared memory 1.94 (its extra reads and writes slow the MMAs), one-block
+// stages 2.2, two-block stages for items of two tiles 2.0.
 constexpr int kModeNarrow = 0, kModeWide = 1, kModePair = 2, kModePairFused = 3;
 constexpr int kEpiStageBytes = 32 * 128;  // pair mode: one warp's 32 rows x 16 (re, im) words
 
 template <int MODE>
 struct Shape {
   static constexpr bool pair = MODE == kModePair || MODE == kModePairFused;
-  static constexpr int warps = MODE == kModeWide ? 12 : 10;
+  static constexpr int warps = MODE == kModeWide ? 12 : MODE == kModePairFused ? 18 : 10;
   // warps 2 .. 2+conv_warps-1: B' builders (wide only)
   static constexpr int conv_warps = MODE == kModeWide ? 2 : 0;
-  static constexpr int epi0 = 2 + conv_warps;  // 8 epilogue warps from here to the last
+  static constexpr int epi0 = 2 + conv_warps;  // 8 epilogue warps (fused: 16) from here to the last
   static constexpr int epi_warps = warps - epi0;
   // fused pair mode: the epilogue warps convert the samples (full-barrier arrivals per stage)
   static constexpr int fill_arrivals = MODE == kModePairFused ? epi_warps : 1;
@@ -97,7 +102,8 @@ struct Shape {
   static constexpr int block_bytes = (MODE == kModeNarrow ? 2 : 3) * kTileBytes;  // tiles of one block
   static constexpr int stage_bytes = kps * block_bytes;
   static constexpr int max_stages = MODE == kModeWide ? 4 : 2;
-  static constexpr int epi_bytes = pair ? epi_warps * kEpiStageBytes : 0;
+  static constexpr int epi_bytes = MODE == kModePair ? epi_warps * kEpiStageBytes : 0;  // (fused: in the stages)
+
 };
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAccCols = 256;  // re 128 | im 128
@@ -408,6 +414,39 @@ __device__ __forceinline__ void item_blocks(const PairItem &it, int KB, int &k0,
   k1 = (int)((uint32_t)((it.split + 1) * KB) / (uint32_t)it.n_split);
 }
 
+// Tiles that an item reads, in shared-memory order (channel tc[t], tile ti[t]).
+__device__ __forceinline__ int item_tiles(const PairItem &it, int (&tc)[3], int (&ti)[3]) {
+  tc[0] = tc[1] = tc[2] = it.c0;
+  ti[0] = it.I0;
+  ti[1] = it.J0;
+  ti[2] = 0;
+  if (it.type == kItemShared) {
+    ti[0] = it.J0;
+    ti[1] = it.J1;  // A_I itself when J1 == I0
+    ti[2] = it.I0;
+    return it.J1 == it.I0 ? 2 : 3;
+  }
+  if (it.type == kItemTwoDiag) {
+    tc[1] = it.c1;
+    ti[1] = it.I1;
+    return 2;
+  }
+  return it.I0 == it.J0 ? 1 : 2;
+}
+
+// Tiles of an item, and K blocks in a pair-mode stage (96 KB, every role takes
+// the same count): two blocks of three tiles, or three of two in the fused pair
+// mode and in jobs of two tiles.  With more tiles the pair mode keeps two for
+// both: items that share operand tiles through L2 would drift apart (384 inputs
+// 4.01 -> 4.36 ms, measured).
+__device__ __forceinline__ int item_tile_count(const PairItem &it) {
+  if (it.type == kItemShared) return it.J1 == it.I0 ? 2 : 3;
+  return it.type == kItemOne && it.I0 == it.J0 ? 1 : 2;
+}
+__device__ __forceinline__ int stage_blocks(int nt, bool fused, int n_tiles) {
+  return nt < 3 && (fused || n_tiles <= 2) ? 3 : 2;
+}
+
 // Pair-mode epilogue: each lane writes column j (lane & 15) of 16 of the 32
 // staged rows i0 + r (r = 2 r2 + lane / 16) of one half-block, lower triangle
 // only; ADD: add into the output with int32 atomics (one time range of several)
@@ -457,82 +496,95 @@ __device__ __forceinline__ void narrow_block(uint32_t d_re, uint32_t d_im, uint6
   block_mmas<BITS, kTile>(d_re, d_im, da, db, acc0);
 }
 
-// Fused pair mode: one converter thread's share of tile I of channel c, time
-// block kb (64 samples): the packed samples of kConvUnits (sample, 16-input)
-// units (unit u = sample u / 8, inputs 16 (u % 8) ..; thread ct takes units
-// ct + 256 m), loaded first (fused_load), then written as E4M3 codes
-// (fused_store), re plane at row t and im plane at row 64 + t of the tile,
-// each 16-byte chunk at its 128-byte swizzle position.  Samples past T and
-// inputs past N read as zero (N is a multiple of 16).
-__device__ __forceinline__ uint4 ld_stream16(const uint8_t *p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
+constexpr int kConvThreads = Shape<kModePairFused>::epi_warps * 32;
+static_assert(kConvThreads == 64 * 8, "one (sample, 16 inputs) unit per converter thread and tile block");
 
-#ifndef MWAX_FUSED_PREFETCH
-#define MWAX_FUSED_PREFETCH 3  // fused pair mode: stages of L2 prefetch ahead of the converters (0: none)
-#endif
-constexpr int kFusedPrefetch = MWAX_FUSED_PREFETCH;
-constexpr int kConvThreads = 256;                  // fused pair mode: the 8 epilogue warps
-constexpr int kConvUnits = 64 * 8 / kConvThreads;  // (sample, 16 inputs) units per thread per tile
+// Fused pair mode: one converter thread's loads of a work item: unit ct of a tile block is sample
+// ct / 8 of the block, inputs 16 (ct % 8) .. of the tile.  Tile block k of a
+// stage is tile k % nt of its block k / nt.  Samples past T and inputs past N
+// read as zero (N is a multiple of 16).
+constexpr int kStageTiles = 6;
+struct RawLoads {
+  const uint8_t *base;      // the unit of tile 0, block 0 of the next stage to load
+  int64_t off[kStageTiles];  // each tile block's unit, from there
+  int lim[kStageTiles];      // samples from that unit's row on in the first stage (0: no such inputs)
+  int done, rows;            // samples of the stages loaded so far, of one stage
+  int64_t step;              // bytes of a stage's sample rows
 
-struct FusedTile {
-  const uint8_t *row0;  // sample 0 of the block, input 128 I, channel c (never dereferenced as is)
-  int t_left;           // samples of the block that exist (T - 64 kb, may be <= 0)
-  int in_left;          // inputs of the tile that exist (N - 128 I)
+  __device__ __forceinline__ int start(const PairItem &it, const KJob &jb, int k0, int ct) {
+    int tc[3], ti[3];
+    const int nt = item_tiles(it, tc, ti), kps = stage_blocks(nt, true, 0);
+    const int N = jb.n_inputs, T = jb.n_time, row = k0 * 64 + (ct >> 3), x = (ct & 7) << 4;
+    base = jb.volt + ((int64_t)tc[0] * T + row) * N + ti[0] * kTile + x;
+    const int64_t d1 = (int64_t)(tc[1] - tc[0]) * T * N + (ti[1] - ti[0]) * kTile;
+    const int64_t d2 = (int64_t)(ti[2] - ti[0]) * kTile;
+    bool in[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) in[t] = t < nt && x < N - ti[t] * kTile;
+#pragma unroll
+    for (int k = 0; k < kStageTiles; ++k) {
+      const int j = nt == 3 ? k / 3 : nt == 2 ? k / 2 : k;
+      const int t = nt == 3 ? k % 3 : nt == 2 ? k % 2 : 0;
+      off[k] = (t == 0 ? 0 : t == 1 ? d1 : d2) + (int64_t)j * 64 * N;
+      lim[k] = j < kps && (t == 0 ? in[0] : t == 1 ? in[1] : in[2]) ? T - row - 64 * j : 0;
+    }
+    rows = 64 * kps;
+    step = (int64_t)rows * N;
+    done = 0;
+    return nt;
+  }
+  // the next stage's units (lim: the sample rows past T read as zero)
+  __device__ __forceinline__ void load(uint4 (&w)[kStageTiles]) {
+#pragma unroll
+    for (int k = 0; k < kStageTiles; ++k) {
+      w[k] = make_uint4(0, 0, 0, 0);
+      if (done < lim[k])
+        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w[k].x), "=r"(w[k].y), "=r"(w[k].z), "=r"(w[k].w)
+                     : "l"(base + off[k]));
+    }
+    base += step;
+    done += rows;
+  }
 };
 
-__device__ __forceinline__ void fused_load(const FusedTile &f, int N, int ct, uint4 (&w)[kConvUnits]) {
-#pragma unroll
-  for (int m = 0; m < kConvUnits; ++m) {
-    const int u = ct + kConvThreads * m;
-    const int t = u >> 3, x = (u & 7) << 4;
-    w[m] = t < f.t_left && x < f.in_left ? ld_stream16(f.row0 + (int64_t)t * N + x) : make_uint4(0, 0, 0, 0);
-  }
+// One 16-byte unit of packed samples to its place in a tile: sample row t
+// (plane re) and 64 + t (plane im), chunk ch at its swizzled position.
+__device__ __forceinline__ void fused_store(uint8_t *tile, int u, const uint4 &v) {
+  const int t = u >> 3, ch = u & 7;
+  const int off = t * kRowBytes + ((ch ^ (t & 7)) << 4);
+  *reinterpret_cast<uint4 *>(tile + off) = make_uint4(nib4_re(v.x), nib4_re(v.y), nib4_re(v.z), nib4_re(v.w));
+  *reinterpret_cast<uint4 *>(tile + 64 * kRowBytes + off) =
+      make_uint4(nib4_im(v.x), nib4_im(v.y), nib4_im(v.z), nib4_im(v.w));
 }
 
-__device__ __forceinline__ void fused_store(uint8_t *tile, int ct, const uint4 (&w)[kConvUnits]) {
-#pragma unroll
-  for (int m = 0; m < kConvUnits; ++m) {
-    const int u = ct + kConvThreads * m;
-    const int t = u >> 3, ch = u & 7;
-    const int off = t * kRowBytes + ((ch ^ (t & 7)) << 4);
-    const uint4 v = w[m];
-    *reinterpret_cast<uint4 *>(tile + off) =
-        make_uint4(nib4_re(v.x), nib4_re(v.y), nib4_re(v.z), nib4_re(v.w));
-    *reinterpret_cast<uint4 *>(tile + 64 * kRowBytes + off) =
-        make_uint4(nib4_im(v.x), nib4_im(v.y), nib4_im(v.z), nib4_im(v.w));
-  }
-}
-
-// Pair-mode epilogue of one work item (warp (q, h) of the eight epilogue
-// warps): wait for the accumulator (one thread; the result goes through a
-// two-entry flag so all eight warps take the same branch), convert, release
-// the accumulator, store the item's lower-triangle visibilities.  false: a
-// wait ran out (every warp stops).
+// The integer that an accumulator word holds (exact below 2^24 units).
 template <int BITS>
 __device__ __forceinline__ int acc_int(uint32_t v) {
   return __float2int_rn(__uint_as_float(v) * Op<BITS>::units);
 }
 
-template <int BITS, int KIND>
+// Pair-mode epilogue of one work item (warp (q, h) of the EW = 8 epilogue
+// warps, or (q, h, column half) of 16): wait for the accumulator (one thread; the result goes through a
+// two-entry flag so all the warps take the same branch), convert, release
+// the accumulator, store the item's lower-triangle visibilities.  false: a
+// wait ran out (every warp stops).
+template <int BITS, int KIND, int EW>
 __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it, uint32_t n_it,
                                            uint32_t tfull, uint32_t tempty, uint32_t tmem_base,
                                            uint8_t *stg, volatile int *abort_flag,
                                            volatile int *epi_flag, int warp, int lane, int epi0) {
   const unsigned long long tmo = p.timeout_ns;
   const int q = warp & 3;
-  const int h = (warp - epi0) >> 2;
+  const int part = (warp - epi0) >> 2;  // 0 .. EW / 4 - 1
+  const int h = part / (EW / 8);       // pair of the item
   const KJob &jb = p.job[it.job];
   if (warp == epi0 && lane == 0) {
     const bool got = mbar_wait(tfull, n_it & 1u, abort_flag, tmo);
     if (!got) raise_timeout(abort_flag, p.status);
     epi_flag[n_it & 1u] = got ? 1 : 0;
   }
-  named_bar_sync(1, 8 * 32);
+  named_bar_sync(1, EW * 32);
   if (!epi_flag[n_it & 1u]) return false;
   tc_fence_after();
   const bool has = h == 0 || it.type != kItemOne;
@@ -553,15 +605,17 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * kTile);
   uint32_t *out = reinterpret_cast<uint32_t *>(jb.out) + (int64_t)c * jb.n_bl * 2;
   const int n = jb.n_inputs;
+  constexpr int kChunks = 4 * 8 / EW;  // 32-column chunks of this warp
+  const int col0 = 32 * kChunks * (part % (EW / 8));
 #pragma unroll
-  for (int cc = 0; cc < 4; ++cc) {
+  for (int cc = 0; cc < kChunks; ++cc) {
     uint32_t vre[32], vim[32];
     if (has) {
-      tc_ld32(trow + 32 * cc, vre);
-      tc_ld32(trow + 2 * kTile + 32 * cc, vim);
+      tc_ld32(trow + col0 + 32 * cc, vre);
+      tc_ld32(trow + 2 * kTile + col0 + 32 * cc, vim);
       tc_wait_ld();
     }
-    if (cc == 3) {
+    if (cc == kChunks - 1) {
       // every column of this warp is in registers: release the accumulator
       // (test hook: withholding one release makes the MMA warp's bounded
       // wait run out -> MWAX_ERR_TIMEOUT, clean exit)
@@ -584,7 +638,7 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
         *reinterpret_cast<uint2 *>(stg + lane * 128 + ((k ^ (lane & 15)) << 3)) =
             make_uint2(vre[16 * half + k], vim[16 * half + k]);
       __syncwarp();
-      const int j = J * kTile + 32 * cc + 16 * half + (lane & 15);
+      const int j = J * kTile + col0 + 32 * cc + 16 * half + (lane & 15);
       const int i0 = I * kTile + q * 32;
       if (it.n_split > 1)  // one time range of several: exact integer adds
         store_rows<true>(stg, out, lane, i0, j, n);
@@ -598,26 +652,25 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
 
 // The same as a separate call (fused pair mode: the converters' state stays
 // out of the epilogue's register allocation).
-template <int BITS, int KIND>
+template <int BITS, int KIND, int EW>
 __device__ __noinline__ bool drain_item_call(const KParams &p, const PairItem &it, uint32_t n_it,
                                              uint32_t tfull, uint32_t tempty, uint32_t tmem_base,
                                              uint8_t *stg, volatile int *abort_flag,
                                              volatile int *epi_flag, int warp, int lane, int epi0) {
-  return drain_item<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag, warp,
-                          lane, epi0);
+  return drain_item<BITS, KIND, EW>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag,
+                                    warp, lane, epi0);
 }
 
 // The roles in pair mode.  Warp 0: TMA producer (idle in the fused pair
 // mode), warp 1: MMA issuer, warps 2..9: epilogue (in the fused pair mode
-// also the sample converters).  Barriers as in the kernel: full[0..S)
+// warps 2..17, also the sample converters).  Barriers as in the kernel: full[0..S)
 // empty[S..2S) tfull[3S] tempty[3S+2] drain[3S+4] (one accumulator buffer:
 // index 0 only).
 template <int BITS, int KIND, bool FUSED>
 __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, uint8_t *smem,
                                            uint32_t smem_base, uint8_t *epi_smem, uint32_t bar0,
                                            uint32_t tmem_base, volatile int *abort_flag,
-                                           volatile int *epi_flag, volatile int *conv_done,
-                                           int warp, int lane) {
+                                           volatile int *epi_flag, int warp, int lane) {
   using Sh = Shape<FUSED ? kModePairFused : kModePair>;
   constexpr int kStageBytes = Sh::stage_bytes;
   const int S = p.stages;
@@ -643,29 +696,16 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
         const KJob &jb = p.job[it.job];
         const CUtensorMap *map = &maps.m[it.job];
         const int n_rows = jb.n_tiles * kTile;
-        // each tile of the item at K block 0, in shared-memory order
-        TileAt<BITS> ts[3] = {TileAt<BITS>(0, 0, 0, 0), TileAt<BITS>(0, 0, 0, 0),
-                              TileAt<BITS>(0, 0, 0, 0)};
-        int nt;
-        if (it.type == kItemShared) {
-          ts[0] = TileAt<BITS>(it.c0, it.J0, jb.kb, n_rows);
-          ts[1] = TileAt<BITS>(it.c0, it.J1, jb.kb, n_rows);  // A_I itself when J1 == I0
-          ts[2] = TileAt<BITS>(it.c0, it.I0, jb.kb, n_rows);
-          nt = it.J1 == it.I0 ? 2 : 3;
-        } else if (it.type == kItemTwoDiag) {
-          ts[0] = TileAt<BITS>(it.c0, it.I0, jb.kb, n_rows);
-          ts[1] = TileAt<BITS>(it.c1, it.I1, jb.kb, n_rows);
-          nt = 2;
-        } else {
-          ts[0] = TileAt<BITS>(it.c0, it.I0, jb.kb, n_rows);
-          ts[1] = TileAt<BITS>(it.c0, it.J0, jb.kb, n_rows);
-          nt = it.I0 == it.J0 ? 1 : 2;
-        }
+        // each tile of the item at K block 0
+        int tc[3], ti[3];
+        const int nt = item_tiles(it, tc, ti), kps = stage_blocks(nt, FUSED, jb.n_tiles);
+        const TileAt<BITS> ts[3] = {TileAt<BITS>(tc[0], ti[0], jb.kb, n_rows), TileAt<BITS>(tc[1], ti[1], jb.kb, n_rows),
+                                    TileAt<BITS>(tc[2], ti[2], jb.kb, n_rows)};
         const uint32_t blk_bytes = (uint32_t)nt * kTileBytes;
         int k0, k1;
         item_blocks(it, jb.kb, k0, k1);
-        for (int kb = k0; kb < k1; kb += Sh::kps) {
-          const int nb = min(Sh::kps, k1 - kb);
+        for (int kb = k0; kb < k1; kb += kps) {
+          const int nb = min(kps, k1 - kb);
           if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag, tmo)) {
             raise_timeout(abort_flag, p.status);
             ok = false;
@@ -675,7 +715,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           mbar_arrive_expect_tx(full(stage), (uint32_t)nb * blk_bytes);
           for (int j = 0; j < nb; ++j)
             for (int t = 0; t < nt; ++t)
-              tma_load_2d(a + (uint32_t)(j * Sh::block_bytes + t * kTileBytes), map, ts[t].x,
+              tma_load_2d(a + (uint32_t)(j * nt + t) * kTileBytes, map, ts[t].x,
                           ts[t].y + (kb + j) * ts[t].step, full(stage));
           ++issued;
           if (++stage == S) {
@@ -693,47 +733,6 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           ph ^= 1u;
         }
         mbar_wait(full(st), ph, nullptr, tmo);
-      }
-    }
-    if (FUSED && kFusedPrefetch > 0 && lane == 0) {
-      // ------------ fused pair mode: L2 prefetch of the packed samples ------------
-      // The sample rows of each stage's channels, kFusedPrefetch stages ahead
-      // of the converters (paced by their count of filled stages, conv_done;
-      // a hint only: no result is read), so that their loads hit L2.
-      int64_t g = 0;  // stages of this CTA so far
-      bool ok = true;
-      for (int64_t item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-        const PairItem it = decode_pair_item(__ldg(p.items + item));
-        const KJob &jb = p.job[it.job];
-        const int N = jb.n_inputs, T = jb.n_time;
-        const int cb = it.type == kItemTwoDiag ? it.c1 : it.c0;
-        int k0, k1;
-        item_blocks(it, jb.kb, k0, k1);
-        for (int kb = k0; kb < k1; kb += Sh::kps, ++g) {
-          if (*conv_done < g - kFusedPrefetch) {
-            const uint64_t t0 = globaltimer();
-            while (*conv_done < g - kFusedPrefetch) {
-              if (*abort_flag || globaltimer() - t0 > tmo) {
-                ok = false;
-                break;
-              }
-              __nanosleep(128);
-            }
-            if (!ok) break;
-          }
-          const int r0 = kb * 64, r1 = min((kb + Sh::kps) * 64, T);
-          if (r1 <= r0) continue;
-          const uint32_t bytes = (uint32_t)(r1 - r0) * (uint32_t)N;
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                           jb.volt + ((int64_t)it.c0 * T + r0) * N),
-                       "r"(bytes)
-                       : "memory");
-          if (cb != it.c0)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                             jb.volt + ((int64_t)cb * T + r0) * N),
-                         "r"(bytes)
-                         : "memory");
-        }
       }
     }
     __syncwarp();
@@ -754,9 +753,10 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           break;
         }
         tc_fence_after();
-        const uint32_t a_off = it.J1 == it.I0 ? kTileBytes : 2 * kTileBytes;  // A_I of a shared item
-        for (int kb = k0; kb < k1; kb += Sh::kps) {
-          const int nb = min(Sh::kps, k1 - kb);
+        const int nt = item_tile_count(it), kps = stage_blocks(nt, FUSED, p.job[it.job].n_tiles);
+        const uint32_t a_off = (uint32_t)(nt - 1) * kTileBytes;  // A_I of a shared item
+        for (int kb = k0; kb < k1; kb += kps) {
+          const int nb = min(kps, k1 - kb);
           if (!mbar_wait(full(stage), phase, abort_flag, tmo)) {
             raise_timeout(abort_flag, p.status);
             ok = false;
@@ -764,7 +764,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           }
           tc_fence_after();
           for (int j = 0; j < nb; ++j) {
-            const uint32_t a = smem_base + (uint32_t)stage * kStageBytes + (uint32_t)(j * Sh::block_bytes);
+            const uint32_t a = smem_base + (uint32_t)stage * kStageBytes + (uint32_t)(j * nt) * kTileBytes;
             const uint32_t acc0 = kb + j == k0 ? 0u : 1u;
             if (it.type == kItemShared) {
               // B = [A_J0 ; A_J1]: columns 0..127 give pair (I, J0), 128..255 pair (I, J1)
@@ -796,20 +796,21 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
     __syncwarp();
   } else {
     // ---------------- epilogue: convert + integration dump ----------------
-    // Warp (q, h): tensor-memory lanes 32q.. (rows of the tile) of pair h.
+    // Warp (q, h): tensor-memory lanes 32q.. (rows of the tile) of pair h (fused
+    // pair mode: (q, h, column half)).
     // Each 32-column chunk goes through this warp's shared-memory buffer, 16
     // columns at a time: lane r writes row r (16 (re, im) words, XOR-swizzled
     // so the 16 lanes of a phase hit distinct banks), then each store
     // instruction writes rows r and r+1 as two contiguous 128-byte runs.
     // One thread waits for the accumulator; the result goes through a
-    // two-entry flag so all eight warps take the same branch (false: stop).
-    uint8_t *stg = epi_smem + (warp - Sh::epi0) * kEpiStageBytes;
+    // two-entry flag so all the warps take the same branch (false: stop).
+    uint8_t *stg = (FUSED ? smem : epi_smem) + (warp - Sh::epi0) * kEpiStageBytes;
     auto drain = [&](const PairItem &it, uint32_t n_it) -> bool {
       if constexpr (FUSED)
-        return drain_item_call<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag,
+        return drain_item_call<BITS, KIND, Sh::epi_warps>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag,
                                      epi_flag, warp, lane, Sh::epi0);
       else
-        return drain_item<BITS, KIND>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag,
+        return drain_item<BITS, KIND, Sh::epi_warps>(p, it, n_it, tfull, tempty, tmem_base, stg, abort_flag, epi_flag,
                                 warp, lane, Sh::epi0);
     };
     uint32_t n_it = 0;
@@ -820,79 +821,45 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
       }
     } else {
       // Fused pair mode: first every stage of the item (the same items and
-      // blocks as the MMA issuer; each stage written by all eight warps and
-      // released with one arrival per warp after a proxy fence, since the
-      // tensor core reads generic-proxy stores), then the item's drain.  A
-      // warp whose wait for a free stage runs out skips the rest of the item
-      // and still joins the drain, where the shared flag ends every warp.
+      // blocks as the MMA issuer; each stage written by all the warps and
+      // released with one arrival per warp after a proxy fence, since the tensor
+      // core reads generic-proxy stores), then the item's drain.  A stage's
+      // samples are loaded into registers as soon as the stage before it is
+      // released, so they arrive while the warps wait for a free stage.  A warp
+      // whose wait for a free stage runs out skips the rest of the item and still
+      // joins the drain, where the shared flag ends every warp.
       const int ct = (int)threadIdx.x - 32 * Sh::epi0;
       int stage = 0;
       uint32_t phase = 0;
-      int64_t filled = 0;  // stages of this CTA filled so far
       for (int64_t item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         const PairItem it = decode_pair_item(__ldg(p.items + item));
-        const KJob &jb = p.job[it.job];
-        const int N = jb.n_inputs, T = jb.n_time;
-        // the item's tiles in shared-memory order (as the producer loads them)
-        int tc[3] = {it.c0, it.c0, it.c0}, ti[3] = {0, 0, 0};
-        int nt;
-        if (it.type == kItemShared) {
-          ti[0] = it.J0;
-          ti[1] = it.J1;
-          ti[2] = it.I0;
-          nt = it.J1 == it.I0 ? 2 : 3;
-        } else if (it.type == kItemTwoDiag) {
-          ti[0] = it.I0;
-          tc[1] = it.c1;
-          ti[1] = it.I1;
-          nt = 2;
-        } else {
-          ti[0] = it.I0;
-          ti[1] = it.J0;
-          nt = it.I0 == it.J0 ? 1 : 2;
-        }
         int k0, k1;
-        item_blocks(it, jb.kb, k0, k1);
-        for (int kb = k0; kb < k1; kb += Sh::kps) {
-          const int nb = min(Sh::kps, k1 - kb);
+        item_blocks(it, p.job[it.job].kb, k0, k1);
+        RawLoads ld;
+        const int nt = ld.start(it, p.job[it.job], k0, ct), kps = stage_blocks(nt, true, 0);
+        uint4 w[kStageTiles];
+        ld.load(w);
+        for (int kb = k0; kb < k1; kb += kps) {
           if (!warp_wait(empty(stage), phase ^ 1u, abort_flag, tmo, lane)) {
             if (lane == 0) raise_timeout(abort_flag, p.status);
             break;
           }
           uint8_t *st_base = smem + (size_t)stage * kStageBytes;
-          // every load of the stage first (one memory latency per stage), then
-          // the conversions and shared-memory stores
-          uint4 w[Sh::kps][3][kConvUnits];
+          const int n = nt * min(kps, k1 - kb);  // tile blocks of the stage
 #pragma unroll
-          for (int j = 0; j < Sh::kps; ++j) {
-            const int s0 = (kb + j) * 64;
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-              if (j < nb && t < nt) {
-                FusedTile f;
-                f.row0 = jb.volt + ((int64_t)tc[t] * T + s0) * N + ti[t] * kTile;
-                f.t_left = T - s0;
-                f.in_left = N - ti[t] * kTile;
-                fused_load(f, N, ct, w[j][t]);
-              }
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < Sh::kps; ++j)
-#pragma unroll
-            for (int t = 0; t < 3; ++t)
-              if (j < nb && t < nt) fused_store(st_base + j * Sh::block_bytes + t * kTileBytes, ct, w[j][t]);
+          for (int k = 0; k < kStageTiles; ++k)
+            if (k < n) fused_store(st_base + k * kTileBytes, ct, w[k]);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(full(stage));
-          ++filled;
-          if (warp == Sh::epi0 && lane == 0) *conv_done = (int)filled;  // paces the L2 prefetch
+          if (kb + kps < k1) ld.load(w);
           if (++stage == S) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!drain(it, n_it)) break;
+        named_bar_sync(1, Sh::epi_warps * 32);  // the stages, the drain's staging, are written again
         ++n_it;
       }
     }
@@ -916,7 +883,7 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
   // full[0..S) empty[S..2S) bfull[2S..3S) tfull[3S..3S+2) tempty[3S+2..3S+4) drain[3S+4]
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 3 * S + 5);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  // [0..1]: result of the epilogue's accumulator wait; [2]: fused pair mode's filled-stage count
+  // [0..1]: result of the epilogue's accumulator wait
   volatile int *epi_flag = abort_flag + 1;
   auto full = [&](int s) { return smem_u32(bars + s); };
   auto empty = [&](int s) { return smem_u32(bars + S + s); };
@@ -941,7 +908,6 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
-    epi_flag[2] = 0;  // fused pair mode: stages the converters have filled
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -959,7 +925,7 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
 
   if constexpr (PAIR) {
     pair_roles<BITS, KIND, FUSED>(maps, p, smem, smem_base, epi_smem, smem_u32(bars), tmem_base,
-                                  abort_flag, epi_flag, epi_flag + 2, warp, lane);
+                                  abort_flag, epi_flag, warp, lane);
   } else if (warp == 0) {
     // ---------------- TMA producer (one thread) ----------------
     if (lane == 0) {

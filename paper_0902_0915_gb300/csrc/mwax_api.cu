@@ -261,24 +261,39 @@ int resolve_split(const mwax_job &job, int mode, int kb, int64_t base_items, int
   return std::max(k, 1);
 }
 
-// Fused pair mode chosen automatically up to this many 128-input tiles: each
-// operand tile is converted once per work item that reads it (about n_tiles /
-// 2 + 1 times per channel and time block), against one write and one read of
-// the unpacked operands through HBM without the fusion.
-constexpr int kFusedAutoTiles = 2;
+// Where the fused pair mode is the automatic choice.  Every operand tile is
+// converted once per work item that reads it (about n_tiles / 2 + 1 times per
+// channel and time block), against one write and one read of the unpacked
+// operands through HBM or, while they fit it, L2 without the fusion; and its
+// conversion stops during an item's drain.  So: always up to two tiles; with
+// more, when the launch's operands take over half of the L2 (64 MB) and an item
+// has enough blocks per tile to hide the drain.  Measured, fused against unpack
+// + pair, in microseconds: 256 inputs x 768 channels x 20,000 samples 1791 /
+// 3413, 384 x 512 x 20,000 2652 / 4004, 512 x 128 x 2000 179 / 201, 768 x 256 x
+// 20,000 4490 / 5228, 1024 x 192 x 20,000 5658 / 6127, 1024 x 64 x 3000 374 /
+// 379; and on the other side 512 x 32 x 1000 50 / 47, 768 x 32 x 1000 76 / 73,
+// 1024 x 64 x 1000 209 / 181.
+constexpr int kFusedTiles = 2, kFusedBlocksPerTile = 4;
+constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
 
-// Kernel mode for a job's mma_shape (0 = auto: the fused pair mode for small
-// 4-bit exact arrays that allow it (fused_ok, at most kFusedAutoTiles tiles),
-// else the pair mode where every job integrates in one exact segment, else
-// narrow); -1 when an explicit pair or fused pair request cannot be served.
+bool fused_pays(const TcJob &j) {
+  if (j.n_tiles <= kFusedTiles) return true;
+  const int64_t operands = (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes;
+  return operands > kFusedOperandBytes && j.kb >= kFusedBlocksPerTile * j.n_tiles;
+}
+
+// Kernel mode for a job's mma_shape (0 = auto: the fused pair mode for 4-bit
+// exact arrays that allow it (fused_ok) where it pays for every job, else the
+// pair mode where every job integrates in one exact segment, else narrow); -1
+// when an explicit pair or fused pair request cannot be served.
 int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok) {
   const bool pair_ok = pair_mode_supported(tj.data(), (int)tj.size());
   if (mma_shape == 4) return pair_ok && fused_ok ? 3 : -1;
   if (mma_shape == 3) return pair_ok ? 2 : -1;
   if (mma_shape == 1 || mma_shape == 2) return mma_shape - 1;
-  bool small = true;
-  for (const TcJob &j : tj) small = small && j.n_tiles <= kFusedAutoTiles;
-  if (pair_ok && fused_ok && small) return 3;
+  bool pays = true;
+  for (const TcJob &j : tj) pays = pays && fused_pays(j);
+  if (pair_ok && fused_ok && pays) return 3;
   return pair_ok ? 2 : 0;
 }
 
