@@ -40,7 +40,8 @@ namespace {
 
 constexpr int kCT = 32;        // inputs per calibration tile side
 constexpr int kCalThreads = 256;
-constexpr int kMaxChanGroups = 12;  // 528 tiles x 12 = 13.9 waves of 3 CTAs per SM at 1024 inputs
+constexpr int kCalibCtas = 3;  // of the loss/adjoint pass, per SM
+constexpr int kMaxChanGroups = 12;
 
 struct Kahan {
   float s = 0.f, c = 0.f;
@@ -52,7 +53,29 @@ struct Kahan {
   }
 };
 
-int chan_groups(int n_chan) { return n_chan < kMaxChanGroups ? n_chan : kMaxChanGroups; }
+// Most channel groups of a shape (the workspaces are sized for them).
+int max_chan_groups(int n_chan) { return n_chan < kMaxChanGroups ? n_chan : kMaxChanGroups; }
+
+// Channel groups of a launch of `tiles` x groups CTAs whose eight warps share a
+// group's channels, `ctas` of them resident per SM: the count that leaves the
+// fewest channels to the busiest warp of the last round, rounds of CTAs times
+// channels per warp (of equal counts the largest that gives every warp a
+// channel).  At 1024 inputs that is 12 groups for 768 channels, as measured
+// best; 256 channels take 11 for the Jones pass (5 rounds of 3 channels, against
+// 6 of 3 with 12).
+int chan_groups(int tiles, int n_chan, int ctas) {
+  const int64_t slots = 152 * (int64_t)ctas;
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int n = 1; n <= max_chan_groups(n_chan) && n <= (n_chan + 7) / 8; ++n) {
+    const int64_t cost = (((int64_t)tiles * n + slots - 1) / slots) * ((n_chan + 8 * n - 1) / (8 * n));
+    if (cost <= best_cost) {
+      best = n;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
 
 __device__ __forceinline__ void tile_of(int p, int &I, int &J) {
   int i = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
@@ -166,7 +189,7 @@ __device__ __forceinline__ int tile_row_of_lane(int lane) {
 // sums of |g_other|^2 |M|^2 (the gain solve's normal-equation weight; sums of
 // positive terms, plain FP32).
 template <bool DEN>
-__global__ void __launch_bounds__(kCalThreads, 3) calib_tile_kernel(
+__global__ void __launch_bounds__(kCalThreads, kCalibCtas) calib_tile_kernel(
     const float2 *__restrict__ V, const float2 *__restrict__ M, const float2 *__restrict__ g,
     int N, int C, int n_cg, float *__restrict__ part_loss, float2 *__restrict__ part_row,
     float2 *__restrict__ part_col, float *__restrict__ part_rden, float *__restrict__ part_cden) {
@@ -244,80 +267,131 @@ __global__ void __launch_bounds__(kCalThreads, 3) calib_tile_kernel(
   }
 }
 
+// Full-warp sum, every lane holding it (pairwise, fixed order).
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Full-warp sum of s + e, the rounding errors of the additions kept in e.
+__device__ __forceinline__ void warp_sum2(float &s, float &e) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float x = __shfl_xor_sync(0xffffffffu, s, o);
+    e += __shfl_xor_sync(0xffffffffu, e, o);
+    const float t = s + x, z = t - s;
+    e += (s - (t - z)) + (x - z);
+    s = t;
+  }
+}
+
+// Sum of n loss partials by a whole block, compensated, into *loss; red: two
+// floats per warp.
+__device__ __forceinline__ void sum_losses(const float *__restrict__ part, int64_t n, float *red,
+                                           float *__restrict__ loss) {
+  Kahan acc;
+  for (int64_t k = threadIdx.x; k < n; k += 4 * (int64_t)blockDim.x) {
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = k + u * (int64_t)blockDim.x;
+      v[u] = i < n ? part[i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc.add(v[u]);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float s = acc.s, e = -acc.c;
+  warp_sum2(s, e);
+  if (lane == 0) {
+    red[2 * warp] = s;
+    red[2 * warp + 1] = e;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const bool has = lane < (int)(blockDim.x >> 5);
+    s = has ? red[2 * lane] : 0.f;
+    e = has ? red[2 * lane + 1] : 0.f;
+    warp_sum2(s, e);
+    if (lane == 0) *loss = s + e;
+  }
+}
+
 // grid: n_blocks + 1.  Block K < n_blocks gathers grad for inputs K*32..;
 // the last block sums the loss partials.  SOLVE: instead of grad, apply one
 // gain-solve sweep to g in place (each block reads and writes only its own
 // 32 gains): g = h (avg == 0) or g = (g + h) / 2 (avg == 1).
+// A chain of dependent loads bounds it: 32 threads per input take every 32nd
+// contribution, four in flight each (8 threads with one in flight took 23 us
+// at 1024 inputs).
+constexpr int kGatherThreads = 1024;
 template <bool SOLVE>
-__global__ void __launch_bounds__(kCalThreads) calib_gather_kernel(
+__global__ void __launch_bounds__(kGatherThreads) calib_gather_kernel(
     int N, int n_blocks, int n_cg, const float *__restrict__ part_loss,
     const float2 *__restrict__ part_row, const float2 *__restrict__ part_col,
     const float *__restrict__ part_rden, const float *__restrict__ part_cden,
     float *__restrict__ loss, float2 *__restrict__ grad, float2 *__restrict__ g_io, int avg) {
+  constexpr int kL = kGatherThreads / kCT;
   const int K = blockIdx.x;
+  __shared__ float2 sacc[kL][kCT + 1];
+  __shared__ float sden[kL][kCT + 1];
   if (K == n_blocks) {
-    if (!loss) return;
-    __shared__ float sred[kCalThreads];
-    const int n_part = n_blocks * (n_blocks + 1) / 2 * n_cg;
-    Kahan acc;
-    for (int k = threadIdx.x; k < n_part; k += kCalThreads) acc.add(part_loss[k]);
-    sred[threadIdx.x] = acc.s;
-    __syncthreads();
-    for (int w = kCalThreads / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) sred[threadIdx.x] += sred[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = sred[0];
+    if (loss) sum_losses(part_loss, (int64_t)n_blocks * (n_blocks + 1) / 2 * n_cg, &sden[0][0], loss);
     return;
   }
   if (!SOLVE && !grad) return;
-  // 32 inputs x 8 partial lanes: thread (r, l) sums every 8th contribution
-  __shared__ float2 sacc[8][kCT];
-  __shared__ float sden[8][kCT];
   const int r = threadIdx.x & 31, l = threadIdx.x >> 5;
   Kahan ar, ai, ad;
   // contributions n = 0, 1, ...: the row partials of tiles (K, J <= K), then
   // the column partials of tiles (I >= K, K), each over the channel groups;
-  // thread l takes n = l, l + 8, ...
+  // thread l takes n = l, l + 32, ...
   const int n_row = (K + 1) * n_cg;
   const int n_tot = n_row + (n_blocks - K) * n_cg;
-  for (int n = l; n < n_tot; n += 8) {
-    const bool is_row = n < n_row;
-    const int m = is_row ? n : n - n_row;
-    const int t = m / n_cg, cg = m - t * n_cg;
-    const int tile = is_row ? K * (K + 1) / 2 + t : (K + t) * (K + t + 1) / 2 + K;
-    const int64_t idx = ((int64_t)tile * n_cg + cg) * kCT + r;
-    const float2 v = is_row ? part_row[idx] : part_col[idx];
-    ar.add(v.x);
-    ai.add(v.y);
-    if constexpr (SOLVE) ad.add(is_row ? part_rden[idx] : part_cden[idx]);
+  for (int n0 = l; n0 < n_tot; n0 += 4 * kL) {
+    float2 v[4];
+    float d[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int n = n0 + u * kL;
+      v[u] = make_float2(0.f, 0.f);
+      d[u] = 0.f;
+      if (n < n_tot) {
+        const bool is_row = n < n_row;
+        const int m = is_row ? n : n - n_row;
+        const int t = m / n_cg, cg = m - t * n_cg;
+        const int tile = is_row ? K * (K + 1) / 2 + t : (K + t) * (K + t + 1) / 2 + K;
+        const int64_t idx = ((int64_t)tile * n_cg + cg) * kCT + r;
+        v[u] = is_row ? part_row[idx] : part_col[idx];
+        if constexpr (SOLVE) d[u] = is_row ? part_rden[idx] : part_cden[idx];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      ar.add(v[u].x);
+      ai.add(v[u].y);
+      if constexpr (SOLVE) ad.add(d[u]);
+    }
   }
   sacc[l][r] = make_float2(ar.s, ai.s);
   if constexpr (SOLVE) sden[l][r] = ad.s;
   __syncthreads();
-  if (l == 0) {
-    float2 acc = sacc[0][r];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) {
-      acc.x += sacc[w][r].x;
-      acc.y += sacc[w][r].y;
+  // warp w sums the 32 partials of input w
+  const float2 p = sacc[r][l];
+  const float2 acc = make_float2(warp_sum(p.x), warp_sum(p.y));
+  const int k = K * kCT + l;
+  if constexpr (SOLVE) {
+    const float den = warp_sum(sden[r][l]);
+    if (r == 0 && k < N && den > 0.f) {
+      // h = g - (grad / 2) / den; acc holds grad / 2
+      const float2 gk = g_io[k];
+      const float inv = 1.f / den;
+      float2 h = make_float2(gk.x - acc.x * inv, gk.y - acc.y * inv);
+      if (avg) h = make_float2(0.5f * (gk.x + h.x), 0.5f * (gk.y + h.y));
+      g_io[k] = h;
     }
-    const int k = K * kCT + r;
-    if constexpr (SOLVE) {
-      float den = sden[0][r];
-#pragma unroll
-      for (int w = 1; w < 8; ++w) den += sden[w][r];
-      if (k < N && den > 0.f) {
-        // h = g - (grad / 2) / den; acc holds grad / 2
-        const float2 gk = g_io[k];
-        const float inv = 1.f / den;
-        float2 h = make_float2(gk.x - acc.x * inv, gk.y - acc.y * inv);
-        if (avg) h = make_float2(0.5f * (gk.x + h.x), 0.5f * (gk.y + h.y));
-        g_io[k] = h;
-      }
-    } else {
-      if (k < N) grad[k] = make_float2(2.f * acc.x, 2.f * acc.y);
-    }
+  } else if (r == 0 && k < N) {
+    grad[k] = make_float2(2.f * acc.x, 2.f * acc.y);
   }
 }
 
@@ -388,17 +462,8 @@ __global__ void __launch_bounds__(kCalThreads) calib_chan_gather_kernel(
   const int K = blockIdx.x;
   if (K == n_blocks) {
     if (blockIdx.y != 0 || !loss) return;
-    __shared__ float sred[kCalThreads];
-    const int64_t n_part = (int64_t)n_blocks * (n_blocks + 1) / 2 * gridDim.y;
-    Kahan acc;
-    for (int64_t k = threadIdx.x; k < n_part; k += kCalThreads) acc.add(part_loss[k]);
-    sred[threadIdx.x] = acc.s;
-    __syncthreads();
-    for (int h = kCalThreads / 2; h > 0; h >>= 1) {
-      if (threadIdx.x < h) sred[threadIdx.x] += sred[threadIdx.x + h];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = sred[0];
+    __shared__ float sred[2 * kCalThreads / 32];
+    sum_losses(part_loss, (int64_t)n_blocks * (n_blocks + 1) / 2 * gridDim.y, sred, loss);
     return;
   }
   if (!SOLVE && !grad) return;
@@ -452,10 +517,7 @@ __global__ void __launch_bounds__(kCalThreads) calib_chan_gather_kernel(
 // b >= a) load V = M = 0 and contribute exactly 0.
 constexpr int kJT = 32;  // Jones blocks per calibration tile side
 constexpr int kJQ = 12;  // per-tile partial quantities
-#ifndef MWAX_JONES_CHAN_GROUPS
-#define MWAX_JONES_CHAN_GROUPS 12  // channel groups of the Jones pass (CTAs per calibration tile)
-#endif
-constexpr int kJonesChanGroups = MWAX_JONES_CHAN_GROUPS;
+constexpr int kJonesCtas = 2;  // of the pass, per SM
 
 // acc + a b,  acc + a conj(b),  acc + conj(a) b
 __device__ __forceinline__ float2 cfma(float2 acc, float2 a, float2 b) {
@@ -618,7 +680,7 @@ constexpr int jones2_smem_bytes() {
   return (kCalThreads / 32) * kJPairs * 2 * 4 * 32 * 16 + kJT * 4 * 8;
 }
 template <bool DEN>
-__global__ void __launch_bounds__(kCalThreads, 2) calib_jones_tile2_kernel(
+__global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_kernel(
     const float2 *__restrict__ V, const float2 *__restrict__ M, const float2 *__restrict__ Jm,
     int n_tiles, int C, int n_cg, float *__restrict__ part_loss, float *__restrict__ part_row,
     float *__restrict__ part_col) {
@@ -755,51 +817,64 @@ __global__ void __launch_bounds__(kCalThreads, 2) calib_jones_tile2_kernel(
   }
 }
 
-// grid: n_jt + 1 blocks of kJT * kJQ threads.  Block K < n_jt: thread (t, q)
-// sums quantity q of tile K*32 + t over the row partials of calibration tiles
-// (K, J <= K) and the column partials of tiles (I >= K, K), every channel
-// group, in that order; then thread t < 32 writes grad = 2 G or (SOLVE) the
-// update J <- J - G D^-1 (averaged with J when avg), J kept where
-// det D <= 0.  The last block sums the loss partials.
+// grid: (n_jt + 1, kJT / 2).  Block (K < n_jt, y) sums the twelve quantities of
+// Jones tiles K*32 + 2y and the next (lane = 12 t + q of 24): warp w takes every
+// 16th contribution, four in flight -- the row partials of calibration tiles
+// (K, J <= K), then the column partials of tiles (I >= K, K), every channel
+// group -- and the sixteen sums are added in warp order; then lane t < 2 writes
+// grad = 2 G or (SOLVE) the update J <- J - G D^-1 (averaged with J when avg), J
+// kept where det D <= 0.  Block (n_jt, 0) sums the loss partials.  (One thread
+// per quantity for all the contributions took 24 us at 1024 inputs.)
+constexpr int kJGatherWarps = 16;
 template <bool SOLVE>
-__global__ void __launch_bounds__(kJT * kJQ) calib_jones_gather_kernel(
+__global__ void __launch_bounds__(kJGatherWarps * 32) calib_jones_gather_kernel(
     int n_tiles, int n_jt, int n_cg, const float *__restrict__ part_loss,
     const float *__restrict__ part_row, const float *__restrict__ part_col,
     float *__restrict__ loss, float2 *__restrict__ grad, float2 *__restrict__ J_io, int avg) {
   const int K = blockIdx.x;
-  __shared__ float sacc[kJT * kJQ];
+  __shared__ float spart[kJGatherWarps][2 * kJQ];
+  __shared__ float sacc[2 * kJQ];
   if (K == n_jt) {
-    if (!loss) return;
-    const int n_part = n_jt * (n_jt + 1) / 2 * n_cg;
-    Kahan acc;
-    for (int k = threadIdx.x; k < n_part; k += blockDim.x) acc.add(part_loss[k]);
-    sacc[threadIdx.x] = acc.s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = 0.f;
-      for (int k = 0; k < (int)blockDim.x; ++k) t += sacc[k];
-      *loss = t;
-    }
+    if (loss && blockIdx.y == 0) sum_losses(part_loss, (int64_t)n_jt * (n_jt + 1) / 2 * n_cg, &spart[0][0], loss);
     return;
   }
   if (!SOLVE && !grad) return;
-  const int e = threadIdx.x;  // = t * kJQ + q
-  Kahan acc;
-  for (int Jt = 0; Jt <= K; ++Jt) {
-    const int tile = K * (K + 1) / 2 + Jt;
-    for (int cg = 0; cg < n_cg; ++cg)
-      acc.add(part_row[((int64_t)tile * n_cg + cg) * kJT * kJQ + e]);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane < 2 * kJQ) {
+    Kahan acc;
+    const int e = blockIdx.y * 2 * kJQ + lane;
+    const int n_row = (K + 1) * n_cg, n_tot = n_row + (n_jt - K) * n_cg;
+    for (int n0 = w; n0 < n_tot; n0 += 4 * kJGatherWarps) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int n = n0 + u * kJGatherWarps;
+        v[u] = 0.f;
+        if (n < n_tot) {
+          const bool is_row = n < n_row;
+          const int m = is_row ? n : n - n_row;
+          const int t = m / n_cg, cg = m - t * n_cg;
+          const int tile = is_row ? K * (K + 1) / 2 + t : (K + t) * (K + t + 1) / 2 + K;
+          v[u] = (is_row ? part_row : part_col)[((int64_t)tile * n_cg + cg) * kJT * kJQ + e];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc.add(v[u]);
+    }
+    spart[w][lane] = acc.s;
   }
-  for (int It = K; It < n_jt; ++It) {
-    const int tile = It * (It + 1) / 2 + K;
-    for (int cg = 0; cg < n_cg; ++cg)
-      acc.add(part_col[((int64_t)tile * n_cg + cg) * kJT * kJQ + e]);
-  }
-  sacc[e] = acc.s;
   __syncthreads();
-  const int t = threadIdx.x;
-  const int a = K * kJT + t;
-  if (t >= kJT || a >= n_tiles) return;
+  if (w != 0) return;
+  if (lane < 2 * kJQ) {
+    Kahan acc;
+#pragma unroll
+    for (int k = 0; k < kJGatherWarps; ++k) acc.add(spart[k][lane]);
+    sacc[lane] = acc.s;
+  }
+  __syncwarp();
+  const int t = lane;
+  const int a = K * kJT + 2 * blockIdx.y + t;
+  if (t >= 2 || a >= n_tiles) return;
   const float *q = sacc + t * kJQ;
   const float2 G00 = make_float2(q[0], q[1]), G01 = make_float2(q[2], q[3]);
   const float2 G10 = make_float2(q[4], q[5]), G11 = make_float2(q[6], q[7]);
@@ -907,16 +982,13 @@ ChanWs chan_carve(void *ws, int nb, int n_chan, int n_cy, bool solve) {
   return w;
 }
 
-int jones_chan_groups(int n_chan) {
-  return n_chan < kJonesChanGroups ? n_chan : kJonesChanGroups;
-}
 
 // Layout: row partials, column partials ([tile][cg][32][12] floats each), loss
 // partials [tile][cg].
 int64_t jones_ws_bytes(int n_inputs, int n_chan) {
   if (n_inputs < 2 || (n_inputs & 1) || n_inputs > 65536 || n_chan < 1) return -1;
   const int64_t n_jt = (n_inputs / 2 + kJT - 1) / kJT;
-  const int64_t slots = n_jt * (n_jt + 1) / 2 * jones_chan_groups(n_chan);
+  const int64_t slots = n_jt * (n_jt + 1) / 2 * max_chan_groups(n_chan);
   return slots * kJT * kJQ * (int64_t)sizeof(float) * 2 + slots * (int64_t)sizeof(float);
 }
 
@@ -931,7 +1003,7 @@ int64_t mwax_calib_workspace_bytes(int n_inputs, int n_chan) {
   if (n_inputs < 2 || n_chan < 1) return -1;
   const int64_t nb = (n_inputs + kCT - 1) / kCT;
   const int64_t tiles = nb * (nb + 1) / 2;
-  const int64_t cg = chan_groups(n_chan);
+  const int64_t cg = max_chan_groups(n_chan);
   return tiles * cg * kCT * (int64_t)sizeof(float2) * 2 + tiles * cg * (int64_t)sizeof(float) + 256;
 }
 
@@ -945,7 +1017,7 @@ mwax_status mwax_calib_loss_grad(const float *V, const float *M, const float *g,
   if ((loss && !dev_ptr(loss)) || (grad && !dev_ptr(grad))) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(n_chan);
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas);
   Ws w = carve(workspace, nb, n_cg, false);
   calib_tile_kernel<false><<<dim3(tiles, n_cg), kCalThreads, 0, stream>>>(
       reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M),
@@ -953,7 +1025,7 @@ mwax_status mwax_calib_loss_grad(const float *V, const float *M, const float *g,
       nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return MWAX_ERR_CUDA;
-  calib_gather_kernel<false><<<nb + 1, kCalThreads, 0, stream>>>(
+  calib_gather_kernel<false><<<nb + 1, kGatherThreads, 0, stream>>>(
       n_inputs, nb, n_cg, w.loss, w.row, w.col, nullptr, nullptr, loss,
       reinterpret_cast<float2 *>(grad), nullptr, 0);
   return cudaGetLastError() == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
@@ -963,7 +1035,7 @@ int64_t mwax_calib_solve_workspace_bytes(int n_inputs, int n_chan) {
   if (n_inputs < 2 || n_chan < 1) return -1;
   const int64_t nb = (n_inputs + kCT - 1) / kCT;
   const int64_t tiles = nb * (nb + 1) / 2;
-  const int64_t cg = chan_groups(n_chan);
+  const int64_t cg = max_chan_groups(n_chan);
   return tiles * cg * kCT * (int64_t)sizeof(float2) * 2 +
          (tiles * cg * (int64_t)sizeof(float) + 255) / 256 * 256 +
          tiles * cg * kCT * (int64_t)sizeof(float) * 2 + 256;
@@ -977,7 +1049,7 @@ mwax_status mwax_calib_solve(const float *V, const float *M, float *g, int n_inp
   if (loss_hist && !dev_ptr(loss_hist)) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(n_chan);
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas);
   Ws w = carve(workspace, nb, n_cg, true);
   float2 *g2 = reinterpret_cast<float2 *>(g);
   for (int t = 1; t <= n_iter; ++t) {
@@ -985,7 +1057,7 @@ mwax_status mwax_calib_solve(const float *V, const float *M, float *g, int n_inp
         reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M), g2, n_inputs,
         n_chan, n_cg, w.loss, w.row, w.col, w.rden, w.cden);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
-    calib_gather_kernel<true><<<nb + 1, kCalThreads, 0, stream>>>(
+    calib_gather_kernel<true><<<nb + 1, kGatherThreads, 0, stream>>>(
         n_inputs, nb, n_cg, w.loss, w.row, w.col, w.rden, w.cden,
         loss_hist ? loss_hist + (t - 1) : nullptr, nullptr, g2, (t % 2 == 0) ? 1 : 0);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
@@ -1060,7 +1132,7 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
   const int n_tiles = n_inputs / 2;
   const int n_jt = (n_tiles + kJT - 1) / kJT;
   const int tiles = n_jt * (n_jt + 1) / 2;
-  const int n_cg = jones_chan_groups(n_chan);
+  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas);
   const int64_t slots = (int64_t)tiles * n_cg;
   float *prow = reinterpret_cast<float *>(workspace);
   float *pcol = prow + slots * kJT * kJQ;
@@ -1085,14 +1157,14 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
   if (!solve) {
     tile_pass(false);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
-    calib_jones_gather_kernel<false><<<n_jt + 1, kJT * kJQ, 0, stream>>>(
+    calib_jones_gather_kernel<false><<<dim3(n_jt + 1, kJT / 2), kJGatherWarps * 32, 0, stream>>>(
         n_tiles, n_jt, n_cg, ploss, prow, pcol, loss, reinterpret_cast<float2 *>(grad), nullptr, 0);
     return cudaGetLastError() == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
   }
   for (int t = 1; t <= n_iter; ++t) {
     tile_pass(true);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
-    calib_jones_gather_kernel<true><<<n_jt + 1, kJT * kJQ, 0, stream>>>(
+    calib_jones_gather_kernel<true><<<dim3(n_jt + 1, kJT / 2), kJGatherWarps * 32, 0, stream>>>(
         n_tiles, n_jt, n_cg, ploss, prow, pcol, loss ? loss + (t - 1) : nullptr, nullptr, J2,
         (t % 2 == 0) ? 1 : 0);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
