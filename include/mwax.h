@@ -106,10 +106,13 @@ typedef struct {
                               shared memory, so no operand buffer and no unpack pass
                               (4-bit exact samples in one exact segment with n_inputs a
                               multiple of 16 -- every job of a batch plan --, else
-                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 where it applies and, for
-                              every job, n_inputs <= 256 or the launch's operand tiles
-                              exceed 64 MB and the integration has at least 256 samples
-                              per 128-input tile, else 3 where it applies, else 1         */
+                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 where it applies and
+                              n_inputs <= 256, or the operand tiles would exceed 64 MB and
+                              the integration has at least 256 samples per 128-input tile
+                              (other n_inputs too, from 16 MB of operand tiles on: their
+                              rows are copied to padded ones first; batch plans: where
+                              this holds for most of the operand bytes), else 3 where it
+                              applies, else 1                                             */
   int32_t pipeline;        /* tuning: 1 = unpack then correlate each channel group on the
                               plan's stream, 2 = unpack the next group (second stream,
                               second scratch buffer) while the current group correlates,
@@ -186,7 +189,8 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
 
 /* Plan several jobs (uneven N, C, T) that are correlated together by one
  * persistent launch per call.  On first use (and whenever the buffers
- * change) the calls are captured into two CUDA graphs: every job's unpack,
+ * change) the calls are captured into two CUDA graphs: every job's unpack (in
+ * the fused pair mode only the copies of rows that are not whole 16-byte units),
  * then the single persistent correlate launch over all jobs' work items. */
 mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
                             cudaStream_t stream);

@@ -116,6 +116,7 @@ struct KJob {
   int64_t n_bl;        // N(N+1)/2
   int32_t n_inputs, n_tiles, n_pairs, kb, flush_blocks;
   int32_t n_time;       // fused pair mode: samples per integration
+  int32_t row_bytes;    // fused pair mode: bytes per sample row
   const uint8_t *volt;  // fused pair mode: packed samples of the launch's first channel
 };
 
@@ -501,8 +502,8 @@ static_assert(kConvThreads == 64 * 8, "one (sample, 16 inputs) unit per converte
 
 // Fused pair mode: one converter thread's loads of a work item: unit ct of a tile block is sample
 // ct / 8 of the block, inputs 16 (ct % 8) .. of the tile.  Tile block k of a
-// stage is tile k % nt of its block k / nt.  Samples past T and inputs past N
-// read as zero (N is a multiple of 16).
+// stage is tile k % nt of its block k / nt.  Samples past T and units
+// past the row (a whole number of them) read as zero.
 constexpr int kStageTiles = 6;
 struct RawLoads {
   const uint8_t *base;      // the unit of tile 0, block 0 of the next stage to load
@@ -514,7 +515,7 @@ struct RawLoads {
   __device__ __forceinline__ int start(const PairItem &it, const KJob &jb, int k0, int ct) {
     int tc[3], ti[3];
     const int nt = item_tiles(it, tc, ti), kps = stage_blocks(nt, true, 0);
-    const int N = jb.n_inputs, T = jb.n_time, row = k0 * 64 + (ct >> 3), x = (ct & 7) << 4;
+    const int N = jb.row_bytes, T = jb.n_time, row = k0 * 64 + (ct >> 3), x = (ct & 7) << 4;
     base = jb.volt + ((int64_t)tc[0] * T + row) * N + ti[0] * kTile + x;
     const int64_t d1 = (int64_t)(tc[1] - tc[0]) * T * N + (ti[1] - ti[0]) * kTile;
     const int64_t d2 = (int64_t)(ti[2] - ti[0]) * kTile;
@@ -1333,7 +1334,7 @@ bool pair_mode_supported(const TcJob *jobs, int n_jobs) {
 bool fused_pair_supported(const TcJob *jobs, int n_jobs, int sample_bits, int kind) {
   if (sample_bits != 4 || kind != MWAX_KIND_EXACT) return false;
   for (int j = 0; j < n_jobs; ++j)
-    if (jobs[j].n_inputs % 16 != 0 || jobs[j].n_time < 1 ||
+    if (jobs[j].row_bytes % 16 != 0 || jobs[j].row_bytes < jobs[j].n_inputs || jobs[j].n_time < 1 ||
         (jobs[j].op && (reinterpret_cast<uintptr_t>(jobs[j].op) & 15u) != 0))
       return false;
   return true;
@@ -1437,6 +1438,7 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
     kj.kb = job.kb;
     kj.flush_blocks = job.flush_blocks;
     kj.n_time = job.n_time;
+    kj.row_bytes = job.row_bytes;
     kj.volt = fused ? job.op : nullptr;  // the fused pair mode reads the packed samples
     items += (int64_t)job.n_chan * job.n_pairs;
     if (fused) continue;  // no operand tiles, no tensor map

@@ -254,6 +254,63 @@ __global__ void __launch_bounds__(256) unpack4_mn_kernel(const uint8_t *__restri
   }
 }
 
+// ---- 4-bit samples: rows padded to whole 16-byte units -----------------------------
+// For the fused pair mode, whose warps read whole 16-byte units: rows of N
+// bytes (N not a multiple of 16) copied to rows of P = N rounded up.  A thread
+// makes one 16-byte unit of a row from the one or two aligned units of the input
+// that hold it (an aligned unit is only read when at least one of its bytes is
+// wanted, so no read leaves the last unit of the buffer) by selecting words and
+// funnel shifts.  The P - N bytes past a row's end are whatever follows it: they
+// are operand rows past the last input, whose products are never stored.
+// HBM-bound, 2 bytes per sample (the unpack moves 3, and its operands are read
+// twice as wide).
+constexpr int kRepackRows = 4;  // rows in flight per thread
+__global__ void __launch_bounds__(256) repack4_kernel(const uint8_t *__restrict__ volt,
+                                                      uint8_t *__restrict__ out, int N, int P,
+                                                      int64_t rows) {
+  const int upr = P / 16;  // units per row
+  const bool long_rows = upr >= (int)blockDim.x;
+  const int rpb = long_rows ? 1 : (int)blockDim.x / upr;
+  const int r_off = long_rows ? 0 : (int)threadIdx.x / upr;
+  const int g0 = long_rows ? (int)threadIdx.x : (int)threadIdx.x - r_off * upr;
+  const int gstep = long_rows ? (int)blockDim.x : upr;
+  if (r_off >= rpb) return;
+  const int64_t rstride = (int64_t)gridDim.x * rpb;
+  for (int64_t r = (int64_t)blockIdx.x * rpb + r_off; r < rows; r += rstride * kRepackRows) {
+    for (int g = g0; g < upr; g += gstep) {
+      uint4 a[kRepackRows], b[kRepackRows];
+      int s[kRepackRows];
+#pragma unroll
+      for (int k = 0; k < kRepackRows; ++k) {
+        const int64_t rk = r + k * rstride;
+        a[k] = b[k] = make_uint4(0, 0, 0, 0);
+        s[k] = 0;
+        if (rk < rows) {
+          const uint8_t *at = volt + rk * N + 16 * g;
+          s[k] = (int)(reinterpret_cast<uintptr_t>(at) & 15);
+          const uint4 *src = reinterpret_cast<const uint4 *>(at - s[k]);
+          a[k] = __ldg(src);
+          if (s[k] + min(16, N - 16 * g) > 16) b[k] = __ldg(src + 1);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kRepackRows; ++k) {
+        const int64_t rk = r + k * rstride;
+        if (rk >= rows) break;
+        // words w[s/4 ..] of the eight, then the byte shift
+        const bool w2 = s[k] & 8, w1 = s[k] & 4;
+        const uint32_t x0 = w2 ? a[k].z : a[k].x, x1 = w2 ? a[k].w : a[k].y, x2 = w2 ? b[k].x : a[k].z,
+                       x3 = w2 ? b[k].y : a[k].w, x4 = w2 ? b[k].z : b[k].x, x5 = w2 ? b[k].w : b[k].y;
+        const uint32_t y0 = w1 ? x1 : x0, y1 = w1 ? x2 : x1, y2 = w1 ? x3 : x2, y3 = w1 ? x4 : x3, y4 = w1 ? x5 : x4;
+        const int sh = 8 * (s[k] & 3);
+        *reinterpret_cast<uint4 *>(out + rk * P + 16 * (int64_t)g) =
+            make_uint4(__funnelshift_r(y0, y1, sh), __funnelshift_r(y1, y2, sh), __funnelshift_r(y2, y3, sh),
+                       __funnelshift_r(y3, y4, sh));
+      }
+    }
+  }
+}
+
 constexpr int kPersistSmem = 64 * 1024;  // > what a correlate CTA leaves free on an SM
 
 // ---- TMA tile path --------------------------------------------------------------
@@ -478,6 +535,14 @@ cudaError_t launch_unpack4(const uint8_t *volt, int n_inputs, int n_time, int n_
     unpack4_mn_kernel<4><<<ctas, 256, smem, s>>>(volt, op, n_inputs, n_time, n_rows, kb, chan0, n_chan);
   else
     unpack4_mn_kernel<1><<<ctas, 256, smem, s>>>(volt, op, n_inputs, n_time, n_rows, kb, chan0, n_chan);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_repack4(const uint8_t *volt, int n_inputs, int row_bytes, int64_t rows, uint8_t *out,
+                           int sm_count, cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  if (n_inputs < 1 || row_bytes % 16 || row_bytes < n_inputs || sm_count < 1) return cudaErrorInvalidValue;
+  repack4_kernel<<<8 * sm_count, 256, 0, s>>>(volt, out, n_inputs, row_bytes, rows);
   return cudaGetLastError();
 }
 

@@ -34,7 +34,12 @@ struct JobState {
   int64_t op_chan_bytes = 0;  // operand bytes of one channel
   int64_t in_chan_bytes = 0;  // packed input bytes of one channel
   int64_t out_chan_bytes = 0;
-  uint8_t *op = nullptr;  // batch plans: operand buffer for all channels of this job
+  // 4-bit samples: a sample row in whole 16-byte units (more than n_inputs: the
+  // fused pair mode reads rows copied to that length)
+  int row_bytes = 0;
+  uint8_t *op = nullptr;  // batch plans: operand buffer (fused: padded rows) for all channels of this job
+  bool ragged() const { return row_bytes != job.n_inputs; }
+  int64_t row_chan_bytes() const { return (int64_t)job.n_time * row_bytes; }
 };
 
 }  // namespace
@@ -180,6 +185,7 @@ void derive(JobState &s) {
   s.op_chan_bytes = (int64_t)s.n_tiles * kTile * s.kb * kRowBytes;
   s.in_chan_bytes = (int64_t)j.n_time * j.n_inputs * bytes_per_sample(j.sample_bits);
   s.out_chan_bytes = s.n_bl * 8;
+  s.row_bytes = (j.n_inputs + 15) / 16 * 16;
   int64_t g = j.chan_group > 0 ? j.chan_group : kDefaultScratchBudget / s.op_chan_bytes;
   s.chan_group = (int)std::max<int64_t>(1, std::min<int64_t>(g, j.n_chan));
 }
@@ -240,6 +246,7 @@ TcJob tc_job(const JobState &s, const uint8_t *op, void *out_c0, int nc) {
   tj.flush_blocks = s.flush_blocks;
   tj.n_chan = nc;
   tj.n_time = s.job.n_time;
+  tj.row_bytes = s.row_bytes;
   tj.n_bl = s.n_bl;
   tj.k_split = s.k_split;
   return tj;
@@ -276,24 +283,37 @@ int resolve_split(const mwax_job &job, int mode, int kb, int64_t base_items, int
 constexpr int kFusedTiles = 2, kFusedBlocksPerTile = 4;
 constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
 
+// Rows that are not whole 16-byte units are copied to padded ones first (2 bytes
+// of traffic per sample, against 3 for the unpack and operands twice as wide);
+// the extra launch needs operands of 16 MB to pay.
+constexpr int64_t kRaggedOperandBytes = int64_t(16) << 20;
+
+int64_t operand_bytes(const TcJob &j) { return (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes; }
+
 bool fused_pays(const TcJob &j) {
+  if (j.row_bytes != j.n_inputs && operand_bytes(j) <= kRaggedOperandBytes) return false;
   if (j.n_tiles <= kFusedTiles) return true;
-  const int64_t operands = (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes;
-  return operands > kFusedOperandBytes && j.kb >= kFusedBlocksPerTile * j.n_tiles;
+  return operand_bytes(j) > kFusedOperandBytes && j.kb >= kFusedBlocksPerTile * j.n_tiles;
 }
 
 // Kernel mode for a job's mma_shape (0 = auto: the fused pair mode for 4-bit
-// exact arrays that allow it (fused_ok) where it pays for every job, else the
-// pair mode where every job integrates in one exact segment, else narrow); -1
-// when an explicit pair or fused pair request cannot be served.
+// exact arrays that allow it (fused_ok) where it pays for the jobs that hold most
+// of the launch's operands, else the pair mode where every job integrates in one
+// exact segment, else narrow); -1 when an explicit pair or fused pair request
+// cannot be served (an explicit fused request takes whole-unit rows only).
 int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok) {
   const bool pair_ok = pair_mode_supported(tj.data(), (int)tj.size());
-  if (mma_shape == 4) return pair_ok && fused_ok ? 3 : -1;
+  bool whole = true;
+  int64_t all = 0, pays = 0;
+  for (const TcJob &j : tj) {
+    whole = whole && j.row_bytes == j.n_inputs;
+    all += operand_bytes(j);
+    if (fused_pays(j)) pays += operand_bytes(j);
+  }
+  if (mma_shape == 4) return pair_ok && fused_ok && whole ? 3 : -1;
   if (mma_shape == 3) return pair_ok ? 2 : -1;
   if (mma_shape == 1 || mma_shape == 2) return mma_shape - 1;
-  bool pays = true;
-  for (const TcJob &j : tj) pays = pays && fused_pays(j);
-  if (pair_ok && fused_ok && pays) return 3;
+  if (pair_ok && fused_ok && 2 * pays > all) return 3;
   return pair_ok ? 2 : 0;
 }
 
@@ -445,10 +465,22 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
 
 // Channels [c0, c0+nc) of a single-job tensor plan, one after the other on
 // `st`: unpack into the scratch, then one persistent correlate launch (the
-// fused pair mode reads the packed samples itself: the launch only).
+// fused pair mode reads the packed samples itself, or the scratch's padded copy
+// of their rows).
 mwax_status run_group(mwax_plan_s *p, const JobState &s, const uint8_t *volt, int64_t c0, int nc,
                       void *out_c0, cudaStream_t st, bool use_pair = true) {
-  if (p->mode == 3) return correlate_group(p, s, volt + c0 * s.in_chan_bytes, nc, out_c0, st, use_pair);
+  if (p->mode == 3) {
+    const uint8_t *rows = volt + c0 * s.in_chan_bytes;
+    if (s.ragged()) {
+      TimedLaunch tu(p, 0, st);
+      const cudaError_t e = launch_repack4(rows, s.job.n_inputs, s.row_bytes, (int64_t)nc * s.job.n_time, p->scratch,
+                                           p->sm_count, st);
+      tu.done();
+      if (e != cudaSuccess) return cuda_status(e);
+      rows = p->scratch;
+    }
+    return correlate_group(p, s, rows, nc, out_c0, st, use_pair);
+  }
   mwax_status r = unpack_group(p, s, volt, c0, nc, p->scratch, 0, st);
   if (r != MWAX_OK) return r;
   return correlate_group(p, s, p->scratch, nc, out_c0, st, use_pair);
@@ -643,7 +675,8 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
       free_plan(p);
       return MWAX_ERR_INVALID_ARG;
     }
-    const int64_t one = p->mode == 3 ? 0 : s.op_chan_bytes * s.chan_group;  // fused: no operands
+    // fused: no operands, only the padded copy of ragged rows
+    const int64_t one = (p->mode != 3 ? s.op_chan_bytes : s.ragged() ? s.row_chan_bytes() : 0) * s.chan_group;
     const bool even = s.job.sample_bits == 8 ? s.job.n_inputs % 2 == 0 : true;
     // unpack_sms 0: the small unpack CTA runs beside the correlate on every SM
     // where the shape allows it, else 20 SMs are set aside for the unpack
@@ -733,20 +766,21 @@ mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
   }
   std::vector<TcJob> tj;
   for (const JobState &s : p->jobs) tj.push_back(tc_job(s, nullptr, nullptr, s.job.n_chan));
-  // the fused pair mode where every job allows it (the correlate then reads
-  // each job's voltages itself: no unpack graph, no operand buffers)
+  // the fused pair mode (the correlate then reads each job's voltages itself: no
+  // operand buffers, and an unpack graph only for the padded copies of ragged rows)
   const bool fused_ok = fused_pair_supported(tj.data(), n_jobs, jobs[0].sample_bits, jobs[0].kind);
   p->mode = choose_mode(jobs[0].mma_shape, tj, fused_ok);
   if (p->mode < 0) {
     free_plan(p);
     return MWAX_ERR_UNSUPPORTED;
   }
-  for (int k = 0; k < n_jobs && p->mode != 3; ++k) {
+  for (int k = 0; k < n_jobs; ++k) {
     JobState &s = p->jobs[k];
-    cudaError_t e = plan_alloc(reinterpret_cast<void **>(&s.op), (size_t)(s.op_chan_bytes * s.job.n_chan));
-    if (e == cudaSuccess)
-      e = cudaMemsetAsync(s.op, 0, (size_t)(s.op_chan_bytes * s.job.n_chan), stream);
-    p->scratch_bytes += s.op_chan_bytes * s.job.n_chan;
+    if (p->mode == 3 && !s.ragged()) continue;
+    const int64_t bytes = (p->mode == 3 ? s.row_chan_bytes() : s.op_chan_bytes) * s.job.n_chan;
+    cudaError_t e = plan_alloc(reinterpret_cast<void **>(&s.op), (size_t)bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s.op, 0, (size_t)bytes, stream);
+    p->scratch_bytes += bytes;
     tj[k].op = s.op;
     if (e != cudaSuccess) {
       free_plan(p);
@@ -856,8 +890,10 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages, 
     if (!is_device_ptr(voltages[k]) || !is_device_ptr(out[k]) || !aligned16(voltages[k]) ||
         !aligned16(out[k]))
       return MWAX_ERR_INVALID_ARG;
-  const bool fused = plan->mode == 3;  // no unpack graph: the correlate reads the voltages
-  bool same = (fused || plan->graph != nullptr) && plan->graph2 != nullptr;
+  const bool fused = plan->mode == 3;  // the correlate reads the voltages, or padded copies of ragged rows
+  bool prep = !fused;                  // graph 1: unpacks or copies
+  for (const JobState &s : plan->jobs) prep = prep || s.ragged();
+  bool same = (!prep || plan->graph != nullptr) && plan->graph2 != nullptr;
   for (int k = 0; k < nj && same; ++k)
     same = plan->graph_in[k] == voltages[k] && plan->graph_out[k] == out[k];
   if (!same) {
@@ -869,14 +905,16 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages, 
     std::vector<TcJob> tj(nj);
     for (int k = 0; k < nj; ++k)
       tj[k] = tc_job(plan->jobs[k],
-                     fused ? reinterpret_cast<const uint8_t *>(voltages[k]) : plan->jobs[k].op, out[k],
+                     fused && !plan->jobs[k].ragged() ? reinterpret_cast<const uint8_t *>(voltages[k])
+                                                      : plan->jobs[k].op,
+                     out[k],
                      plan->jobs[k].job.n_chan);
     cudaStream_t cs;
     cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_status(e);
-    // graph 1: every job's unpack (none in the fused pair mode); graph 2: one
+    // graph 1: every job's unpack (fused pair mode: ragged jobs' copies); graph 2: one
     // persistent launch over all items
-    for (int part = fused ? 1 : 0; part < 2 && e == cudaSuccess; ++part) {
+    for (int part = prep ? 0 : 1; part < 2 && e == cudaSuccess; ++part) {
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (part == 0) {
@@ -884,7 +922,11 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages, 
           const JobState &s = plan->jobs[k];
           const uint8_t *v = reinterpret_cast<const uint8_t *>(voltages[k]);
           const int uv = unpack_choice(s, v);
-          if (uv == 5)
+          if (fused && !s.ragged()) continue;
+          if (fused)
+            e = launch_repack4(v, s.job.n_inputs, s.row_bytes, (int64_t)s.job.n_chan * s.job.n_time, s.op,
+                               plan->sm_count, cs);
+          else if (uv == 5)
             e = launch_unpack_tile(v, s.job.sample_bits, s.job.n_inputs, s.job.n_time, s.n_tiles,
                                    s.kb, 0, s.job.n_chan, s.op, plan->sm_count * kTileCtasPerSm,
                                    plan->status, plan->timeout_ns, cs);
@@ -920,7 +962,7 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages, 
     plan->graph_out.assign(out, out + nj);
   }
   cudaError_t e = cudaSuccess;
-  if (!fused) {
+  if (prep) {
     TimedLaunch tu(plan, 0, plan->stream);
     e = cudaGraphLaunch(plan->graph, plan->stream);
     tu.done();

@@ -65,6 +65,11 @@ cudaError_t launch_unpack_persistent(const uint8_t *volt, int sample_bits, int n
 // 4-bit samples, any n_inputs: the streaming kernel (no shared memory) on
 // ctas / 2 CTAs of 256 threads.
 bool unpack_tile_supported(int sample_bits, int n_inputs);
+// 4-bit samples: `rows` rows of n_inputs bytes (inside a buffer that starts on a
+// 16-byte boundary) to rows of row_bytes (a multiple of 16; the bytes past
+// n_inputs are not defined).
+cudaError_t launch_repack4(const uint8_t *volt, int n_inputs, int row_bytes, int64_t rows, uint8_t *out,
+                           int sm_count, cudaStream_t s);
 cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_inputs, int n_time,
                                int n_tiles, int kb, int64_t chan0, int n_chan, uint8_t *op,
                                int ctas, int32_t *status, unsigned long long timeout_ns,
@@ -74,10 +79,11 @@ cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_input
 
 struct TcJob {
   const uint8_t *op;  // operand tiles of n_chan channels (layout: see launch_unpack); fused
-                      // pair mode: the packed samples [n_chan][n_time][n_inputs] themselves
+                      // pair mode: the packed samples [n_chan][n_time][row_bytes] themselves
   void *out;          // visibilities of the first of these n_chan channels
   int32_t n_inputs, n_tiles, n_pairs, kb, flush_blocks, n_chan;
   int32_t n_time = 0;  // samples per integration (read by the fused pair mode)
+  int32_t row_bytes = 0;  // bytes per sample row of op (fused pair mode: a multiple of 16)
   int64_t n_bl;
   // pair mode: time ranges per work item (1: whole integration; > 1: each
   // range's partial sums are added into the zeroed output with int32 atomics)
@@ -116,8 +122,8 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
 // Pair mode needs every job's integration in one exact segment (kb <=
 // flush_blocks), at most 255 tiles, kb < 2^28 and 1 <= k_split <= min(kb, 8).
 bool pair_mode_supported(const TcJob *jobs, int n_jobs);
-// The fused pair mode also needs 4-bit exact samples, n_inputs a multiple of
-// 16 (whole 16-byte sample rows) and sample buffers on 16-byte boundaries.
+// The fused pair mode also needs 4-bit exact samples, sample rows of whole
+// 16-byte units and sample buffers on 16-byte boundaries.
 bool fused_pair_supported(const TcJob *jobs, int n_jobs, int sample_bits, int kind);
 // The pair-mode work list of one launch over `jobs` (16 bytes per item).
 void build_pair_items(const TcJob *jobs, int n_jobs, std::vector<int4> &items);

@@ -52,3 +52,37 @@ def test_fused_choice_beyond_two_tiles(mw):  # noqa: F811
     p = mw.Plan(384, 2 * C, 11 * 64, 4)
     assert p.info().mma_shape == 3
     p.close()
+
+
+@pytest.mark.parametrize("N,T,C,G", [
+    (250, 2000, 140, 0), (129, 333, 700, 300), (115, 4097, 66, 0), (255, 1000, 66, 64), (17, 3000, 400, 0),
+    (300, 1001, 200, 95), (497, 1100, 70, 0)])
+def test_fused_ragged_rows(mw, N, T, C, G):  # noqa: F811
+    """Sample rows that are not whole 16-byte units, copied to padded ones:
+    every byte shift, channel groups that start inside a unit, odd N and T."""
+    kw = {"chan_group": G} if G else {}
+    spec = synth.Spec("rg", N, C, T, 4, seed=N + 5 * T + C, sigma=2, tone_amp=0.3)
+    p = mw.Plan(N, C, T, 4, **kw)
+    assert p.info().mma_shape == 4
+    out = p.correlate(device_volt(spec))
+    assert p.status() == 0
+    chans = sorted({0, 1, C // 2, C - 2, C - 1} | ({G - 1, G} if G else set()))
+    assert_exact(out.cpu().numpy()[chans], oracle_for(spec, chans), f"ragged {N},{T},{C},{G}")
+    p.close()
+
+
+def test_fused_batch_with_ragged_jobs(mw):  # noqa: F811
+    """One persistent launch over whole-unit and ragged jobs; the graphs are
+    built again for other buffers."""
+    jobs = [(300, 40, 1500), (48, 5, 300), (256, 60, 3000), (33, 7, 999)]
+    specs = [synth.Spec(f"rb{k}", n, c, t, 4, seed=70 + k, sigma=2, tone_amp=0.3) for k, (n, c, t) in enumerate(jobs)]
+    bp = mw.BatchPlan(jobs, sample_bits=4)
+    assert bp.info().mma_shape == 4
+    for _ in range(2):
+        vs = [device_volt(s) for s in specs]
+        outs = bp.correlate(vs)
+        assert bp.status() == 0
+        for s, o in zip(specs, outs):
+            chans = [0, s.n_chan // 2, s.n_chan - 1]
+            assert_exact(o.cpu().numpy()[chans], oracle_for(s, chans), f"ragged batch {s.name}")
+    bp.close()
