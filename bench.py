@@ -1080,13 +1080,14 @@ def main():
                     "kernel_ms_per_launch": tim.correlate_ms / max(1, tim.correlate_launches),
                     "unpack_ms_per_step": tim.unpack_ms / args.steps,
                     "correlate_ms_per_step": tim.correlate_ms / args.steps}
-        if tim.unpack_ms > 0:
+        if tim.unpack_ms > 0 and info.mma_shape != 4:
             roofline["unpack"] = unpack_roofline(rspec, info, tim, args.steps, peaks, peak_src)
         if info.mma_shape == 4:
             roofline["note"] = ("fused pair mode: the kernel also converts the packed samples into its "
                                 "operand tiles (no unpack pass, no operand buffer), so its duration is the "
-                                "whole step; the tensor pipe waits on that conversion")
-            roofline["packed_samples_gbs"] = (rspec.n_chan * rspec.n_time * rspec.n_inputs * args.steps
+                                "whole step; the tensor pipe shares the shared memory with that conversion")
+            roofline["packed_samples_gbs"] = (rspec.n_chan * rspec.n_time * rspec.n_inputs
+                                              * rspec.bytes_per_sample * args.steps
                                               / (tim.correlate_ms / 1e3) / 1e9)
         pk = tensor_peak_at_clock(rspec.sample_bits, clk,
                                   torch.cuda.get_device_properties(dev).multi_processor_count)
@@ -1122,9 +1123,11 @@ def main():
         "rtf": rtf,
         "roofline": roofline,
         # a checked-segment correlate launch is followed by the check kernel and
-        # the (usually empty) recompute launch inside the same timed record
+        # the (usually empty) recompute launch inside the same timed record (in the
+        # fused pair mode also the unpack of the channels to recompute)
         "gpu_launches": int(tim.unpack_launches
-                            + tim.correlate_launches * (3 if info.checked_segment else 1)),
+                            + tim.correlate_launches * (1 if not info.checked_segment
+                                                        else 4 if info.mma_shape == 4 else 3)),
         "clocks": clk,
     }
 

@@ -101,18 +101,19 @@ typedef struct {
                               for longer exact single-job plans with flush_blocks 0,
                               one checked segment, see mwax_plan_info.checked_segment;
                               else MWAX_ERR_UNSUPPORTED), 4 = the same work items with
-                              the unpack folded into the correlate: converter warps
+                              the unpack folded into the correlate: the epilogue warps
                               read the packed samples and write the operand tiles into
                               shared memory, so no operand buffer and no unpack pass
                               (4-bit exact samples in one exact segment with n_inputs a
                               multiple of 16 -- every job of a batch plan --, else
-                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 where it applies and
-                              n_inputs <= 256, or the operand tiles would exceed 64 MB and
-                              the integration has at least 256 samples per 128-input tile
-                              (other n_inputs too, from 16 MB of operand tiles on: their
-                              rows are copied to padded ones first; batch plans: where
-                              this holds for most of the operand bytes), else 3 where it
-                              applies, else 1                                             */
+                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 (also with 8-bit samples,
+                              the FP16 kind, a checked segment and any n_inputs, whose rows
+                              are copied to padded ones first where they are not whole
+                              16-byte units) for 4-bit jobs of n_inputs <= 256 and where the
+                              operand tiles would exceed 64 MB and the integration has at
+                              least 8 + n_tiles^2 / 2 time blocks (rows to be copied: 16 MB
+                              at least; batch plans: where this holds for most of the
+                              operand bytes), else 3 where it applies, else 1             */
   int32_t pipeline;        /* tuning: 1 = unpack then correlate each channel group on the
                               plan's stream, 2 = unpack the next group (second stream,
                               second scratch buffer) while the current group correlates,

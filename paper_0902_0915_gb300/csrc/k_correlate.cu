@@ -54,6 +54,7 @@
 // waits (bounded) for its own copies and MMAs in flight, frees its tensor
 // memory and returns.
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 #include <string.h>
 
@@ -75,16 +76,17 @@ constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB
 // about as much as two N=128 MMA issues, and every stage boundary leaves a
 // bubble in the tensor pipe, so the narrow shape takes three blocks (24
 // MMAs) per wait and per commit: two stages of 96 KB.
-// 3, fused pair: the pair mode for 4-bit samples with the unpack folded in:
-// sixteen warps read the packed samples from global memory and write the E4M3
-// operand tiles into the stages themselves (no operand buffer in HBM, no unpack
+// 3, fused pair: the pair mode with the unpack folded in: sixteen warps read the
+// packed samples from global memory and write the operand tiles (E4M3, or
+// binary16 for 8-bit samples, MN-major) into the stages themselves (no operand buffer in HBM, no unpack
 // pass), and drain each item's accumulator after its last stage.  Bound by the
 // shared memory that the MMAs' operands, 93 (N = 256) or 122 (N = 128) bytes of
 // 128 a cycle, and the converters' stores share.  256 inputs x 768 channels x
 // 20,000 samples: 1.87 ms (1.28 ms of MMA work at 2.07 GHz); eight converting
 // warps with an L2 prefetch ahead of them took 2.12, a ring of packed samples in
 // shared memory 1.94 (its extra reads and writes slow the MMAs), one-block
-// stages 2.2, two-block stages for items of two tiles 2.0.
+// stages 2.2, two-block stages for items of two tiles 2.0.  8 bits, 1024 x 384 x
+// 10,000: 11.2 ms, against 3.5 of unpack and 8.55 of pair mode.
 constexpr int kModeNarrow = 0, kModeWide = 1, kModePair = 2, kModePairFused = 3;
 constexpr int kEpiStageBytes = 32 * 128;  // pair mode: one warp's 32 rows x 16 (re, im) words
 
@@ -242,7 +244,14 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t addr) {
   return d;
 }
 
-// Operand tile of each sample width: its descriptor and the descriptor
+// The same for 16-bit operands: an MN atom is 64 inputs (8 K rows x 128 bytes),
+// so a 128-input tile has two, 8 KB apart, and B's next tile goes on in step.
+__device__ __forceinline__ uint64_t sw128_mn16_desc(uint32_t addr) {
+  return (sw128_mn_desc(addr) & ~((uint64_t)0x3FFF << 16)) | (uint64_t)(kTileBytes / 2 >> 4) << 16;
+}
+
+// Operand tile of each sample width (16: 8-bit samples in the fused pair mode,
+// whose converters write them MN-major, as they arrive): its descriptor and the descriptor
 // offsets (16-byte units) of the K slices re 0, re 1, im 0, im 1.
 // (and the factor that makes an accumulator value an integer)
 template <int BITS>
@@ -253,6 +262,13 @@ struct Op<8> {  // binary16, K-major
   static constexpr bool mn = false;
   static constexpr uint64_t re0 = 0, re1 = 2, im0 = 4, im1 = 6;
   static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return sw128_desc(addr); }
+};
+template <>
+struct Op<16> {  // binary16, MN-major: per 64 inputs 32 re rows, 32 im rows
+  static constexpr float units = 1.f;
+  static constexpr bool mn = true;
+  static constexpr uint64_t re0 = 0, re1 = 128, im0 = 256, im1 = 384;
+  static __device__ __forceinline__ uint64_t desc(uint32_t addr) { return sw128_mn16_desc(addr); }
 };
 template <>
 struct Op<4> {  // E4M3, MN-major
@@ -295,7 +311,7 @@ struct TileAt {
 template <int BITS>
 __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                        uint32_t accumulate) {
-  if constexpr (BITS == 8) {
+  if constexpr (BITS != 4) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
@@ -320,6 +336,17 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
         "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
         "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr));
+}
+
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&v)[32]) { tc_ld32(taddr, v); }
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+      "%12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+        "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
 }
 
@@ -497,14 +524,24 @@ __device__ __forceinline__ void narrow_block(uint32_t d_re, uint32_t d_im, uint6
   block_mmas<BITS, kTile>(d_re, d_im, da, db, acc0);
 }
 
+// Fused pair mode: the converter threads, one 16-byte unit of packed samples of
+// each tile block per thread: 16 inputs of one of 64 samples at 4 bits, 8 inputs
+// of one of 32 samples at 8 bits.
 constexpr int kConvThreads = Shape<kModePairFused>::epi_warps * 32;
-static_assert(kConvThreads == 64 * 8, "one (sample, 16 inputs) unit per converter thread and tile block");
+static_assert(kConvThreads == 512, "one unit per converter thread and tile block");
+template <int BITS>
+struct Unit {
+  static constexpr int samples = BITS == 4 ? 64 : 32;         // of a block
+  static constexpr int tile_bytes = BITS == 4 ? 128 : 256;    // of a tile in a sample row
+  static constexpr int per_row = tile_bytes / 16;
+};
 
-// Fused pair mode: one converter thread's loads of a work item: unit ct of a tile block is sample
-// ct / 8 of the block, inputs 16 (ct % 8) .. of the tile.  Tile block k of a
-// stage is tile k % nt of its block k / nt.  Samples past T and units
-// past the row (a whole number of them) read as zero.
+// One converter thread's loads of a work item: unit ct of a tile block is sample
+// ct / per_row of the block, 16 bytes at 16 (ct % per_row) of the tile's part of
+// the sample row.  Tile block k of a stage is tile k % nt of its block k / nt.
+// Samples past T and units past the row (a whole number of them) read as zero.
 constexpr int kStageTiles = 6;
+template <int BITS>
 struct RawLoads {
   const uint8_t *base;      // the unit of tile 0, block 0 of the next stage to load
   int64_t off[kStageTiles];  // each tile block's unit, from there
@@ -513,28 +550,29 @@ struct RawLoads {
   int64_t step;              // bytes of a stage's sample rows
 
   __device__ __forceinline__ int start(const PairItem &it, const KJob &jb, int k0, int ct) {
+    using U = Unit<BITS>;
     int tc[3], ti[3];
     const int nt = item_tiles(it, tc, ti), kps = stage_blocks(nt, true, 0);
-    const int N = jb.row_bytes, T = jb.n_time, row = k0 * 64 + (ct >> 3), x = (ct & 7) << 4;
-    base = jb.volt + ((int64_t)tc[0] * T + row) * N + ti[0] * kTile + x;
-    const int64_t d1 = (int64_t)(tc[1] - tc[0]) * T * N + (ti[1] - ti[0]) * kTile;
-    const int64_t d2 = (int64_t)(ti[2] - ti[0]) * kTile;
+    const int N = jb.row_bytes, T = jb.n_time, row = k0 * U::samples + ct / U::per_row, x = (ct % U::per_row) << 4;
+    base = jb.volt + ((int64_t)tc[0] * T + row) * N + ti[0] * U::tile_bytes + x;
+    const int64_t d1 = (int64_t)(tc[1] - tc[0]) * T * N + (ti[1] - ti[0]) * U::tile_bytes;
+    const int64_t d2 = (int64_t)(ti[2] - ti[0]) * U::tile_bytes;
     bool in[3];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) in[t] = t < nt && x < N - ti[t] * kTile;
+    for (int t = 0; t < 3; ++t) in[t] = t < nt && x < N - ti[t] * U::tile_bytes;
 #pragma unroll
     for (int k = 0; k < kStageTiles; ++k) {
       const int j = nt == 3 ? k / 3 : nt == 2 ? k / 2 : k;
       const int t = nt == 3 ? k % 3 : nt == 2 ? k % 2 : 0;
-      off[k] = (t == 0 ? 0 : t == 1 ? d1 : d2) + (int64_t)j * 64 * N;
-      lim[k] = j < kps && (t == 0 ? in[0] : t == 1 ? in[1] : in[2]) ? T - row - 64 * j : 0;
+      off[k] = (t == 0 ? 0 : t == 1 ? d1 : d2) + (int64_t)j * U::samples * N;
+      lim[k] = j < kps && (t == 0 ? in[0] : t == 1 ? in[1] : in[2]) ? T - row - U::samples * j : 0;
     }
-    rows = 64 * kps;
+    rows = U::samples * kps;
     step = (int64_t)rows * N;
     done = 0;
     return nt;
   }
-  // the next stage's units (lim: the sample rows past T read as zero)
+  // the next stage's units
   __device__ __forceinline__ void load(uint4 (&w)[kStageTiles]) {
 #pragma unroll
     for (int k = 0; k < kStageTiles; ++k) {
@@ -549,14 +587,38 @@ struct RawLoads {
   }
 };
 
-// One 16-byte unit of packed samples to its place in a tile: sample row t
-// (plane re) and 64 + t (plane im), chunk ch at its swizzled position.
+// int8 bytes (offset by 128, in the low bytes of two halves 0x64..) -> binary16:
+// 1024 + v + 128 exactly, minus 1152.
+__device__ __forceinline__ uint32_t s8_halves(uint32_t t) {
+  const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&t), bias);
+  return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// One unit to its place in a tile.  4-bit: sample row t of the re plane and 64 + t
+// (im), 16-byte chunk u % 8; 8-bit: 8 KB per 64 inputs, sample row t (re) and 32 + t
+// (im), chunk u % 8 of inputs half (u / 8) % 2; each chunk at its 128-byte swizzle
+// position.
+template <int BITS>
 __device__ __forceinline__ void fused_store(uint8_t *tile, int u, const uint4 &v) {
-  const int t = u >> 3, ch = u & 7;
+  const int t = u / Unit<BITS>::per_row, ch = u & 7;
   const int off = t * kRowBytes + ((ch ^ (t & 7)) << 4);
-  *reinterpret_cast<uint4 *>(tile + off) = make_uint4(nib4_re(v.x), nib4_re(v.y), nib4_re(v.z), nib4_re(v.w));
-  *reinterpret_cast<uint4 *>(tile + 64 * kRowBytes + off) =
-      make_uint4(nib4_im(v.x), nib4_im(v.y), nib4_im(v.z), nib4_im(v.w));
+  if constexpr (BITS == 4) {
+    *reinterpret_cast<uint4 *>(tile + off) = make_uint4(nib4_re(v.x), nib4_re(v.y), nib4_re(v.z), nib4_re(v.w));
+    *reinterpret_cast<uint4 *>(tile + 64 * kRowBytes + off) =
+        make_uint4(nib4_im(v.x), nib4_im(v.y), nib4_im(v.z), nib4_im(v.w));
+  } else {
+    uint8_t *half = tile + ((u >> 3) & 1) * (kTileBytes / 2);
+    const uint32_t x[4] = {v.x ^ 0x80808080u, v.y ^ 0x80808080u, v.z ^ 0x80808080u, v.w ^ 0x80808080u};
+    uint32_t re[4], im[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      re[k] = s8_halves(__byte_perm(x[k], 0x64646464u, 0x4240));
+      im[k] = s8_halves(__byte_perm(x[k], 0x64646464u, 0x4341));
+    }
+    *reinterpret_cast<uint4 *>(half + off) = make_uint4(re[0], re[1], re[2], re[3]);
+    *reinterpret_cast<uint4 *>(half + 32 * kRowBytes + off) = make_uint4(im[0], im[1], im[2], im[3]);
+  }
 }
 
 // The integer that an accumulator word holds (exact below 2^24 units).
@@ -606,17 +668,18 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
   const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * kTile);
   uint32_t *out = reinterpret_cast<uint32_t *>(jb.out) + (int64_t)c * jb.n_bl * 2;
   const int n = jb.n_inputs;
-  constexpr int kChunks = 4 * 8 / EW;  // 32-column chunks of this warp
-  const int col0 = 32 * kChunks * (part % (EW / 8));
+  constexpr int kCols = kTile * 8 / EW;     // this warp's columns
+  constexpr int kChunk = EW == 8 ? 32 : 16;  // at a time (96 registers a thread with 16 warps)
+  const int col0 = kCols * (part % (EW / 8));
 #pragma unroll
-  for (int cc = 0; cc < kChunks; ++cc) {
-    uint32_t vre[32], vim[32];
+  for (int cc = 0; cc < kCols; cc += kChunk) {
+    uint32_t vre[kChunk], vim[kChunk];
     if (has) {
-      tc_ld32(trow + col0 + 32 * cc, vre);
-      tc_ld32(trow + 2 * kTile + col0 + 32 * cc, vim);
+      tc_ld(trow + col0 + cc, vre);
+      tc_ld(trow + 2 * kTile + col0 + cc, vim);
       tc_wait_ld();
     }
-    if (cc == kChunks - 1) {
+    if (cc + kChunk == kCols) {
       // every column of this warp is in registers: release the accumulator
       // (test hook: withholding one release makes the MMA warp's bounded
       // wait run out -> MWAX_ERR_TIMEOUT, clean exit)
@@ -627,19 +690,19 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
     if (!has) continue;
     if constexpr (KIND == MWAX_KIND_EXACT) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
+      for (int k = 0; k < kChunk; ++k) {
         vre[k] = (uint32_t)acc_int<BITS>(vre[k]);
         vim[k] = (uint32_t)acc_int<BITS>(vim[k]);
       }
     }
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < kChunk; half += 16) {
 #pragma unroll
       for (int k = 0; k < 16; ++k)
         *reinterpret_cast<uint2 *>(stg + lane * 128 + ((k ^ (lane & 15)) << 3)) =
-            make_uint2(vre[16 * half + k], vim[16 * half + k]);
+            make_uint2(vre[half + k], vim[half + k]);
       __syncwarp();
-      const int j = J * kTile + col0 + 32 * cc + 16 * half + (lane & 15);
+      const int j = J * kTile + col0 + cc + half + (lane & 15);
       const int i0 = I * kTile + q * 32;
       if (it.n_split > 1)  // one time range of several: exact integer adds
         store_rows<true>(stg, out, lane, i0, j, n);
@@ -836,7 +899,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
         const PairItem it = decode_pair_item(__ldg(p.items + item));
         int k0, k1;
         item_blocks(it, p.job[it.job].kb, k0, k1);
-        RawLoads ld;
+        RawLoads<BITS> ld;
         const int nt = ld.start(it, p.job[it.job], k0, ct), kps = stage_blocks(nt, true, 0);
         uint4 w[kStageTiles];
         ld.load(w);
@@ -849,7 +912,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           const int n = nt * min(kps, k1 - kb);  // tile blocks of the stage
 #pragma unroll
           for (int k = 0; k < kStageTiles; ++k)
-            if (k < n) fused_store(st_base + k * kTileBytes, ct, w[k]);
+            if (k < n) fused_store<BITS>(st_base + k * kTileBytes, ct, w[k]);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(full(stage));
@@ -1309,9 +1372,9 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
   if (mode == kModeWide) return prepare_shape<kModeWide>(sample_bits, kind, bytes);
   if (mode == kModePair) return prepare_shape<kModePair>(sample_bits, kind, bytes);
   if (mode == kModePairFused)
-    return sample_bits == 4 && kind == MWAX_KIND_EXACT
-               ? set_smem_attr<4, MWAX_KIND_EXACT, kModePairFused>(bytes)
-               : cudaErrorInvalidValue;
+    return sample_bits == 4          ? set_smem_attr<4, MWAX_KIND_EXACT, kModePairFused>(bytes)
+           : kind == MWAX_KIND_FP16 ? set_smem_attr<16, MWAX_KIND_FP16, kModePairFused>(bytes)
+                                    : set_smem_attr<16, MWAX_KIND_EXACT, kModePairFused>(bytes);
   return prepare_shape<kModeNarrow>(sample_bits, kind, bytes);
 }
 
@@ -1331,10 +1394,9 @@ bool pair_mode_supported(const TcJob *jobs, int n_jobs) {
   return n_jobs >= 1 && n_jobs <= kMaxJobs;
 }
 
-bool fused_pair_supported(const TcJob *jobs, int n_jobs, int sample_bits, int kind) {
-  if (sample_bits != 4 || kind != MWAX_KIND_EXACT) return false;
+bool fused_pair_supported(const TcJob *jobs, int n_jobs) {
   for (int j = 0; j < n_jobs; ++j)
-    if (jobs[j].row_bytes % 16 != 0 || jobs[j].row_bytes < jobs[j].n_inputs || jobs[j].n_time < 1 ||
+    if (jobs[j].row_bytes % 16 != 0 || jobs[j].row_bytes < jobs[j].packed_row || jobs[j].n_time < 1 ||
         (jobs[j].op && (reinterpret_cast<uintptr_t>(jobs[j].op) & 15u) != 0))
       return false;
   return true;
@@ -1412,7 +1474,7 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
   const bool fused = cfg.mode == kModePairFused;
   if (pair && (!pair_mode_supported(jobs, n_jobs) || !cfg.items || cfg.n_items < 0))
     return cudaErrorInvalidValue;
-  if (fused && !fused_pair_supported(jobs, n_jobs, cfg.sample_bits, cfg.kind))
+  if (fused && !fused_pair_supported(jobs, n_jobs))
     return cudaErrorInvalidValue;
   if ((cfg.chan_map || cfg.n_chan_dev) &&
       (pair || n_jobs != 1 || !cfg.chan_map || !cfg.n_chan_dev))
@@ -1478,9 +1540,15 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
     launch_shape<kModeWide>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
   else if (cfg.mode == kModePair)
     launch_shape<kModePair>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else if (fused)
-    correlate_tc_kernel<4, MWAX_KIND_EXACT, kModePairFused>
-        <<<grid, Shape<kModePairFused>::warps * 32, smem, s>>>(maps, kp);
+  else if (fused) {
+    constexpr int threads = Shape<kModePairFused>::warps * 32;
+    if (cfg.sample_bits == 4)
+      correlate_tc_kernel<4, MWAX_KIND_EXACT, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
+    else if (cfg.kind == MWAX_KIND_FP16)
+      correlate_tc_kernel<16, MWAX_KIND_FP16, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
+    else
+      correlate_tc_kernel<16, MWAX_KIND_EXACT, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
+  }
   else
     launch_shape<kModeNarrow>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
   return cudaGetLastError();

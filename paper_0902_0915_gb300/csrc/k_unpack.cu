@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) unpack4_mn_kernel(const uint8_t *__restri
   }
 }
 
-// ---- 4-bit samples: rows padded to whole 16-byte units -----------------------------
+// ---- sample rows padded to whole 16-byte units -------------------------------------
 // For the fused pair mode, whose warps read whole 16-byte units: rows of N
 // bytes (N not a multiple of 16) copied to rows of P = N rounded up.  A thread
 // makes one 16-byte unit of a row from the one or two aligned units of the input
@@ -262,10 +262,10 @@ __global__ void __launch_bounds__(256) unpack4_mn_kernel(const uint8_t *__restri
 // wanted, so no read leaves the last unit of the buffer) by selecting words and
 // funnel shifts.  The P - N bytes past a row's end are whatever follows it: they
 // are operand rows past the last input, whose products are never stored.
-// HBM-bound, 2 bytes per sample (the unpack moves 3, and its operands are read
-// twice as wide).
+// HBM-bound, twice the sample bytes (the unpack moves three times as many, and
+// its operands are read twice as wide).
 constexpr int kRepackRows = 4;  // rows in flight per thread
-__global__ void __launch_bounds__(256) repack4_kernel(const uint8_t *__restrict__ volt,
+__global__ void __launch_bounds__(256) repack_kernel(const uint8_t *__restrict__ volt,
                                                       uint8_t *__restrict__ out, int N, int P,
                                                       int64_t rows) {
   const int upr = P / 16;  // units per row
@@ -375,13 +375,16 @@ __device__ __forceinline__ void put_raw_box(uint8_t *raw, const uint32_t (&v)[kR
   for (int j = 0; j < kRawWords; ++j) reinterpret_cast<uint32_t *>(raw)[j * kTileThreads + threadIdx.x] = v[j];
 }
 
+__device__ __forceinline__ int chan_at(const int32_t *map, int64_t k) { return map ? __ldg(map + k) : (int)k; }
+
 // TMA_IN = false: the raw box is loaded by the threads (load_raw_box).
+// chan_map, n_chan_dev (or null): the channels to unpack, listed on the device.
 template <bool TMA_IN>
 __global__ void __launch_bounds__(kTileThreads, 6)
     unpack8_tile_kernel(const __grid_constant__ CUtensorMap in_map,
                         const __grid_constant__ CUtensorMap out_map, const uint8_t *volt, int N,
                         int T, int n_tiles, int kb, int64_t chan0, int n_chan, int32_t *status,
-                        unsigned long long tmo) {
+                        unsigned long long tmo, const int32_t *chan_map, const int32_t *n_chan_dev) {
   extern __shared__ __align__(1024) uint8_t sm_base[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(sm_base) + 1023) &
                                             ~static_cast<uintptr_t>(1023));
@@ -389,6 +392,7 @@ __global__ void __launch_bounds__(kTileThreads, 6)
   uint8_t *raw = sm + kTile * kRowBytes;  // 32 samples x 256 B
   __shared__ __align__(8) uint64_t bar;
   const uint32_t b = (uint32_t)__cvta_generic_to_shared(&bar);
+  if (n_chan_dev) n_chan = *n_chan_dev;
   const int64_t tasks = (int64_t)n_chan * kb * n_tiles;  // tile fastest
   const int n_rows = n_tiles * kTile;
   if (threadIdx.x == 0) {
@@ -403,7 +407,7 @@ __global__ void __launch_bounds__(kTileThreads, 6)
   auto issue = [&](int64_t k) {
     const int tile = (int)(k % n_tiles);
     const int64_t cb = k / n_tiles;
-    const int c = (int)(cb / kb), tb = (int)(cb % kb);
+    const int c = chan_at(chan_map, cb / kb), tb = (int)(cb % kb);
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b),
                  "r"((uint32_t)kTileRawBytes)
                  : "memory");
@@ -420,7 +424,7 @@ __global__ void __launch_bounds__(kTileThreads, 6)
   auto fetch = [&](int64_t kk) {
     const int tile_l = (int)(kk % n_tiles);
     const int64_t cb_l = kk / n_tiles;
-    const int c_l = (int)(cb_l / kb), tb_l = (int)(cb_l % kb);
+    const int c_l = chan_at(chan_map, cb_l / kb), tb_l = (int)(cb_l % kb);
     fetch_raw_box<8>(volt, rv, 2 * (int64_t)N, (chan0 + c_l) * (int64_t)T + (int64_t)tb_l * 32,
                        min(32, T - tb_l * 32), tile_l * 256);
   };
@@ -446,7 +450,7 @@ __global__ void __launch_bounds__(kTileThreads, 6)
     __syncthreads();
     const int tile = (int)(k % n_tiles);
     const int64_t cb = k / n_tiles;
-    const int c = (int)(cb / kb), tb = (int)(cb % kb);
+    const int c = chan_at(chan_map, cb / kb), tb = (int)(cb % kb);
     const int rows = min(32, T - tb * 32);  // samples of this block (the box may run into the next channel)
     uint32_t v[32];
 #pragma unroll
@@ -538,11 +542,11 @@ cudaError_t launch_unpack4(const uint8_t *volt, int n_inputs, int n_time, int n_
   return cudaGetLastError();
 }
 
-cudaError_t launch_repack4(const uint8_t *volt, int n_inputs, int row_bytes, int64_t rows, uint8_t *out,
-                           int sm_count, cudaStream_t s) {
+cudaError_t launch_repack(const uint8_t *volt, int packed_row, int row_bytes, int64_t rows, uint8_t *out,
+                          int sm_count, cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
-  if (n_inputs < 1 || row_bytes % 16 || row_bytes < n_inputs || sm_count < 1) return cudaErrorInvalidValue;
-  repack4_kernel<<<8 * sm_count, 256, 0, s>>>(volt, out, n_inputs, row_bytes, rows);
+  if (packed_row < 1 || row_bytes % 16 || row_bytes < packed_row || sm_count < 1) return cudaErrorInvalidValue;
+  repack_kernel<<<8 * sm_count, 256, 0, s>>>(volt, out, packed_row, row_bytes, rows);
   return cudaGetLastError();
 }
 
@@ -587,9 +591,10 @@ int unpack_tile_smem_bytes() { return 1024 + kTile * kRowBytes + kTileRawBytes; 
 cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_inputs, int n_time,
                                int n_tiles, int kb, int64_t chan0, int n_chan, uint8_t *op,
                                int ctas, int32_t *status, unsigned long long timeout_ns,
-                               cudaStream_t s) {
+                               cudaStream_t s, const int32_t *chan_map, const int32_t *n_chan_dev) {
   if (n_chan <= 0) return cudaSuccess;
   if (ctas < 1 || !unpack_tile_supported(sample_bits, n_inputs)) return cudaErrorInvalidValue;
+  if ((chan_map || n_chan_dev) && (sample_bits != 8 || !chan_map || !n_chan_dev)) return cudaErrorInvalidValue;
   if (sample_bits == 4) {
     // (`ctas` counts 128-thread tile CTAs; the streaming kernel's CTAs have 256;
     // run alone it takes MWAX_U4_CTAS_PER_SM per SM)
@@ -645,7 +650,8 @@ cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_input
     return r;
   });
   if (ea != cudaSuccess) return ea;
-#define MWAX_TILE_ARGS in_map, out_map, volt, n_inputs, n_time, n_tiles, kb, chan0, n_chan, status, timeout_ns
+#define MWAX_TILE_ARGS \
+  in_map, out_map, volt, n_inputs, n_time, n_tiles, kb, chan0, n_chan, status, timeout_ns, chan_map, n_chan_dev
   if (tma_in)
     unpack8_tile_kernel<true><<<ctas, kTileThreads, smem, s>>>(MWAX_TILE_ARGS);
   else

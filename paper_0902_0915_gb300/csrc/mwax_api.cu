@@ -34,11 +34,11 @@ struct JobState {
   int64_t op_chan_bytes = 0;  // operand bytes of one channel
   int64_t in_chan_bytes = 0;  // packed input bytes of one channel
   int64_t out_chan_bytes = 0;
-  // 4-bit samples: a sample row in whole 16-byte units (more than n_inputs: the
-  // fused pair mode reads rows copied to that length)
-  int row_bytes = 0;
+  // a sample row as it arrives and in whole 16-byte units (more: the fused pair
+  // mode reads rows copied to that length)
+  int packed_row = 0, row_bytes = 0;
   uint8_t *op = nullptr;  // batch plans: operand buffer (fused: padded rows) for all channels of this job
-  bool ragged() const { return row_bytes != job.n_inputs; }
+  bool ragged() const { return row_bytes != packed_row; }
   int64_t row_chan_bytes() const { return (int64_t)job.n_time * row_bytes; }
 };
 
@@ -61,6 +61,7 @@ struct mwax_plan_s {
   unsigned long long timeout_ns = mwax::kDefaultTimeoutNs;
   std::vector<mwax::JobState> jobs;
   uint8_t *scratch = nullptr;  // single-job plans: operand buffer for one channel group
+  uint8_t *rows = nullptr;      // fused pair mode: padded copies of a group's ragged rows
   uint8_t *scratch2 = nullptr;  // second buffer when unpack and correlate overlap
   int64_t scratch_bytes = 0;
   // overlapped pipeline: unpack of group g+1 (aux stream) runs beside the
@@ -185,7 +186,8 @@ void derive(JobState &s) {
   s.op_chan_bytes = (int64_t)s.n_tiles * kTile * s.kb * kRowBytes;
   s.in_chan_bytes = (int64_t)j.n_time * j.n_inputs * bytes_per_sample(j.sample_bits);
   s.out_chan_bytes = s.n_bl * 8;
-  s.row_bytes = (j.n_inputs + 15) / 16 * 16;
+  s.packed_row = j.n_inputs * bytes_per_sample(j.sample_bits);
+  s.row_bytes = (s.packed_row + 15) / 16 * 16;
   int64_t g = j.chan_group > 0 ? j.chan_group : kDefaultScratchBudget / s.op_chan_bytes;
   s.chan_group = (int)std::max<int64_t>(1, std::min<int64_t>(g, j.n_chan));
 }
@@ -247,6 +249,7 @@ TcJob tc_job(const JobState &s, const uint8_t *op, void *out_c0, int nc) {
   tj.n_chan = nc;
   tj.n_time = s.job.n_time;
   tj.row_bytes = s.row_bytes;
+  tj.packed_row = s.packed_row;
   tj.n_bl = s.n_bl;
   tj.k_split = s.k_split;
   return tj;
@@ -272,15 +275,18 @@ int resolve_split(const mwax_job &job, int mode, int kb, int64_t base_items, int
 // converted once per work item that reads it (about n_tiles / 2 + 1 times per
 // channel and time block), against one write and one read of the unpacked
 // operands through HBM or, while they fit it, L2 without the fusion; and its
-// conversion stops during an item's drain.  So: always up to two tiles; with
-// more, when the launch's operands take over half of the L2 (64 MB) and an item
-// has enough blocks per tile to hide the drain.  Measured, fused against unpack
-// + pair, in microseconds: 256 inputs x 768 channels x 20,000 samples 1791 /
-// 3413, 384 x 512 x 20,000 2652 / 4004, 512 x 128 x 2000 179 / 201, 768 x 256 x
-// 20,000 4490 / 5228, 1024 x 192 x 20,000 5658 / 6127, 1024 x 64 x 3000 374 /
-// 379; and on the other side 512 x 32 x 1000 50 / 47, 768 x 32 x 1000 76 / 73,
-// 1024 x 64 x 1000 209 / 181.
-constexpr int kFusedTiles = 2, kFusedBlocksPerTile = 4;
+// conversion stops during an item's drain.  So: always for 4-bit samples of up
+// to two tiles; else when the launch's operands take over half of the L2 (64 MB)
+// and an item has enough blocks to hide the drain, the more the less each block
+// saves (8 + n_tiles^2 / 2).  Measured, fused against unpack + pair, in
+// microseconds, 4 bits: 256 inputs x 768 channels x 20,000 samples 1821 / 3449,
+// 384 x 512 x 20,000 2652 / 4004, 512 x 64 x 1000 73 / 76, 768 x 256 x 20,000 4490
+// / 5228, 1024 x 192 x 20,000 5644 / 6188, 1024 x 64 x 3000 374 / 379; 8 bits: 128 x
+// 300 x 5000 152 / 332, 512 x 96 x 10,000 929 / 1233, 1024 x 384 x 10,000 11,186 /
+// 12,069, 1024 x 64 x 2000 481 / 515; on the other side 512 x 32 x 1000 (4 bits, 33
+// MB) 50 / 47, 768 x 32 x 1000 76 / 73, 1024 x 64 x 1000 209 / 181, 1024 x 128 x 1000
+// (8 bits, 32 blocks) 609 / 568.
+constexpr int kFusedTiles = 2;
 constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
 
 // Rows that are not whole 16-byte units are copied to padded ones first (2 bytes
@@ -290,25 +296,26 @@ constexpr int64_t kRaggedOperandBytes = int64_t(16) << 20;
 
 int64_t operand_bytes(const TcJob &j) { return (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes; }
 
-bool fused_pays(const TcJob &j) {
-  if (j.row_bytes != j.n_inputs && operand_bytes(j) <= kRaggedOperandBytes) return false;
-  if (j.n_tiles <= kFusedTiles) return true;
-  return operand_bytes(j) > kFusedOperandBytes && j.kb >= kFusedBlocksPerTile * j.n_tiles;
+bool fused_pays(const TcJob &j, int sample_bits) {
+  if (j.row_bytes != j.packed_row && operand_bytes(j) <= kRaggedOperandBytes) return false;
+  if (sample_bits == 4 && j.n_tiles <= kFusedTiles) return true;
+  return operand_bytes(j) > kFusedOperandBytes && j.kb >= 8 + j.n_tiles * j.n_tiles / 2;
 }
 
-// Kernel mode for a job's mma_shape (0 = auto: the fused pair mode for 4-bit
-// exact arrays that allow it (fused_ok) where it pays for the jobs that hold most
+// Kernel mode for a job's mma_shape (0 = auto: the fused pair mode for arrays
+// that allow it (fused_ok) where it pays for the jobs that hold most
 // of the launch's operands, else the pair mode where every job integrates in one
 // exact segment, else narrow); -1 when an explicit pair or fused pair request
-// cannot be served (an explicit fused request takes whole-unit rows only).
-int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok) {
+// cannot be served (an explicit fused request takes 4-bit samples in whole-unit
+// rows only).
+int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int sample_bits) {
   const bool pair_ok = pair_mode_supported(tj.data(), (int)tj.size());
   bool whole = true;
   int64_t all = 0, pays = 0;
   for (const TcJob &j : tj) {
-    whole = whole && j.row_bytes == j.n_inputs;
+    whole = whole && j.row_bytes == j.packed_row && sample_bits == 4;
     all += operand_bytes(j);
-    if (fused_pays(j)) pays += operand_bytes(j);
+    if (fused_pays(j, sample_bits)) pays += operand_bytes(j);
   }
   if (mma_shape == 4) return pair_ok && fused_ok && whole ? 3 : -1;
   if (mma_shape == 3) return pair_ok ? 2 : -1;
@@ -420,11 +427,21 @@ cudaError_t checked_call_done(mwax_plan_s *p, cudaStream_t st) {
   return e;
 }
 
+// Fused checked plans: the operands of nc channels (or of the listed ones) from
+// sample rows of whole 16-byte units; inputs past N only make operand rows whose
+// products are never stored.
+cudaError_t unpack_rows(mwax_plan_s *p, const JobState &s, const uint8_t *rows, int nc, cudaStream_t st,
+                        const int32_t *chan_map, const int32_t *n_chan_dev) {
+  return launch_unpack_tile(rows, s.job.sample_bits, s.row_bytes / bytes_per_sample(s.job.sample_bits), s.job.n_time,
+                            s.n_tiles, s.kb, 0, nc, p->scratch, p->sm_count * kTileCtasPerSm, p->status,
+                            p->timeout_ns, st, chan_map, n_chan_dev);
+}
+
 mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op, int nc,
                             void *out_c0, cudaStream_t st, bool use_pair = true) {
   TcJob tj = tc_job(s, op, out_c0, nc);
   TcLaunch cfg = launch_cfg(p);
-  if (p->mode == 2 && !use_pair) {  // a checked plan's narrow call (never fused)
+  if (pair_like(p->mode) && !use_pair) {  // a checked plan's narrow call (op: operand tiles)
     cfg.mode = 0;
     cfg.stages = correlate_tc_max_stages(0);
     TimedLaunch tn(p, 1, st);
@@ -449,6 +466,10 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
     if (e == cudaSuccess) {
       // the flagged channels again, narrow shape, exact segments (an empty
       // list makes every CTA return at once)
+      if (p->mode == 3) {  // their operands first
+        e = unpack_rows(p, s, op, nc, st, p->bad + 1, p->bad);
+        op = p->scratch;
+      }
       TcJob fj = tc_job(s, op, out_c0, nc);
       TcLaunch fc = launch_cfg(p);
       fc.mode = 0;
@@ -456,7 +477,7 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
       fc.withhold_seg = -1;
       fc.chan_map = p->bad + 1;
       fc.n_chan_dev = p->bad;
-      e = launch_correlate_tc(&fj, 1, fc, st);
+      if (e == cudaSuccess) e = launch_correlate_tc(&fj, 1, fc, st);
     }
   }
   tc.done();
@@ -473,8 +494,15 @@ mwax_status run_group(mwax_plan_s *p, const JobState &s, const uint8_t *volt, in
     const uint8_t *rows = volt + c0 * s.in_chan_bytes;
     if (s.ragged()) {
       TimedLaunch tu(p, 0, st);
-      const cudaError_t e = launch_repack4(rows, s.job.n_inputs, s.row_bytes, (int64_t)nc * s.job.n_time, p->scratch,
-                                           p->sm_count, st);
+      const cudaError_t e = launch_repack(rows, s.packed_row, s.row_bytes, (int64_t)nc * s.job.n_time, p->rows,
+                                          p->sm_count, st);
+      tu.done();
+      if (e != cudaSuccess) return cuda_status(e);
+      rows = p->rows;
+    }
+    if (!use_pair) {  // a checked plan's narrow call: the operands of every channel
+      TimedLaunch tu(p, 0, st);
+      const cudaError_t e = unpack_rows(p, s, rows, nc, st, nullptr, nullptr);
       tu.done();
       if (e != cudaSuccess) return cuda_status(e);
       rows = p->scratch;
@@ -544,6 +572,7 @@ void free_plan(mwax_plan_s *p) {
     if (s.op) cudaFree(s.op);
   if (p->scratch) cudaFree(p->scratch);
   if (p->scratch2) cudaFree(p->scratch2);
+  if (p->rows) cudaFree(p->rows);
   if (p->status) cudaFree(p->status);
   if (p->items) cudaFree(p->items);
   if (p->bad) cudaFree(p->bad);
@@ -655,8 +684,8 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
                  (job->mma_shape == 0 || job->mma_shape == 3) && s.flush_blocks < s.kb &&
                  s.n_tiles <= 255;
     if (p->checked) full[0].flush_blocks = s.kb;
-    const bool fused_ok = !p->checked && fused_pair_supported(full.data(), 1, job->sample_bits, job->kind);
-    p->mode = choose_mode(job->mma_shape, full, fused_ok);
+    const bool fused_ok = fused_pair_supported(full.data(), 1) && !(p->checked && job->sample_bits == 4);
+    p->mode = choose_mode(job->mma_shape, full, fused_ok, job->sample_bits);
     if (p->mode < 0) {
       free_plan(p);
       return MWAX_ERR_UNSUPPORTED;
@@ -675,8 +704,10 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
       free_plan(p);
       return MWAX_ERR_INVALID_ARG;
     }
-    // fused: no operands, only the padded copy of ragged rows
-    const int64_t one = (p->mode != 3 ? s.op_chan_bytes : s.ragged() ? s.row_chan_bytes() : 0) * s.chan_group;
+    // fused: no operands (but a checked plan's, for the channels to recompute),
+    // only the padded copy of ragged rows
+    const int64_t one = (p->mode != 3 || p->checked ? s.op_chan_bytes : 0) * s.chan_group;
+    const int64_t rows = (p->mode == 3 && s.ragged() ? s.row_chan_bytes() : 0) * s.chan_group;
     const bool even = s.job.sample_bits == 8 ? s.job.n_inputs % 2 == 0 : true;
     // unpack_sms 0: the small unpack CTA runs beside the correlate on every SM
     // where the shape allows it, else 20 SMs are set aside for the unpack
@@ -687,9 +718,10 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
                         : 20;
     p->overlap = job->pipeline == 2 && s.chan_group < s.job.n_chan && even &&
                  p->unpack_sms < p->sm_count && p->mode != 3;
-    p->scratch_bytes = one * (p->overlap ? 2 : 1);
+    p->scratch_bytes = one * (p->overlap ? 2 : 1) + rows;
     cudaError_t e = cudaSuccess;
-    if (one > 0) {
+    if (rows > 0) e = plan_alloc(reinterpret_cast<void **>(&p->rows), (size_t)rows);
+    if (e == cudaSuccess && one > 0) {
       e = plan_alloc(reinterpret_cast<void **>(&p->scratch), (size_t)one);
       if (e == cudaSuccess) e = cudaMemsetAsync(p->scratch, 0, (size_t)one, stream);
     }
@@ -768,8 +800,8 @@ mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
   for (const JobState &s : p->jobs) tj.push_back(tc_job(s, nullptr, nullptr, s.job.n_chan));
   // the fused pair mode (the correlate then reads each job's voltages itself: no
   // operand buffers, and an unpack graph only for the padded copies of ragged rows)
-  const bool fused_ok = fused_pair_supported(tj.data(), n_jobs, jobs[0].sample_bits, jobs[0].kind);
-  p->mode = choose_mode(jobs[0].mma_shape, tj, fused_ok);
+  const bool fused_ok = fused_pair_supported(tj.data(), n_jobs);
+  p->mode = choose_mode(jobs[0].mma_shape, tj, fused_ok, jobs[0].sample_bits);
   if (p->mode < 0) {
     free_plan(p);
     return MWAX_ERR_UNSUPPORTED;
@@ -924,7 +956,7 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages, 
           const int uv = unpack_choice(s, v);
           if (fused && !s.ragged()) continue;
           if (fused)
-            e = launch_repack4(v, s.job.n_inputs, s.row_bytes, (int64_t)s.job.n_chan * s.job.n_time, s.op,
+            e = launch_repack(v, s.packed_row, s.row_bytes, (int64_t)s.job.n_chan * s.job.n_time, s.op,
                                plan->sm_count, cs);
           else if (uv == 5)
             e = launch_unpack_tile(v, s.job.sample_bits, s.job.n_inputs, s.job.n_time, s.n_tiles,

@@ -65,15 +65,18 @@ cudaError_t launch_unpack_persistent(const uint8_t *volt, int sample_bits, int n
 // 4-bit samples, any n_inputs: the streaming kernel (no shared memory) on
 // ctas / 2 CTAs of 256 threads.
 bool unpack_tile_supported(int sample_bits, int n_inputs);
-// 4-bit samples: `rows` rows of n_inputs bytes (inside a buffer that starts on a
-// 16-byte boundary) to rows of row_bytes (a multiple of 16; the bytes past
-// n_inputs are not defined).
-cudaError_t launch_repack4(const uint8_t *volt, int n_inputs, int row_bytes, int64_t rows, uint8_t *out,
-                           int sm_count, cudaStream_t s);
+// `rows` sample rows of packed_row bytes (inside a buffer that starts on a 16-byte
+// boundary) to rows of row_bytes (a multiple of 16; the bytes past packed_row are
+// not defined).
+cudaError_t launch_repack(const uint8_t *volt, int packed_row, int row_bytes, int64_t rows, uint8_t *out,
+                          int sm_count, cudaStream_t s);
+// (8-bit samples: with chan_map and n_chan_dev, device memory, only the channels
+// chan_map[0 .. *n_chan_dev) of the n_chan are unpacked)
 cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_inputs, int n_time,
                                int n_tiles, int kb, int64_t chan0, int n_chan, uint8_t *op,
                                int ctas, int32_t *status, unsigned long long timeout_ns,
-                               cudaStream_t s);
+                               cudaStream_t s, const int32_t *chan_map = nullptr,
+                               const int32_t *n_chan_dev = nullptr);
 // ---- tensor-core correlator -------------------------------------------------
 #define MWAX_MAX_JOBS 8
 
@@ -83,7 +86,8 @@ struct TcJob {
   void *out;          // visibilities of the first of these n_chan channels
   int32_t n_inputs, n_tiles, n_pairs, kb, flush_blocks, n_chan;
   int32_t n_time = 0;  // samples per integration (read by the fused pair mode)
-  int32_t row_bytes = 0;  // bytes per sample row of op (fused pair mode: a multiple of 16)
+  int32_t row_bytes = 0;   // bytes per sample row of op (fused pair mode: a multiple of 16)
+  int32_t packed_row = 0;  // bytes per sample row as it arrives (less: op holds padded copies)
   int64_t n_bl;
   // pair mode: time ranges per work item (1: whole integration; > 1: each
   // range's partial sums are added into the zeroed output with int32 atomics)
@@ -98,7 +102,7 @@ struct TcLaunch {
   int prefetch;  // K-blocks of L2 prefetch ahead of the TMA loads (0 = none; narrow only)
   int mode;      // 0: narrow (N=128 MMAs), 1: wide (N=256 with B' built in shared
                  // memory), 2: pair (two tile pairs per work item, see items), 3: fused
-                 // pair (pair mode reading packed 4-bit samples, no unpack pass)
+                 // pair (pair mode reading packed samples, no unpack pass)
   int withhold_seg;  // test hook (-1: off): see mwax_job.test_fault
   int32_t *status;
   unsigned long long timeout_ns;
@@ -122,9 +126,9 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
 // Pair mode needs every job's integration in one exact segment (kb <=
 // flush_blocks), at most 255 tiles, kb < 2^28 and 1 <= k_split <= min(kb, 8).
 bool pair_mode_supported(const TcJob *jobs, int n_jobs);
-// The fused pair mode also needs 4-bit exact samples, sample rows of whole
-// 16-byte units and sample buffers on 16-byte boundaries.
-bool fused_pair_supported(const TcJob *jobs, int n_jobs, int sample_bits, int kind);
+// The fused pair mode also needs sample rows of whole 16-byte units and sample
+// buffers on 16-byte boundaries.
+bool fused_pair_supported(const TcJob *jobs, int n_jobs);
 // The pair-mode work list of one launch over `jobs` (16 bytes per item).
 void build_pair_items(const TcJob *jobs, int n_jobs, std::vector<int4> &items);
 

@@ -86,3 +86,62 @@ def test_fused_batch_with_ragged_jobs(mw):  # noqa: F811
             chans = [0, s.n_chan // 2, s.n_chan - 1]
             assert_exact(o.cpu().numpy()[chans], oracle_for(s, chans), f"ragged batch {s.name}")
     bp.close()
+
+
+# ---- 8-bit samples in the fused pair mode (automatic above 64 MB of operands) ----------
+@pytest.mark.parametrize("N,T,C,fp16", [
+    (256, 2049, 35, False), (250, 2080, 33, False), (128, 1500, 94, True), (96, 4001, 35, True),
+    (300, 2000, 24, False), (384, 513, 90, True), (131, 2111, 33, False), (640, 1000, 27, False),
+    (255, 512, 140, False), (1000, 1400, 13, False)])
+def test_fused_8bit(mw, N, T, C, fp16):  # noqa: F811
+    """One to eight tiles, whole-unit and ragged rows (even and odd N), stage and
+    block edges, one exact segment (T = 512) and checked ones; the FP16 kind is
+    exact here too (every sum below 2^24)."""
+    spec = synth.Spec("f8", N, C, T, 8, seed=N + 3 * T + C, sigma=20, tone_amp=3.0)
+    p = mw.Plan(N, C, T, 8, kind=mw.KIND_FP16 if fp16 else mw.KIND_EXACT)
+    inf = p.info()
+    assert inf.mma_shape == 4 and inf.checked_segment == (0 if fp16 or T <= 512 else 1)
+    v = device_volt(spec)
+    out = p.correlate(v)
+    out = p.correlate(v, out)
+    assert p.status() == 0 and p.recomputed_channels() == 0
+    chans = [0, 1, C // 2, C - 1]
+    got = out.cpu().numpy()[chans]
+    assert_exact(got.astype("int64") if fp16 else got, oracle_for(spec, chans), f"fused8 {N},{T},{C},{fp16}")
+    p.close()
+
+
+@pytest.mark.parametrize("N,group", [(256, 0), (250, 31), (129, 37)])
+def test_fused_8bit_recompute(mw, N, group):  # noqa: F811
+    """Full-scale channels leave the one-segment window: the check flags them,
+    their operands are made from the rows and the narrow launch recomputes them;
+    with all channels flagged the next calls unpack and run narrow."""
+    import numpy as np
+    import oracle
+    import torch
+
+    T, C = 2200, 40
+    C = C if N > 200 else 74
+    rng = np.random.default_rng(N)
+    x = np.clip(np.rint(rng.normal(0, 20, (C, T, N, 2))), -127, 127).astype(np.int8)
+    loud = [1, 24, C - 1]
+    for c in loud:
+        x[c] = rng.choice([-127, 127], (T, N, 2)).astype(np.int8)
+    p = mw.Plan(N, C, T, 8, **({"chan_group": group} if group else {}))
+    assert p.info().mma_shape == 4
+    chans = loud + [0, 2, 23, 25, C - 2]
+    v = torch.from_numpy(x.view(np.uint8).ravel().copy()).cuda()
+    out = p.correlate(v)
+    assert p.status() == 0
+    assert p.recomputed_channels() == len(loud)
+    ref = oracle.correlate(x[chans].view(np.uint8).ravel().copy(), 8, N, len(chans), T)
+    assert_exact(out.cpu().numpy()[chans], ref, f"recompute {N}")
+    x[:] = rng.choice([-127, 127], x.shape).astype(np.int8)
+    v = torch.from_numpy(x.view(np.uint8).ravel().copy()).cuda()
+    ref = oracle.correlate(x[chans].view(np.uint8).ravel().copy(), 8, N, len(chans), T)
+    for want in (C, 0, 0):
+        out = p.correlate(v)
+        assert p.status() == 0
+        assert p.recomputed_channels() == want
+        assert_exact(out.cpu().numpy()[chans], ref, f"full scale {N}")
+    p.close()
