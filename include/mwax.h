@@ -109,10 +109,11 @@ typedef struct {
                               MWAX_ERR_UNSUPPORTED); 0 = auto: 4 (also with 8-bit samples,
                               the FP16 kind, a checked segment and any n_inputs, whose rows
                               are copied to padded ones first where they are not whole
-                              16-byte units) for 4-bit jobs of n_inputs <= 256 and where the
+                              4-byte words) for 4-bit jobs of n_inputs <= 256 and where the
                               operand tiles would exceed 64 MB and the integration has at
-                              least 8 + n_tiles^2 / 2 time blocks (rows to be copied: 16 MB
-                              at least; batch plans: where this holds for most of the
+                              least 8 + n_tiles^2 / 2 time blocks (rows that are not whole
+                              16-byte units: 16 MB at least, 8 bits at most 384 inputs unless
+                              odd; batch plans: where this holds for most of the
                               operand bytes), else 3 where it applies, else 1             */
   int32_t pipeline;        /* tuning: 1 = unpack then correlate each channel group on the
                               plan's stream, 2 = unpack the next group (second stream,
@@ -191,7 +192,7 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
 /* Plan several jobs (uneven N, C, T) that are correlated together by one
  * persistent launch per call.  On first use (and whenever the buffers
  * change) the calls are captured into two CUDA graphs: every job's unpack (in
- * the fused pair mode only the copies of rows that are not whole 16-byte units),
+ * the fused pair mode only the copies of rows that are not whole 4-byte words),
  * then the single persistent correlate launch over all jobs' work items. */
 mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
                             cudaStream_t stream);

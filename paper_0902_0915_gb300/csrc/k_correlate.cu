@@ -58,6 +58,8 @@
 #include <cudaTypedefs.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "mwax_internal.h"
 #include "mwax_nib4.h"
 
@@ -87,19 +89,22 @@ constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB
 // shared memory 1.94 (its extra reads and writes slow the MMAs), one-block
 // stages 2.2, two-block stages for items of two tiles 2.0.  8 bits, 1024 x 384 x
 // 10,000: 11.2 ms, against 3.5 of unpack and 8.55 of pair mode.
-constexpr int kModeNarrow = 0, kModeWide = 1, kModePair = 2, kModePairFused = 3;
+// 4, fused pair for sample rows that are whole 4-byte words but not 16-byte units
+// (a kernel of its own: both loaders in one spill registers, 1.86 -> 2.2 ms).
+constexpr int kModeNarrow = 0, kModeWide = 1, kModePair = 2, kModePairFused = 3, kModePairFusedWords = 4;
 constexpr int kEpiStageBytes = 32 * 128;  // pair mode: one warp's 32 rows x 16 (re, im) words
 
 template <int MODE>
 struct Shape {
-  static constexpr bool pair = MODE == kModePair || MODE == kModePairFused;
-  static constexpr int warps = MODE == kModeWide ? 12 : MODE == kModePairFused ? 18 : 10;
+  static constexpr bool fused = MODE == kModePairFused || MODE == kModePairFusedWords;
+  static constexpr bool pair = MODE == kModePair || fused;
+  static constexpr int warps = MODE == kModeWide ? 12 : fused ? 18 : 10;
   // warps 2 .. 2+conv_warps-1: B' builders (wide only)
   static constexpr int conv_warps = MODE == kModeWide ? 2 : 0;
   static constexpr int epi0 = 2 + conv_warps;  // 8 epilogue warps (fused: 16) from here to the last
   static constexpr int epi_warps = warps - epi0;
   // fused pair mode: the epilogue warps convert the samples (full-barrier arrivals per stage)
-  static constexpr int fill_arrivals = MODE == kModePairFused ? epi_warps : 1;
+  static constexpr int fill_arrivals = fused ? epi_warps : 1;
   static constexpr int kps = MODE == kModeWide ? 1 : pair ? 2 : 3;  // K blocks per stage
   static constexpr int block_bytes = (MODE == kModeNarrow ? 2 : 3) * kTileBytes;  // tiles of one block
   static constexpr int stage_bytes = kps * block_bytes;
@@ -536,39 +541,48 @@ struct Unit {
   static constexpr int per_row = tile_bytes / 16;
 };
 
+// Rows of whole 4-byte words only (WORDS, a kernel of its own): a thread takes four words instead, word
+// ct % 32 of four consecutive 128-byte pieces of the tile block (a sample row of the
+// tile at 4 bits, half of one at 8), so a warp still reads and writes 128 bytes
+// side by side and the shared-memory traffic is the same, in four times as many
+// instructions.
+//
 // One converter thread's loads of a work item: unit ct of a tile block is sample
 // ct / per_row of the block, 16 bytes at 16 (ct % per_row) of the tile's part of
 // the sample row.  Tile block k of a stage is tile k % nt of its block k / nt.
 // Samples past T and units past the row (a whole number of them) read as zero.
 constexpr int kStageTiles = 6;
-template <int BITS>
+template <int BITS, bool WORDS>
 struct RawLoads {
-  const uint8_t *base;      // the unit of tile 0, block 0 of the next stage to load
+  static constexpr int halves = WORDS && BITS != 4 ? 2 : 1;  // pieces of a sample row
+  const uint8_t *base;       // the unit of tile 0, block 0 of the next stage to load
   int64_t off[kStageTiles];  // each tile block's unit, from there
-  int lim[kStageTiles];      // samples from that unit's row on in the first stage (0: no such inputs)
-  int done, rows;            // samples of the stages loaded so far, of one stage
-  int64_t step;              // bytes of a stage's sample rows
+  // samples from that unit's row on in the first stage (0: no such inputs)
+  int lim[kStageTiles][halves];
+  int done, rows, N;         // samples of the stages loaded so far, of one stage; bytes of a row
 
   __device__ __forceinline__ int start(const PairItem &it, const KJob &jb, int k0, int ct) {
     using U = Unit<BITS>;
     int tc[3], ti[3];
     const int nt = item_tiles(it, tc, ti), kps = stage_blocks(nt, true, 0);
-    const int N = jb.row_bytes, T = jb.n_time, row = k0 * U::samples + ct / U::per_row, x = (ct % U::per_row) << 4;
+    N = jb.row_bytes;
+    const int T = jb.n_time;
+    const int row = k0 * U::samples + (WORDS ? (ct >> 5) * 4 / halves : ct / U::per_row);
+    const int x = WORDS ? (ct & 31) << 2 : (ct % U::per_row) << 4;
     base = jb.volt + ((int64_t)tc[0] * T + row) * N + ti[0] * U::tile_bytes + x;
     const int64_t d1 = (int64_t)(tc[1] - tc[0]) * T * N + (ti[1] - ti[0]) * U::tile_bytes;
     const int64_t d2 = (int64_t)(ti[2] - ti[0]) * U::tile_bytes;
-    bool in[3];
-#pragma unroll
-    for (int t = 0; t < 3; ++t) in[t] = t < nt && x < N - ti[t] * U::tile_bytes;
 #pragma unroll
     for (int k = 0; k < kStageTiles; ++k) {
       const int j = nt == 3 ? k / 3 : nt == 2 ? k / 2 : k;
       const int t = nt == 3 ? k % 3 : nt == 2 ? k % 2 : 0;
+      const int left = N - (t == 0 ? ti[0] : t == 1 ? ti[1] : ti[2]) * U::tile_bytes - x;  // bytes of the row from x on
       off[k] = (t == 0 ? 0 : t == 1 ? d1 : d2) + (int64_t)j * U::samples * N;
-      lim[k] = j < kps && (t == 0 ? in[0] : t == 1 ? in[1] : in[2]) ? T - row - U::samples * j : 0;
+#pragma unroll
+      for (int h = 0; h < halves; ++h)
+        lim[k][h] = j < kps && t < nt && left > kRowBytes * h ? T - row - U::samples * j : 0;
     }
     rows = U::samples * kps;
-    step = (int64_t)rows * N;
     done = 0;
     return nt;
   }
@@ -577,12 +591,23 @@ struct RawLoads {
 #pragma unroll
     for (int k = 0; k < kStageTiles; ++k) {
       w[k] = make_uint4(0, 0, 0, 0);
-      if (done < lim[k])
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(w[k].x), "=r"(w[k].y), "=r"(w[k].z), "=r"(w[k].w)
-                     : "l"(base + off[k]));
+      if constexpr (WORDS) {
+        const uint8_t *p = base + off[k];
+        uint32_t *v = &w[k].x;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (done + q / halves < lim[k][q % halves])
+            asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];"
+                         : "=r"(v[q])
+                         : "l"(p + (int64_t)(q / halves) * N + kRowBytes * (q % halves)));
+      } else {
+        if (done < lim[k][0])
+          asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(w[k].x), "=r"(w[k].y), "=r"(w[k].z), "=r"(w[k].w)
+                       : "l"(base + off[k]));
+      }
     }
-    base += step;
+    base += (int64_t)rows * N;
     done += rows;
   }
 };
@@ -618,6 +643,27 @@ __device__ __forceinline__ void fused_store(uint8_t *tile, int u, const uint4 &v
     }
     *reinterpret_cast<uint4 *>(half + off) = make_uint4(re[0], re[1], re[2], re[3]);
     *reinterpret_cast<uint4 *>(half + 32 * kRowBytes + off) = make_uint4(im[0], im[1], im[2], im[3]);
+  }
+}
+
+// The four words of a WORDS thread (pieces 4 (ct / 32) .. of the tile block).
+template <int BITS>
+__device__ __forceinline__ void fused_store_words(uint8_t *tile, int ct, const uint4 &v) {
+  const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+  const int l = ct & 31;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int piece = (ct >> 5) * 4 + q, t = BITS == 4 ? piece : piece >> 1;
+    const int off = t * kRowBytes + (((l >> 2) ^ (t & 7)) << 4) + ((l & 3) << 2);
+    if constexpr (BITS == 4) {
+      *reinterpret_cast<uint32_t *>(tile + off) = nib4_re(x[q]);
+      *reinterpret_cast<uint32_t *>(tile + 64 * kRowBytes + off) = nib4_im(x[q]);
+    } else {
+      uint8_t *half = tile + (q & 1) * (kTileBytes / 2);
+      const uint32_t y = x[q] ^ 0x80808080u;
+      *reinterpret_cast<uint32_t *>(half + off) = s8_halves(__byte_perm(y, 0x64646464u, 0x4240));
+      *reinterpret_cast<uint32_t *>(half + 32 * kRowBytes + off) = s8_halves(__byte_perm(y, 0x64646464u, 0x4341));
+    }
   }
 }
 
@@ -730,7 +776,7 @@ __device__ __noinline__ bool drain_item_call(const KParams &p, const PairItem &i
 // warps 2..17, also the sample converters).  Barriers as in the kernel: full[0..S)
 // empty[S..2S) tfull[3S] tempty[3S+2] drain[3S+4] (one accumulator buffer:
 // index 0 only).
-template <int BITS, int KIND, bool FUSED>
+template <int BITS, int KIND, bool FUSED, bool WORDS>
 __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, uint8_t *smem,
                                            uint32_t smem_base, uint8_t *epi_smem, uint32_t bar0,
                                            uint32_t tmem_base, volatile int *abort_flag,
@@ -899,7 +945,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
         const PairItem it = decode_pair_item(__ldg(p.items + item));
         int k0, k1;
         item_blocks(it, p.job[it.job].kb, k0, k1);
-        RawLoads<BITS> ld;
+        RawLoads<BITS, WORDS> ld;
         const int nt = ld.start(it, p.job[it.job], k0, ct), kps = stage_blocks(nt, true, 0);
         uint4 w[kStageTiles];
         ld.load(w);
@@ -912,7 +958,12 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
           const int n = nt * min(kps, k1 - kb);  // tile blocks of the stage
 #pragma unroll
           for (int k = 0; k < kStageTiles; ++k)
-            if (k < n) fused_store<BITS>(st_base + k * kTileBytes, ct, w[k]);
+            if (k < n) {
+              if constexpr (WORDS)
+                fused_store_words<BITS>(st_base + k * kTileBytes, ct, w[k]);
+              else
+                fused_store<BITS>(st_base + k * kTileBytes, ct, w[k]);
+            }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(full(stage));
@@ -936,7 +987,7 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
   using Sh = Shape<MODE>;
   constexpr bool WIDE = MODE == kModeWide;
   constexpr bool PAIR = Sh::pair;
-  constexpr bool FUSED = MODE == kModePairFused;
+  constexpr bool FUSED = Sh::fused;
   constexpr int kStageBytes = Sh::stage_bytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -988,7 +1039,7 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
   const int64_t n_items = launch_items(p);
 
   if constexpr (PAIR) {
-    pair_roles<BITS, KIND, FUSED>(maps, p, smem, smem_base, epi_smem, smem_u32(bars), tmem_base,
+    pair_roles<BITS, KIND, FUSED, MODE == kModePairFusedWords>(maps, p, smem, smem_base, epi_smem, smem_u32(bars), tmem_base,
                                   abort_flag, epi_flag, warp, lane);
   } else if (warp == 0) {
     // ---------------- TMA producer (one thread) ----------------
@@ -1329,6 +1380,25 @@ cudaError_t prepare_shape(int sample_bits, int kind, int bytes) {
 }
 
 template <int MODE>
+cudaError_t prepare_fused(int sample_bits, int kind, int bytes) {
+  return sample_bits == 4         ? set_smem_attr<4, MWAX_KIND_EXACT, MODE>(bytes)
+         : kind == MWAX_KIND_FP16 ? set_smem_attr<16, MWAX_KIND_FP16, MODE>(bytes)
+                                  : set_smem_attr<16, MWAX_KIND_EXACT, MODE>(bytes);
+}
+
+template <int MODE>
+void launch_fused(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
+                  const KParams &kp) {
+  const int threads = Shape<MODE>::warps * 32;
+  if (sample_bits == 4)
+    correlate_tc_kernel<4, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
+  else if (kind == MWAX_KIND_FP16)
+    correlate_tc_kernel<16, MWAX_KIND_FP16, MODE><<<grid, threads, smem, s>>>(maps, kp);
+  else
+    correlate_tc_kernel<16, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
+}
+
+template <int MODE>
 void launch_shape(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
                   const KParams &kp) {
   const int threads = Shape<MODE>::warps * 32;
@@ -1371,10 +1441,10 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
   const int bytes = correlate_tc_smem_bytes(stages, mode);
   if (mode == kModeWide) return prepare_shape<kModeWide>(sample_bits, kind, bytes);
   if (mode == kModePair) return prepare_shape<kModePair>(sample_bits, kind, bytes);
-  if (mode == kModePairFused)
-    return sample_bits == 4          ? set_smem_attr<4, MWAX_KIND_EXACT, kModePairFused>(bytes)
-           : kind == MWAX_KIND_FP16 ? set_smem_attr<16, MWAX_KIND_FP16, kModePairFused>(bytes)
-                                    : set_smem_attr<16, MWAX_KIND_EXACT, kModePairFused>(bytes);
+  if (mode == kModePairFused) {
+    const cudaError_t e = prepare_fused<kModePairFused>(sample_bits, kind, bytes);
+    return e != cudaSuccess ? e : prepare_fused<kModePairFusedWords>(sample_bits, kind, bytes);
+  }
   return prepare_shape<kModeNarrow>(sample_bits, kind, bytes);
 }
 
@@ -1396,8 +1466,8 @@ bool pair_mode_supported(const TcJob *jobs, int n_jobs) {
 
 bool fused_pair_supported(const TcJob *jobs, int n_jobs) {
   for (int j = 0; j < n_jobs; ++j)
-    if (jobs[j].row_bytes % 16 != 0 || jobs[j].row_bytes < jobs[j].packed_row || jobs[j].n_time < 1 ||
-        (jobs[j].op && (reinterpret_cast<uintptr_t>(jobs[j].op) & 15u) != 0))
+    if (jobs[j].row_bytes % 4 != 0 || jobs[j].row_bytes < jobs[j].packed_row || jobs[j].n_time < 1 ||
+        (jobs[j].op && reinterpret_cast<uintptr_t>(jobs[j].op) % (jobs[j].row_bytes % 16 == 0 ? 16 : 4) != 0))
       return false;
   return true;
 }
@@ -1486,10 +1556,12 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
   memset(&maps, 0, sizeof(maps));
   memset(&kp, 0, sizeof(kp));
   int64_t items = 0;
+  bool words = false;  // fused pair mode: some job's rows are not whole 16-byte units
   for (int j = 0; j < n_jobs; ++j) {
     const TcJob &job = jobs[j];
     if (job.flush_blocks < 1 || job.kb < 1 || job.n_tiles < 1) return cudaErrorInvalidValue;
     if (fused && !job.op) return cudaErrorInvalidValue;
+    words = words || job.row_bytes % 16 != 0;
     KJob &kj = kp.job[j];
     kj.out = job.out;
     kj.item_begin = items;
@@ -1540,15 +1612,10 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
     launch_shape<kModeWide>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
   else if (cfg.mode == kModePair)
     launch_shape<kModePair>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else if (fused) {
-    constexpr int threads = Shape<kModePairFused>::warps * 32;
-    if (cfg.sample_bits == 4)
-      correlate_tc_kernel<4, MWAX_KIND_EXACT, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
-    else if (cfg.kind == MWAX_KIND_FP16)
-      correlate_tc_kernel<16, MWAX_KIND_FP16, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
-    else
-      correlate_tc_kernel<16, MWAX_KIND_EXACT, kModePairFused><<<grid, threads, smem, s>>>(maps, kp);
-  }
+  else if (fused && words)
+    launch_fused<kModePairFusedWords>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
+  else if (fused)
+    launch_fused<kModePairFused>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
   else
     launch_shape<kModeNarrow>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
   return cudaGetLastError();

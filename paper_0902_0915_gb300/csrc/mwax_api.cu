@@ -34,8 +34,9 @@ struct JobState {
   int64_t op_chan_bytes = 0;  // operand bytes of one channel
   int64_t in_chan_bytes = 0;  // packed input bytes of one channel
   int64_t out_chan_bytes = 0;
-  // a sample row as it arrives and in whole 16-byte units (more: the fused pair
-  // mode reads rows copied to that length)
+  // a sample row as it arrives, and, where that is not whole 4-byte words (batch
+  // plans: not whole 16-byte units), in whole 16-byte units: the fused pair mode
+  // reads rows copied to that length
   int packed_row = 0, row_bytes = 0;
   uint8_t *op = nullptr;  // batch plans: operand buffer (fused: padded rows) for all channels of this job
   bool ragged() const { return row_bytes != packed_row; }
@@ -187,7 +188,7 @@ void derive(JobState &s) {
   s.in_chan_bytes = (int64_t)j.n_time * j.n_inputs * bytes_per_sample(j.sample_bits);
   s.out_chan_bytes = s.n_bl * 8;
   s.packed_row = j.n_inputs * bytes_per_sample(j.sample_bits);
-  s.row_bytes = (s.packed_row + 15) / 16 * 16;
+  s.row_bytes = s.packed_row % 4 == 0 ? s.packed_row : (s.packed_row + 15) / 16 * 16;
   int64_t g = j.chan_group > 0 ? j.chan_group : kDefaultScratchBudget / s.op_chan_bytes;
   s.chan_group = (int)std::max<int64_t>(1, std::min<int64_t>(g, j.n_chan));
 }
@@ -289,15 +290,20 @@ int resolve_split(const mwax_job &job, int mode, int kb, int64_t base_items, int
 constexpr int kFusedTiles = 2;
 constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
 
-// Rows that are not whole 16-byte units are copied to padded ones first (2 bytes
-// of traffic per sample, against 3 for the unpack and operands twice as wide);
-// the extra launch needs operands of 16 MB to pay.
+// Rows that are not whole 4-byte words are copied to padded ones first (twice the
+// sample bytes of traffic, against three times for the unpack and operands twice as
+// wide); the extra launch needs operands of 16 MB to pay, and rows of words take
+// the same line.  8-bit rows of words leave the fused mode above three tiles, where
+// their four-byte stores cost more than the unpack (in microseconds, fused / unpack
+// + pair: 250 x 384 x 4001 484 / 748, 334 x 128 x 3000 313 / 370, 500 x 64 x 4000 423 /
+// 409, 998 x 64 x 4000 1154 / 939; odd N, copied: 999 x 64 x 4000 986 / 1192).
 constexpr int64_t kRaggedOperandBytes = int64_t(16) << 20;
 
 int64_t operand_bytes(const TcJob &j) { return (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes; }
 
 bool fused_pays(const TcJob &j, int sample_bits) {
-  if (j.row_bytes != j.packed_row && operand_bytes(j) <= kRaggedOperandBytes) return false;
+  if (j.packed_row % 16 != 0 && operand_bytes(j) <= kRaggedOperandBytes) return false;
+  if (sample_bits == 8 && j.packed_row % 16 != 0 && j.packed_row % 4 == 0 && j.n_tiles > 3) return false;
   if (sample_bits == 4 && j.n_tiles <= kFusedTiles) return true;
   return operand_bytes(j) > kFusedOperandBytes && j.kb >= 8 + j.n_tiles * j.n_tiles / 2;
 }
@@ -313,7 +319,7 @@ int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int 
   bool whole = true;
   int64_t all = 0, pays = 0;
   for (const TcJob &j : tj) {
-    whole = whole && j.row_bytes == j.packed_row && sample_bits == 4;
+    whole = whole && j.packed_row % 16 == 0 && sample_bits == 4;
     all += operand_bytes(j);
     if (fused_pays(j, sample_bits)) pays += operand_bytes(j);
   }
@@ -428,7 +434,7 @@ cudaError_t checked_call_done(mwax_plan_s *p, cudaStream_t st) {
 }
 
 // Fused checked plans: the operands of nc channels (or of the listed ones) from
-// sample rows of whole 16-byte units; inputs past N only make operand rows whose
+// sample rows of whole words; inputs past N only make operand rows whose
 // products are never stored.
 cudaError_t unpack_rows(mwax_plan_s *p, const JobState &s, const uint8_t *rows, int nc, cudaStream_t st,
                         const int32_t *chan_map, const int32_t *n_chan_dev) {
@@ -794,6 +800,8 @@ mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
     JobState s;
     s.job = jobs[k];
     derive(s);
+    // one kernel for all jobs: that of whole 16-byte units
+    s.row_bytes = (s.packed_row + 15) / 16 * 16;
     p->jobs.push_back(s);
   }
   std::vector<TcJob> tj;

@@ -86,7 +86,7 @@ struct TcJob {
   void *out;          // visibilities of the first of these n_chan channels
   int32_t n_inputs, n_tiles, n_pairs, kb, flush_blocks, n_chan;
   int32_t n_time = 0;  // samples per integration (read by the fused pair mode)
-  int32_t row_bytes = 0;   // bytes per sample row of op (fused pair mode: a multiple of 16)
+  int32_t row_bytes = 0;   // bytes per sample row of op (fused pair mode: a multiple of 4)
   int32_t packed_row = 0;  // bytes per sample row as it arrives (less: op holds padded copies)
   int64_t n_bl;
   // pair mode: time ranges per work item (1: whole integration; > 1: each
@@ -126,8 +126,8 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
 // Pair mode needs every job's integration in one exact segment (kb <=
 // flush_blocks), at most 255 tiles, kb < 2^28 and 1 <= k_split <= min(kb, 8).
 bool pair_mode_supported(const TcJob *jobs, int n_jobs);
-// The fused pair mode also needs sample rows of whole 16-byte units and sample
-// buffers on 16-byte boundaries.
+// The fused pair mode also needs sample rows of whole 4-byte words, and sample
+// buffers on 16-byte boundaries where they are whole 16-byte units.
 bool fused_pair_supported(const TcJob *jobs, int n_jobs);
 // The pair-mode work list of one launch over `jobs` (16 bytes per item).
 void build_pair_items(const TcJob *jobs, int n_jobs, std::vector<int4> &items);
