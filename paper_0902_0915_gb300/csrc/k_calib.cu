@@ -40,7 +40,9 @@ namespace {
 
 constexpr int kCT = 32;        // inputs per calibration tile side
 constexpr int kCalThreads = 256;
-constexpr int kCalibCtas = 3;  // of the loss/adjoint pass, per SM
+constexpr int kCalibCtas = 3;      // of the loss/adjoint pass, per SM (4: 1017 against 1003 us at 1024 x 768)
+constexpr int kCalibChanCtas = 4;  // of the per-channel pass, whose warps wait for one channel's loads
+                                   // (3: 874 against 826 us for 10 sweeps of 256 x 768)
 constexpr int kMaxChanGroups = 12;
 
 struct Kahan {
@@ -185,20 +187,23 @@ __device__ __forceinline__ int tile_row_of_lane(int lane) {
 // (nu = cg + n_cg (w + 8k)), each channel with tile_channel, and adds the
 // channel's sums into Kahan accumulators (one compensated add per channel;
 // the 32-term sums inside a channel are plain FP32).  The eight warps' totals
-// are then summed in a fixed order.  DEN: also the per-row and per-column
+// are then summed in a fixed order.  back: the groups in descending order (a
+// solve's every other sweep, so that it starts with what the last one left in
+// L2).  DEN: also the per-row and per-column
 // sums of |g_other|^2 |M|^2 (the gain solve's normal-equation weight; sums of
 // positive terms, plain FP32).
 template <bool DEN>
 __global__ void __launch_bounds__(kCalThreads, kCalibCtas) calib_tile_kernel(
     const float2 *__restrict__ V, const float2 *__restrict__ M, const float2 *__restrict__ g,
     int N, int C, int n_cg, float *__restrict__ part_loss, float2 *__restrict__ part_row,
-    float2 *__restrict__ part_col, float *__restrict__ part_rden, float *__restrict__ part_cden) {
+    float2 *__restrict__ part_col, float *__restrict__ part_rden, float *__restrict__ part_cden,
+    bool back) {
   constexpr int kWarps = kCalThreads / 32;
   __shared__ float2 sgi[kCT];
   __shared__ float2 srow[kWarps][kCT], scol[kWarps][kCT];
   __shared__ float srden[kWarps][kCT], scden[kWarps][kCT];
   __shared__ float sloss[kWarps];
-  const int tile = blockIdx.x, cg = blockIdx.y;
+  const int tile = blockIdx.x, cg = back ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
   int I, J;
   tile_of(tile, I, J);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -214,7 +219,7 @@ __global__ void __launch_bounds__(kCalThreads, kCalibCtas) calib_tile_kernel(
   float rden = 0.f, cden = 0.f;
   for (int nu = cg + n_cg * w; nu < C; nu += n_cg * kWarps) {
     const TileSums t = tile_channel<DEN>(V + (int64_t)nu * B, M + (int64_t)nu * B, sgi, gj, I, j,
-                                         N, lane);
+                                               N, lane);
     loss.add(t.loss);
     rre.add(t.rre);
     rim.add(t.rim);
@@ -406,17 +411,19 @@ __global__ void __launch_bounds__(kGatherThreads) calib_gather_kernel(
 // part_row / part_col [tile][C][32], DEN: part_rden / part_cden likewise;
 // part_loss [tile][gridDim.y] (the CTA's eight channels).
 template <bool DEN>
-__global__ void __launch_bounds__(kCalThreads, 3) calib_chan_tile_kernel(
+__global__ void __launch_bounds__(kCalThreads, kCalibChanCtas) calib_chan_tile_kernel(
     const float2 *__restrict__ V, const float2 *__restrict__ M, const float2 *__restrict__ g,
     int N, int C, float *__restrict__ part_loss, float2 *__restrict__ part_row,
-    float2 *__restrict__ part_col, float *__restrict__ part_rden, float *__restrict__ part_cden) {
+    float2 *__restrict__ part_col, float *__restrict__ part_rden, float *__restrict__ part_cden,
+    bool back) {
   __shared__ float2 sgi[kCalThreads / 32][kCT];
   __shared__ float sloss[kCalThreads / 32];
   const int tile = blockIdx.x;
   int I, J;
   tile_of(tile, I, J);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int nu = blockIdx.y * (kCalThreads / 32) + w;
+  const int cy = back ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
+  const int nu = cy * (kCalThreads / 32) + w;
   float lsum = 0.f;
   if (nu < C) {
     const int64_t B = (int64_t)N * (N + 1) / 2;
@@ -426,7 +433,7 @@ __global__ void __launch_bounds__(kCalThreads, 3) calib_chan_tile_kernel(
     sgi[w][lane] = il < N ? gn[il] : make_float2(0.f, 0.f);
     __syncwarp();
     const TileSums t = tile_channel<DEN>(V + (int64_t)nu * B, M + (int64_t)nu * B, sgi[w], gj, I,
-                                         j, N, lane);
+                                               j, N, lane);
     const int64_t base = ((int64_t)tile * C + nu) * kCT;
     const int row = tile_row_of_lane(lane);
     part_row[base + row] = make_float2(t.rre, t.rim);
@@ -444,7 +451,7 @@ __global__ void __launch_bounds__(kCalThreads, 3) calib_chan_tile_kernel(
   if (threadIdx.x == 0) {
     float t = 0.f;
     for (int k = 0; k < kCalThreads / 32; ++k) t += sloss[k];
-    part_loss[(int64_t)tile * gridDim.y + blockIdx.y] = t;
+    part_loss[(int64_t)tile * gridDim.y + cy] = t;
   }
 }
 
@@ -584,19 +591,19 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 // entries of the block in that row).  Of the two rows of the triangle one
 // starts the block on a 16-byte boundary (one 16-byte copy), the other on an
 // 8-byte one (two 8-byte copies); the alignment is the same for every lane of
-// the warp.
-__device__ __forceinline__ void jones_load_row(float4 *slot, const float2 *Vn, const float2 *Mn,
-                                               int a, int b) {
-  const int64_t i0 = 2 * (int64_t)a, i1 = i0 + 1;
-  const int64_t o0 = i0 * (i0 + 1) / 2 + 2 * b, o1 = i1 * (i1 + 1) / 2 + 2 * b;
-  const float2 *src[4] = {Vn + o0, Vn + o1, Mn + o0, Mn + o1};
+// the warp.  v0: the block's entries in row 2a of V; row 2a + 1 is `next` bytes
+// on, M is `to_m` bytes from V.
+__device__ __forceinline__ void jones_load_row(float4 *slot, const char *v0, uint32_t next,
+                                               int64_t to_m) {
+  const char *v1 = v0 + next;
+  const char *src[4] = {v0, v1, v0 + to_m, v1 + to_m};
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    if ((reinterpret_cast<uintptr_t>(src[e]) & 15u) == 0) {
+    if (((uint32_t)reinterpret_cast<uintptr_t>(src[e]) & 15u) == 0) {
       cp_async16(slot + e * 32, src[e]);
     } else {
       cp_async8(reinterpret_cast<float2 *>(slot + e * 32), src[e]);
-      cp_async8(reinterpret_cast<float2 *>(slot + e * 32) + 1, src[e] + 1);
+      cp_async8(reinterpret_cast<float2 *>(slot + e * 32) + 1, src[e] + 8);
     }
   }
 }
@@ -670,6 +677,10 @@ __device__ __forceinline__ float jones_row(const float4 *slot, float2 ja00, floa
 // and the warp reduce-scatters them once per row pair; each row pair's loss
 // goes into a Kahan accumulator; the eight warps' partials are summed in a
 // fixed order.
+// Bound by instruction issue (70 % of the slots; scalar multiply-adds alone reach
+// 86 % here): the rows' pointers go on by a channel step instead of being formed
+// for every row and channel, 432 -> 390 us a sweep of 1024 inputs x 256 channels.
+// back: the groups in descending order (see calib_tile_kernel).
 // Outputs per (tile, cg): part_row [32 rows][12], part_col [32 columns][12],
 // part_loss.  DEN: the D quantities (left at 0 otherwise).
 #ifndef MWAX_JONES_PAIRS
@@ -683,7 +694,7 @@ template <bool DEN>
 __global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_kernel(
     const float2 *__restrict__ V, const float2 *__restrict__ M, const float2 *__restrict__ Jm,
     int n_tiles, int C, int n_cg, float *__restrict__ part_loss, float *__restrict__ part_row,
-    float *__restrict__ part_col) {
+    float *__restrict__ part_col, bool back) {
   constexpr int kWarps = kCalThreads / 32;
   extern __shared__ __align__(16) float4 sdyn[];
   // ring [warp][pair slot][row 0/1][4 entries][lane]; afterwards the same memory
@@ -692,7 +703,7 @@ __global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_ker
   float2 *sJ = reinterpret_cast<float2 *>(sdyn + kWarps * kJPairs * 2 * 4 * 32);  // [32 rows][4]
   static_assert(sizeof(float) * (kWarps * kJT * kJQ + kWarps) <= sizeof(float4) * kWarps * kJPairs * 2 * 4 * 32,
                 "aliasing");
-  const int tile = blockIdx.x, cg = blockIdx.y;
+  const int tile = blockIdx.x, cg = back ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
   int I, Jt;
   tile_of(tile, I, Jt);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -712,35 +723,51 @@ __global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_ker
   const int64_t N = 2 * (int64_t)n_tiles, Bn = N * (N + 1) / 2;
   const int first = cg + n_cg * w, stride = n_cg * kWarps;
   const int n_mine = first < C ? (C - 1 - first) / stride + 1 : 0;
-  // pair p = q n_mine + k: row pair q (rows 8 (q >> 2) + (q & 3) + {0, 4}) of
-  // the warp's k-th channel; row pairs outer, channels inner, so each lane
-  // sums a row pair's tile-a quantities over its channels before the one
-  // reduce-scatter of the row pair
-  const int n_pairs = n_mine * (kJT / 2);
+  // row pairs (rows 8 (q >> 2) + (q & 3) + {0, 4}) outer, the warp's channels
+  // inner, so each lane sums a row pair's tile-a quantities over its channels
+  // before the one reduce-scatter of the row pair.  The next pair to issue: its
+  // row pair iq, its channel's number ik, and where its rows' blocks lie (the
+  // pointers go on by a channel step; a new row pair sets them)
   float4 *ring = ringbase + (int64_t)w * kJPairs * 2 * 4 * 32 + lane;
-  int iq = 0, ik = 0;  // row pair and channel of the next pair to issue
-  auto issue = [&](int p) {
-    if (p < n_pairs) {
-      const int nu = first + stride * ik;
-      const float2 *Vn = V + (int64_t)nu * Bn, *Mn = M + (int64_t)nu * Bn;
+  int iq = 0, ik = 0, islot = 0;
+  const char *v0[2];
+  uint32_t next[2];
+  bool has[2];
+  const int64_t step = (int64_t)stride * Bn * sizeof(float2);
+  const int64_t to_m = reinterpret_cast<const char *>(M) - reinterpret_cast<const char *>(V);
+  auto set_rows = [&] {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int a = I * kJT + 8 * (iq >> 2) + (iq & 3) + 4 * h;
+      const int64_t i0 = 2 * (int64_t)a;
+      v0[h] = reinterpret_cast<const char *>(V + (int64_t)first * Bn + i0 * (i0 + 1) / 2 + 2 * b);
+      next[h] = (uint32_t)((i0 + 1) * sizeof(float2));
+      has[h] = a < n_tiles && b < a;
+    }
+  };
+  auto issue = [&] {
+    if (iq < kJT / 2) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        float4 *slot = ring + ((p % kJPairs) * 2 + h) * 4 * 32;
-        const int a = I * kJT + 8 * (iq >> 2) + (iq & 3) + 4 * h;
-        if (a < n_tiles && b < a) {
-          jones_load_row(slot, Vn, Mn, a, b);
+        float4 *slot = ring + (islot * 2 + h) * 4 * 32;
+        if (has[h]) {
+          jones_load_row(slot, v0[h], next[h], to_m);
         } else {
 #pragma unroll
           for (int e = 0; e < 4; ++e) slot[e * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        v0[h] += step;
       }
       if (++ik == n_mine) {
         ik = 0;
         ++iq;
+        set_rows();
       }
     }
+    islot = islot + 1 == kJPairs ? 0 : islot + 1;
     cp_async_commit();
   };
+  set_rows();
   float col[kJQ];
   float row[4][3];
 #pragma unroll
@@ -748,29 +775,30 @@ __global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_ker
 #pragma unroll
   for (int m = 0; m < 4; ++m) row[m][0] = row[m][1] = row[m][2] = 0.f;
   Kahan loss;
+  if (n_mine == 0) iq = kJT / 2;  // nothing to issue
 #pragma unroll
-  for (int k = 0; k < kJPairs - 1; ++k) issue(k);
+  for (int k = 0; k < kJPairs - 1; ++k) issue();
+  int cslot = 0;  // ring slot of the pair in hand
 #pragma unroll
   for (int m = 0; m < 4; ++m)
 #pragma unroll 1
     for (int u = 0; u < 4; ++u) {
-      const int q = 4 * m + u;
       float v[2 * kJQ];
 #pragma unroll
       for (int k = 0; k < 2 * kJQ; ++k) v[k] = 0.f;
       float lq = 0.f;
 #pragma unroll 1
       for (int kc = 0; kc < n_mine; ++kc) {
-        const int p = q * n_mine + kc;
-        issue(p + kJPairs - 1);
-        cp_async_wait<kJPairs - 1>();  // this thread's copies of pair p have landed
+        issue();
+        cp_async_wait<kJPairs - 1>();  // this thread's copies of the pair have landed
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int r = 8 * m + u + 4 * h;
-          const float4 *slot = ring + ((p % kJPairs) * 2 + h) * 4 * 32;
+          const float4 *slot = ring + (cslot * 2 + h) * 4 * 32;
           lq += jones_row<DEN>(slot, sJ[4 * r + 0], sJ[4 * r + 1], sJ[4 * r + 2], sJ[4 * r + 3],
                                jb00, jb01, jb10, jb11, col, v + kJQ * h);
         }
+        cslot = cslot + 1 == kJPairs ? 0 : cslot + 1;
       }
       reduce_scatter24(v, lane);
       if ((lane & 3) == u) {
@@ -1022,7 +1050,7 @@ mwax_status mwax_calib_loss_grad(const float *V, const float *M, const float *g,
   calib_tile_kernel<false><<<dim3(tiles, n_cg), kCalThreads, 0, stream>>>(
       reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M),
       reinterpret_cast<const float2 *>(g), n_inputs, n_chan, n_cg, w.loss, w.row, w.col, nullptr,
-      nullptr);
+      nullptr, false);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return MWAX_ERR_CUDA;
   calib_gather_kernel<false><<<nb + 1, kGatherThreads, 0, stream>>>(
@@ -1055,7 +1083,7 @@ mwax_status mwax_calib_solve(const float *V, const float *M, float *g, int n_inp
   for (int t = 1; t <= n_iter; ++t) {
     calib_tile_kernel<true><<<dim3(tiles, n_cg), kCalThreads, 0, stream>>>(
         reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M), g2, n_inputs,
-        n_chan, n_cg, w.loss, w.row, w.col, w.rden, w.cden);
+        n_chan, n_cg, w.loss, w.row, w.col, w.rden, w.cden, t % 2 == 0);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
     calib_gather_kernel<true><<<nb + 1, kGatherThreads, 0, stream>>>(
         n_inputs, nb, n_cg, w.loss, w.row, w.col, w.rden, w.cden,
@@ -1088,7 +1116,7 @@ mwax_status mwax_calib_chan_loss_grad(const float *V, const float *M, const floa
   calib_chan_tile_kernel<false><<<dim3(tiles, n_cy), kCalThreads, 0, stream>>>(
       reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M),
       reinterpret_cast<const float2 *>(g), n_inputs, n_chan, w.loss, w.row, w.col, nullptr,
-      nullptr);
+      nullptr, false);
   if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
   calib_chan_gather_kernel<false><<<dim3(nb + 1, n_cy), kCalThreads, 0, stream>>>(
       n_inputs, n_chan, nb, w.loss, w.row, w.col, nullptr, nullptr, loss,
@@ -1111,7 +1139,7 @@ mwax_status mwax_calib_chan_solve(const float *V, const float *M, float *g, int 
   for (int t = 1; t <= n_iter; ++t) {
     calib_chan_tile_kernel<true><<<dim3(tiles, n_cy), kCalThreads, 0, stream>>>(
         reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M), g2, n_inputs,
-        n_chan, w.loss, w.row, w.col, w.rden, w.cden);
+        n_chan, w.loss, w.row, w.col, w.rden, w.cden, t % 2 == 0);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
     calib_chan_gather_kernel<true><<<dim3(nb + 1, n_cy), kCalThreads, 0, stream>>>(
         n_inputs, n_chan, nb, w.loss, w.row, w.col, w.rden, w.cden,
@@ -1146,23 +1174,23 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
       cudaFuncSetAttribute(calib_jones_tile2_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            smem2) != cudaSuccess)
     return MWAX_ERR_CUDA;
-  auto tile_pass = [&](bool den) {
+  auto tile_pass = [&](bool den, bool back) {
     if (den)
       calib_jones_tile2_kernel<true><<<dim3(tiles, n_cg), kCalThreads, smem2, stream>>>(
-          V2, M2, J2, n_tiles, n_chan, n_cg, ploss, prow, pcol);
+          V2, M2, J2, n_tiles, n_chan, n_cg, ploss, prow, pcol, back);
     else
       calib_jones_tile2_kernel<false><<<dim3(tiles, n_cg), kCalThreads, smem2, stream>>>(
-          V2, M2, J2, n_tiles, n_chan, n_cg, ploss, prow, pcol);
+          V2, M2, J2, n_tiles, n_chan, n_cg, ploss, prow, pcol, back);
   };
   if (!solve) {
-    tile_pass(false);
+    tile_pass(false, false);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
     calib_jones_gather_kernel<false><<<dim3(n_jt + 1, kJT / 2), kJGatherWarps * 32, 0, stream>>>(
         n_tiles, n_jt, n_cg, ploss, prow, pcol, loss, reinterpret_cast<float2 *>(grad), nullptr, 0);
     return cudaGetLastError() == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
   }
   for (int t = 1; t <= n_iter; ++t) {
-    tile_pass(true);
+    tile_pass(true, t % 2 == 0);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
     calib_jones_gather_kernel<true><<<dim3(n_jt + 1, kJT / 2), kJGatherWarps * 32, 0, stream>>>(
         n_tiles, n_jt, n_cg, ploss, prow, pcol, loss ? loss + (t - 1) : nullptr, nullptr, J2,
