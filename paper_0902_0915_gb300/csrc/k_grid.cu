@@ -26,16 +26,18 @@
 //      band up to W = 7); a (point, band) whose cells reach the half plane is
 //      an entry.  Positions and support bounds are FP64, so the support sets
 //      match an FP64 definition exactly;
-//   2. counting sort of the entries by bin = the band's first cell (integer atomics for counts and slots, an exclusive
-//      prefix sum for bin offsets), then every bin's entries sorted ascending
-//      so the order of each gathered sum is fixed;
+//   2. counting sort of the entries by bin = the band's first cell (integer
+//      atomics for counts and slots, an exclusive prefix sum for bin offsets),
+//      then every bin's entries sorted ascending so the order of each gathered
+//      sum is fixed;
 //   3. the weights: the Gaussian is separable, w = wx(s - x) wy(r - y), and the
 //      support a rectangle, so an entry stores its W column and up to 7 row
 //      factors (computed in FP64, kept in FP32, 0 outside the support) and its
 //      first column: 64 bytes up to W = 7;
 //   4. the units of work: a strip of 4 columns by 32 rows (fewer on small
 //      grids) is one warp's; strips that hold more entries than a quarter of a
-//      warp's even share (the centre of the uv plane) take a CTA of 4 warps.
+//      warp's even share (the centre of the uv plane) take a CTA of 4 warps,
+//      sparse ones are joined to strips of 32 columns by 16 rows.
 // Grid call (per integration): one kernel gathers the four polarisation values
 // of every baseline and channel from the int32 correlator output into its
 // entries; then each warp walks its strip row of bins by row of bins.  The
@@ -49,6 +51,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "mwax_internal.h"
@@ -260,18 +263,29 @@ __global__ void __launch_bounds__(256) grid_weights_kernel(GridGeom g,
 // is complete after it.
 constexpr int kCols = 4;
 constexpr int kUnitRows = 32;
+// Wide units: 32 columns, one entry a step, no sums across groups: a bin row costs
+// its steps alone, while each of eight narrow strips pays about 100 instructions
+// for it.  But the steps follow one another, so only strips of few entries (96 per
+// 32 rows) are joined, and the longest are handed out first.  Measured a call, up
+// to 400 entries in any order / up to 96, longest first: 69 tiles x 21 channels on
+// 1466^2 cells, W = 7: 55 / 38 us (narrow strips alone: 63); 17 x 328 on 1420^2,
+// W = 6: 63 / 34; 100 x 200 on 2000^2, W = 5: 206 / 183; 128 x 768 on 2048^2,
+// W = 7, of which little is sparse: 548 / 541.
+constexpr int kWideCols = 32, kWideRows = 16, kWideEntries = 96;
+constexpr int kWideFlag = 1 << 30;
 constexpr int kMaxBinRows = 40;  // >= kUnitRows + 6
 
-// entries of every unit of `rows` rows (unit = row segment * n_cb + column block)
+// entries of every unit of `rows` rows and `cols` columns (unit = row segment * n_cb +
+// column block)
 __global__ void __launch_bounds__(256) grid_unit_count_kernel(const int *__restrict__ offsets,
                                                               int n_units, int n_cb, int rows,
-                                                              int n_rows, int W, int off, int nbw,
-                                                              int *__restrict__ cnt) {
+                                                              int n_rows, int cols, int W, int off,
+                                                              int nbw, int *__restrict__ cnt) {
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= n_units) return;
-  const int r0 = (u / n_cb) * rows, s0 = (u % n_cb) * kCols;
+  const int r0 = (u / n_cb) * rows, s0 = (u % n_cb) * cols;
   const int nb = min(rows, n_rows - r0) + off;
-  const int c1 = min(s0 + kCols + W - 1, nbw);
+  const int c1 = min(s0 + cols + W - 1, nbw);
   int n = 0;
   for (int i = 0; i < nb; ++i) n += offsets[(r0 + i) * nbw + c1] - offsets[(r0 + i) * nbw + s0];
   cnt[u] = n;
@@ -317,8 +331,8 @@ __global__ void __launch_bounds__(256) grid_values_kernel(const int2 *__restrict
 
 // Grid call, step 2.
 // Staging: a ring of kSlots chunks of 32 entries per warp (values, factors).
-// Every bin row starts on a multiple of 8 entries; the places left over are
-// zeros.  One step is 8 entries, one per group.
+// Every bin row starts on a multiple of G entries; the places left over are
+// zeros.  One step is G entries, one per group of 32 / G lanes.
 constexpr int kSlots = 2;
 constexpr int kChunk = 32, kRing = kSlots * kChunk;
 constexpr int kApplyWarps = 4;
@@ -330,7 +344,7 @@ struct ApplyArgs {
   const int *offsets;
   const float4 *wts, *vals;
   float *grids;
-  const int2 *units;  // x = column block, y = first relative row << 8 | rows
+  const int2 *units;  // x = column block (| kWideFlag), y = first relative row << 8 | rows
   int *next;          // light units handed out so far
   int Ng, W, nbw, f4;  // f4: 16-byte pieces per entry's factors
   int n_heavy, n_light;
@@ -341,17 +355,47 @@ struct BinRows {
   int q[kMaxBinRows], n[kMaxBinRows], s[kMaxBinRows + 4];
 };
 
-// One component (2 (2p + q) + (re, im)) of relative row r, column s: stored at
-// its cell, and mirrored (conj, p and q swapped) unless the row is its own
-// mirror image.
-__device__ __forceinline__ void store_value(const ApplyArgs &A, int r, int s, int comp, float v) {
-  const int Ng = A.Ng, row = Ng / 2 + r, pol = comp >> 1, ri = comp & 1;
-  if (row < Ng && s < Ng) A.grids[(((int64_t)pol * Ng + row) * Ng + s) * 2 + ri] = v;
-  if (r > 0 && s >= 1 && s <= Ng) {
-    const int mp = ((pol & 1) << 1) | (pol >> 1);
-    A.grids[(((int64_t)mp * Ng + (Ng - row)) * Ng + (Ng - s)) * 2 + ri] = ri ? -v : v;
+// Where a lane's values of a unit's rows go, row by row: their cells, and mirrored
+// (conj, p and q swapped) ones unless the row is its own mirror image.  comp = 2
+// (2p + q) + (re, im).
+struct RowOut {
+  float *cell, *mirror;  // of the next row, component comp
+  int r, half, step;     // its relative row; Ng / 2; floats per grid row
+  bool in, min;          // the column has a cell, a mirrored cell
+
+  __device__ __forceinline__ RowOut(const ApplyArgs &A, int r0, int s, int comp) {
+    const int Ng = A.Ng, pol = comp >> 1, ri = comp & 1, mp = ((pol & 1) << 1) | (pol >> 1);
+    r = r0;
+    half = Ng / 2;
+    step = 2 * Ng;
+    in = s < Ng;
+    min = s >= 1 && s <= Ng;
+    cell = A.grids + (((int64_t)pol * Ng + half + r0) * Ng + s) * 2 + ri;
+    mirror = A.grids + (((int64_t)mp * Ng + half - r0) * Ng + (Ng - s)) * 2 + ri;
   }
-}
+  __device__ __forceinline__ void advance() {
+    cell += step;
+    mirror -= step;
+    ++r;
+  }
+  // narrow units: one component (ri: it is an imaginary part)
+  __device__ __forceinline__ void put(float v, bool ri) {
+    if (in && r < half) *cell = v;
+    if (min && r > 0) *mirror = ri ? -v : v;
+    advance();
+  }
+  // wide units (comp = 0): all four products
+  __device__ __forceinline__ void put(const float (&a)[8]) {
+    const int64_t plane = (int64_t)step * (step / 2);  // floats of a product's grid
+#pragma unroll
+    for (int pol = 0; pol < 4; ++pol) {
+      const int mp = ((pol & 1) << 1) | (pol >> 1);
+      if (in && r < half) *reinterpret_cast<float2 *>(cell + pol * plane) = make_float2(a[2 * pol], a[2 * pol + 1]);
+      if (min && r > 0) *reinterpret_cast<float2 *>(mirror + mp * plane) = make_float2(a[2 * pol], -a[2 * pol + 1]);
+    }
+    advance();
+  }
+};
 
 __device__ __forceinline__ float4 lds4(uint32_t a) {
   float4 v;
@@ -369,27 +413,29 @@ __device__ __forceinline__ void cp16z(uint32_t dst, const void *src, bool take) 
                : "memory");
 }
 
-// One warp's walk over a unit of n_bins bin rows.  emit(i, v): after bin row i
-// the lane holds the finished value of row i - off, column lane & 3, component
-// lane >> 2 = 2 (2p + q) + (re, im).
-template <int WN, int F4, class Emit>
+// One warp's walk over a unit of n_bins bin rows.  emit(i, a): after bin row i
+// the lane holds finished values of row i - off; G = 8 (narrow): column lane & 3,
+// component lane >> 2 = 2 (2p + q) + (re, im) in a[0]; G = 1 (wide): column lane,
+// all eight components.
+template <int WN, int F4, int G, class Emit>
 __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bins, uint8_t *sm,
                                            const BinRows &rows, int lane, Emit &&emit) {
   const int f4 = F4 ? F4 : A.f4;
   const int fb = 16 * f4;  // bytes of factors per entry
   const uint32_t uv = (uint32_t)__cvta_generic_to_shared(sm), uw = uv + kRing * 32;
   const int total = rows.s[n_bins];  // steps
-  const int col = s0 + (lane & 3), g = lane >> 2;
+  constexpr int kStepsPerChunk = kChunk / G;
+  const int col = s0 + lane % (32 / G), g = lane / (32 / G);
   // chunk: lane j finds the entry of place j, then consecutive lanes copy
   // consecutive 16-byte pieces
   int my_row = 0;
   auto issue = [&](int chunk) {
-    const int step = chunk * (kChunk / 8) + (lane >> 3);
-    if (chunk * (kChunk / 8) < total) {
+    const int step = chunk * kStepsPerChunk + lane / G;
+    if (chunk * kStepsPerChunk < total) {
       int q = -1;
       if (step < total) {
         while (rows.s[my_row + 1] <= step) ++my_row;
-        const int k = (step - rows.s[my_row]) * 8 + (lane & 7);
+        const int k = (step - rows.s[my_row]) * G + lane % G;
         if (k < rows.n[my_row]) q = rows.q[my_row] + k;
       }
       const int slot = chunk % kSlots;
@@ -427,12 +473,12 @@ __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bin
       if (i < n_bins) {
 #pragma unroll 1
         for (const int end = rows.s[i + 1]; st < end; ++st) {
-          if ((st & 3) == 0) {  // a new chunk: the slot of the one before it is free
+          if (st % kStepsPerChunk == 0) {  // a new chunk: the slot of the one before it is free
             __syncwarp();
-            issue(st / 4 + kSlots - 1);
+            issue(st / kStepsPerChunk + kSlots - 1);
             asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
             __syncwarp();
-            const int slot = (st >> 2) % kSlots;
+            const int slot = st / kStepsPerChunk % kSlots;
             pv = uv + (slot * kChunk + g) * 32;
             pw = uw + (slot * kChunk + g) * fb;
           }
@@ -450,8 +496,8 @@ __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bin
           }
           float wx = 0.f;
           if ((unsigned)d < (unsigned)A.W) wx = __int_as_float(lds1(pw + 4 * d));
-          pv += 8 * 32;
-          pw += 8 * fb;
+          pv += G * 32;
+          pw += G * fb;
           const float t8[8] = {wx * v0.x, wx * v0.y, wx * v0.z, wx * v0.w,
                                wx * v1.x, wx * v1.y, wx * v1.z, wx * v1.w};
 #pragma unroll
@@ -459,15 +505,16 @@ __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bin
 #pragma unroll
             for (int p = 0; p < 8; ++p) acc[ph + t][p] = fmaf(wy[t], t8[p], acc[ph + t][p]);
         }
-        // the row that the window leaves: its eight components summed over the
-        // eight groups (a butterfly over lane bits 4, 3, 2 that halves the
+        // the row that the window leaves: its eight components, with eight groups
+        // summed over them (a butterfly over lane bits 4, 3, 2 that halves the
         // components each lane carries: group g ends with component g)
         float a[8];
 #pragma unroll
         for (int p = 0; p < 8; ++p) a[p] = acc[ph][p];
         if (i >= WN - 1) {
+          static_assert(G == 8 || G == 1, "the butterfly is over eight groups");
 #pragma unroll
-          for (int h = 4; h > 0; h >>= 1) {
+          for (int h = G / 2; h > 0; h >>= 1) {
             const bool up = lane & (4 * h);
 #pragma unroll
             for (int k = 0; k < h; ++k) {
@@ -475,7 +522,7 @@ __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bin
               a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
             }
           }
-          emit(i, a[0]);
+          emit(i, a);
         }
       }
     }
@@ -495,13 +542,14 @@ constexpr int kApplyCtas = 4;  // per SM: 16 warps at up to 128 registers
 // Bound by instruction issue (70 % of the slots, 59 % of the instructions on the
 // FMA pipe): 56 multiply-adds, 8 multiplies and about 20 other instructions per
 // step of 8 entries, of whose 4 x 7 cells the strip's edge leaves 70 % useful.
-// Measured for 12.5 M points on 4 x 2048^2 cells, W = 7: 0.55 ms a call, 0.076 of
+// Measured for 12.5 M points on 4 x 2048^2 cells, W = 7: 0.54 ms a call, 0.076 of
 // it the values; gathering both halves patch by patch with the factors of
 // every (patch, point) pair stored took 1.42 ms.  Not taken: packed two-wide
 // multiply-adds (67 per SM and cycle against 110 for scalar ones, measured),
 // two columns per lane, bins of two rows, seven window phases unrolled instead
 // of shifting registers (fetch stalls), more warps with spills.
-// Persistent CTAs.  Heavy units (units[0 .. n_heavy)): one CTA per unit, warp w takes the w-th quarter of every bin row and the four
+// Persistent CTAs.  Heavy units (units[0 .. n_heavy)): one CTA per unit, warp w
+// takes the w-th quarter of every bin row and the four
 // partial sums are added in warp order.  Then every warp takes the next light
 // unit until none is left (which warp takes it does not touch its sums).
 template <int WN, int F4>
@@ -525,7 +573,9 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
       u += A.n_heavy;
     }
     const int2 unit = __ldg(A.units + u);
-    const int s0 = unit.x * kCols, r0 = unit.y >> 8, n_rows = unit.y & 255;
+    const bool wide = unit.x & kWideFlag;
+    const int s0 = (unit.x & ~kWideFlag) * kCols, r0 = unit.y >> 8, n_rows = unit.y & 255;
+    const int c1 = min(s0 + (wide ? kWideCols : kCols) + A.W - 1, A.nbw);
     const int n_bins = n_rows + off;
     int carry = 0;
 #pragma unroll
@@ -535,14 +585,14 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
       if (i < n_bins) {
         const int *o = A.offsets + (int64_t)(r0 + i) * A.nbw;
         lo = __ldg(o + s0);
-        n = __ldg(o + min(s0 + kCols + A.W - 1, A.nbw)) - lo;
+        n = __ldg(o + c1) - lo;
         if (heavy) {
           const int first = (int)((int64_t)n * warp / kApplyWarps);
           n = (int)((int64_t)n * (warp + 1) / kApplyWarps) - first;
           lo += first;
         }
       }
-      int x = (n + 7) >> 3;  // steps, then their running sum
+      int x = wide ? n : (n + 7) >> 3;  // steps, then their running sum
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, x, d);
@@ -557,15 +607,24 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
     }
     if (lane == 0) rows.s[0] = 0;
     __syncwarp();
-    const int s = s0 + (lane & 3);
+    const int s = s0 + (wide ? lane : lane & 3);
+    RowOut out(A, r0, s, wide ? 0 : comp);
     if (carry == 0 && !heavy) {
-      for (int r = 0; r < n_rows; ++r) store_value(A, r0 + r, s, comp, 0.f);
-    } else {
-      strip_walk<WN, F4>(A, s0, n_bins, sm, rows, lane, [&](int i, float v) {
-        if (heavy)
-          part[(warp * kUnitRows + i - off) * 32 + lane] = v;
+      const float zero[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int r = 0; r < n_rows; ++r) {
+        if (wide)
+          out.put(zero);
         else
-          store_value(A, r0 + i - off, s, comp, v);
+          out.put(0.f, false);
+      }
+    } else if (wide) {
+      strip_walk<WN, F4, 1>(A, s0, n_bins, sm, rows, lane, [&](int, const float (&a)[8]) { out.put(a); });
+    } else {
+      strip_walk<WN, F4, 8>(A, s0, n_bins, sm, rows, lane, [&](int i, const float (&a)[8]) {
+        if (heavy)
+          part[(warp * kUnitRows + i - off) * 32 + lane] = a[0];
+        else
+          out.put(a[0], comp & 1);
       });
     }
     if (heavy) {
@@ -576,7 +635,7 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
         for (int w = 1; w < kApplyWarps; ++w) {
           v += part[(w * kUnitRows + r) * 32 + lane];
         }
-        store_value(A, r0 + r, s, comp, v);
+        RowOut(A, r0 + r, s, comp).put(v, comp & 1);
       }
       __syncthreads();
       h += gridDim.x;
@@ -749,26 +808,42 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
   int rows = kUnitRows;
   while (rows > 8 && (n_rows + rows - 1) / rows * n_cb < 2 * p->sms * kApplyCtas) rows /= 2;
-  const int n_u = (n_rows + rows - 1) / rows * n_cb;
-  std::vector<int> cnt(n_u);
-  if (e == cudaSuccess) e = cudaMalloc(&ucnt, sizeof(int) * n_u);
+  const int n_seg = (n_rows + rows - 1) / rows, per_wide = kWideCols / kCols, n_wcb = (n_cb + per_wide - 1) / per_wide;
+  const int n_u = n_seg * n_cb, n_wu = n_seg * n_wcb;
+  std::vector<int> cnt(n_u + n_wu);
+  if (e == cudaSuccess) e = cudaMalloc(&ucnt, sizeof(int) * (n_u + n_wu));
   if (e == cudaSuccess) {
-    grid_unit_count_kernel<<<(n_u + T - 1) / T, T, 0, stream>>>(p->offsets, n_u, n_cb, rows, n_rows, W, off,
+    grid_unit_count_kernel<<<(n_u + T - 1) / T, T, 0, stream>>>(p->offsets, n_u, n_cb, rows, n_rows, kCols, W, off,
                                                                p->nbw, ucnt);
+    grid_unit_count_kernel<<<(n_wu + T - 1) / T, T, 0, stream>>>(p->offsets, n_wu, n_wcb, rows, n_rows, kWideCols, W,
+                                                                off, p->nbw, ucnt + n_u);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(cnt.data(), ucnt, sizeof(int) * cnt.size(), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   std::vector<int2> heavy, units;
+  std::vector<std::pair<int, int2>> wide;  // (entries, unit)
   if (e == cudaSuccess) {
     int64_t total = 0;
     for (int u = 0; u < n_u; ++u) total += cnt[u];
     const int64_t most = std::max<int64_t>(256, total / ((int64_t)p->sms * kApplyCtas * kApplyWarps * 4));
-    for (int u = 0; u < n_u; ++u) {
-      const int r0 = u / n_cb * rows;
-      (cnt[u] > most ? heavy : units).push_back(make_int2(u % n_cb, r0 << 8 | std::min(rows, n_rows - r0)));
+    for (int seg = 0; seg < n_seg; ++seg) {
+      const int r0 = seg * rows, nr = std::min(rows, n_rows - r0);
+      for (int wb = 0; wb < n_wcb; ++wb) {
+        const int n_wide = cnt[n_u + seg * n_wcb + wb];
+        if (n_wide <= kWideEntries * rows / kUnitRows) {
+          for (int r = 0; r < nr; r += kWideRows)
+            wide.push_back({n_wide, make_int2(wb * per_wide | kWideFlag, (r0 + r) << 8 | std::min(kWideRows, nr - r))});
+          continue;
+        }
+        for (int cb = wb * per_wide; cb < std::min(n_cb, (wb + 1) * per_wide); ++cb)
+          (cnt[seg * n_cb + cb] > most ? heavy : units).push_back(make_int2(cb, r0 << 8 | nr));
+      }
     }
+    // the wide ones last, the shortest at the end
+    std::stable_sort(wide.begin(), wide.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+    for (const auto &w : wide) units.push_back(w.second);
     p->n_heavy = (int)heavy.size();
     p->n_light = (int)units.size();
     heavy.insert(heavy.end(), units.begin(), units.end());

@@ -1,7 +1,8 @@
 """The strip walk of the gridding call against the FP64 oracle where it can go
 wrong: one band and several (W = 1 .. 31), windows of five and seven rows,
 grids whose half plane is not a whole number of strips, columns that are not
-whole blocks, strips dense enough to be cut up and shared by a CTA, points
+whole blocks, strips dense enough to be cut up and shared by a CTA, sparse
+ones that are joined, points
 past every edge and points exactly on the mirror row and column.
 
 Tolerance: an FP32 sum of n terms in a fixed order is off by at most about
@@ -30,6 +31,9 @@ pytestmark = pytest.mark.gpu
     (5, 4, 80, 31, 6.0, 1.4),     # five bands, the largest support
     (24, 40, 16, 7, 1.0, 0.9),    # dense: every strip cut up, CTA-wide ones
     (24, 60, 40, 5, 0.8, 0.6),
+    (5, 3, 262, 7, 1.0, 1.2),     # sparse: joined strips of 32 columns, a short last one
+    (5, 3, 512, 9, 1.2, 1.2),     # the same in two bands
+    (16, 9, 256, 6, 0.8, 1.6),    # both kinds beside each other
 ])
 def test_strips(mw, n_tiles, n_chan, Ng, W, sigma, spill):  # noqa: F811
     tile_xy, vis, f0, df = problem(Ng * 100 + W, n_tiles, n_chan, Ng, 1.0, spill=spill)
