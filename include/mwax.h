@@ -295,8 +295,9 @@ mwax_status mwax_correlate_batch(mwax_plan_t plan, const void *const *voltages,
                                  void *const *out);
 
 /* Same as mwax_correlate with HOST buffers (pinned or pageable): channel
- * groups are copied in, correlated and copied out with copies overlapping
- * compute on the plan's stream and an internal copy stream.  Returns after
+ * groups (chan_group where the job sets it, else up to 16 of at least 32 MB) are
+ * copied in, correlated and copied out with copies overlapping
+ * compute on the plan's stream and internal copy streams.  Returns after
  * the output is complete in host memory. */
 mwax_status mwax_correlate_host(mwax_plan_t plan, const void *voltages_host, int n_inputs,
                                 int n_chan, int n_time, void *out_host);

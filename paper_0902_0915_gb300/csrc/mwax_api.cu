@@ -76,6 +76,11 @@ struct mwax_plan_s {
   // list of their one launch
   int4 *items = nullptr;
   int64_t n_items_full = 0, n_items_last = 0;
+  // host path: its own, smaller channel groups (copies and compute overlap), with
+  // their work lists and time ranges per item
+  int host_group = 0, host_split = 1;
+  int4 *host_items = nullptr;
+  int64_t n_host_full = 0, n_host_last = 0;
   // checked single segment (8-bit exact jobs longer than one exact segment):
   // the pair-mode pass accumulates each item in one FP32 segment, a check
   // lists the channels whose largest auto-correlation reached 2^24 (bad[0] =
@@ -333,18 +338,19 @@ int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int 
 bool pair_like(int mode) { return mode == 2 || mode == 3; }
 
 // Build the pair-mode work lists (a and, if non-empty, b after it) and copy
-// them to a device buffer owned by the plan.
-cudaError_t upload_items(mwax_plan_s *p, const std::vector<TcJob> &a, const std::vector<TcJob> &b) {
+// them to a device buffer (*items, owned by the plan).
+cudaError_t upload_items(const std::vector<TcJob> &a, const std::vector<TcJob> &b, int4 **items,
+                         int64_t *n_a, int64_t *n_b) {
   std::vector<int4> la, lb;
   build_pair_items(a.data(), (int)a.size(), la);
   if (!b.empty()) build_pair_items(b.data(), (int)b.size(), lb);
-  p->n_items_full = (int64_t)la.size();
-  p->n_items_last = (int64_t)lb.size();
+  *n_a = (int64_t)la.size();
+  *n_b = (int64_t)lb.size();
   la.insert(la.end(), lb.begin(), lb.end());
   if (la.empty()) return cudaSuccess;
-  cudaError_t e = plan_alloc(reinterpret_cast<void **>(&p->items), la.size() * sizeof(int4));
+  cudaError_t e = plan_alloc(reinterpret_cast<void **>(items), la.size() * sizeof(int4));
   if (e == cudaSuccess)
-    e = cudaMemcpy(p->items, la.data(), la.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(*items, la.data(), la.size() * sizeof(int4), cudaMemcpyHostToDevice);
   return e;
 }
 
@@ -444,7 +450,7 @@ cudaError_t unpack_rows(mwax_plan_s *p, const JobState &s, const uint8_t *rows, 
 }
 
 mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op, int nc,
-                            void *out_c0, cudaStream_t st, bool use_pair = true) {
+                            void *out_c0, cudaStream_t st, bool use_pair = true, bool host = false) {
   TcJob tj = tc_job(s, op, out_c0, nc);
   TcLaunch cfg = launch_cfg(p);
   if (pair_like(p->mode) && !use_pair) {  // a checked plan's narrow call (op: operand tiles)
@@ -456,9 +462,11 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
     return cuda_status(e);
   }
   if (pair_like(p->mode)) {
-    const bool full = nc == s.chan_group;
-    cfg.items = full ? p->items : p->items + p->n_items_full;
-    cfg.n_items = full ? p->n_items_full : p->n_items_last;
+    const bool full = nc == s.chan_group;  // (host path: s is its own JobState)
+    const int4 *items = host ? p->host_items : p->items;
+    const int64_t n_full = host ? p->n_host_full : p->n_items_full;
+    cfg.items = full ? items : items + n_full;
+    cfg.n_items = full ? n_full : host ? p->n_host_last : p->n_items_last;
     if (p->checked) tj.flush_blocks = s.kb;  // one optimistic segment per item
   }
   TimedLaunch tc(p, 1, st);
@@ -495,7 +503,7 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
 // fused pair mode reads the packed samples itself, or the scratch's padded copy
 // of their rows).
 mwax_status run_group(mwax_plan_s *p, const JobState &s, const uint8_t *volt, int64_t c0, int nc,
-                      void *out_c0, cudaStream_t st, bool use_pair = true) {
+                      void *out_c0, cudaStream_t st, bool use_pair = true, bool host = false) {
   if (p->mode == 3) {
     const uint8_t *rows = volt + c0 * s.in_chan_bytes;
     if (s.ragged()) {
@@ -513,11 +521,11 @@ mwax_status run_group(mwax_plan_s *p, const JobState &s, const uint8_t *volt, in
       if (e != cudaSuccess) return cuda_status(e);
       rows = p->scratch;
     }
-    return correlate_group(p, s, rows, nc, out_c0, st, use_pair);
+    return correlate_group(p, s, rows, nc, out_c0, st, use_pair, host);
   }
   mwax_status r = unpack_group(p, s, volt, c0, nc, p->scratch, 0, st);
   if (r != MWAX_OK) return r;
-  return correlate_group(p, s, p->scratch, nc, out_c0, st, use_pair);
+  return correlate_group(p, s, p->scratch, nc, out_c0, st, use_pair, host);
 }
 
 mwax_status correlate_device(mwax_plan_s *p, const uint8_t *volt, void *out, cudaStream_t st) {
@@ -570,6 +578,37 @@ mwax_status correlate_device(mwax_plan_s *p, const uint8_t *volt, void *out, cud
   return p->checked && use_pair ? cuda_status(checked_call_done(p, st)) : MWAX_OK;
 }
 
+// Channel groups of the host path: at most 16 and at least 32 MB of samples each
+// (a plan's own group is sized for the scratch and often holds every channel, so
+// that nothing overlapped the input copy: 256 inputs x 96 channels x 20,000 4-bit
+// samples took 2.77 ms in one group, 2.47 in 14), unless the caller set chan_group.  Small groups
+// have few work items, so the time ranges per item are chosen for them.
+cudaError_t prepare_host_groups(mwax_plan_s *p) {
+  const JobState &s = p->jobs[0];
+  int64_t g = s.chan_group;
+  if (s.job.chan_group == 0) {
+    const int64_t by_bytes = ((int64_t(32) << 20) + s.in_chan_bytes - 1) / s.in_chan_bytes;
+    g = std::min<int64_t>(g, std::max<int64_t>(by_bytes, (s.job.n_chan + 15) / 16));
+  }
+  p->host_group = (int)g;
+  p->host_split = s.k_split;
+  if (!pair_like(p->mode)) return cudaSuccess;
+  std::vector<TcJob> full = {tc_job(s, nullptr, nullptr, (int)g)}, tail;
+  if (p->checked) full[0].flush_blocks = s.kb;
+  if (s.job.k_split == 0) {
+    full[0].k_split = 1;
+    std::vector<int4> base;
+    build_pair_items(full.data(), 1, base);
+    p->host_split = resolve_split(s.job, p->mode, s.kb, (int64_t)base.size(), p->sm_count);
+  }
+  full[0].k_split = p->host_split;
+  if (const int last = (int)(s.job.n_chan % g)) {
+    tail = full;
+    tail[0].n_chan = last;
+  }
+  return upload_items(full, tail, &p->host_items, &p->n_host_full, &p->n_host_last);
+}
+
 void free_plan(mwax_plan_s *p) {
   if (!p) return;
   if (p->graph) cudaGraphExecDestroy(p->graph);
@@ -581,6 +620,7 @@ void free_plan(mwax_plan_s *p) {
   if (p->rows) cudaFree(p->rows);
   if (p->status) cudaFree(p->status);
   if (p->items) cudaFree(p->items);
+  if (p->host_items) cudaFree(p->host_items);
   if (p->bad) cudaFree(p->bad);
   if (p->recomputed) cudaFree(p->recomputed);
   if (p->recomp_host) cudaFreeHost(p->recomp_host);
@@ -748,7 +788,7 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
         tail.push_back(tc_job(s, nullptr, nullptr, last));
         tail[0].flush_blocks = full[0].flush_blocks;
       }
-      e = upload_items(p, full, tail);
+      e = upload_items(full, tail, &p->items, &p->n_items_full, &p->n_items_last);
     }
     if (e == cudaSuccess && p->checked) {
       e = plan_alloc(reinterpret_cast<void **>(&p->bad), (size_t)(s.chan_group + 1) * sizeof(int32_t));
@@ -840,7 +880,8 @@ mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
   }
   p->stages = jobs[0].stages > 0 ? jobs[0].stages : correlate_tc_max_stages(p->mode);
   cudaError_t e = p->stages <= correlate_tc_max_stages(p->mode) ? cudaSuccess : cudaErrorInvalidValue;
-  if (e == cudaSuccess && pair_like(p->mode)) e = upload_items(p, tj, {});
+  if (e == cudaSuccess && pair_like(p->mode))
+    e = upload_items(tj, {}, &p->items, &p->n_items_full, &p->n_items_last);
   if (e == cudaSuccess) e = correlate_tc_prepare(p->sample_bits, p->kind, p->stages, p->mode);
   if (e != cudaSuccess) {
     free_plan(p);
@@ -1054,11 +1095,23 @@ mwax_status mwax_correlate_host(mwax_plan_t plan, const void *voltages_host, int
                                 int n_chan, int n_time, void *out_host) {
   NvtxRange nvtx_("mwax_correlate_host");
   if (!plan || plan->batch || !voltages_host || !out_host) return MWAX_ERR_INVALID_ARG;
-  JobState &s = plan->jobs[0];
-  if (n_inputs != s.job.n_inputs || n_chan != s.job.n_chan || n_time != s.job.n_time)
+  if (n_inputs != plan->jobs[0].job.n_inputs || n_chan != plan->jobs[0].job.n_chan ||
+      n_time != plan->jobs[0].job.n_time)
     return MWAX_ERR_SHAPE_MISMATCH;
-  const int G = s.chan_group;
   cudaError_t e = cudaSuccess;
+  if (plan->host_group == 0) {
+    e = prepare_host_groups(plan);
+    if (e != cudaSuccess) {
+      if (plan->host_items) cudaFree(plan->host_items);
+      plan->host_items = nullptr;
+      plan->host_group = 0;
+      return cuda_status(e);
+    }
+  }
+  JobState s = plan->jobs[0];
+  s.chan_group = plan->host_group;
+  s.k_split = plan->host_split;
+  const int G = s.chan_group;
   if (!plan->h2d) {
     plan->stage_in_bytes = s.in_chan_bytes * G;
     plan->stage_out_bytes = s.out_chan_bytes * G;
@@ -1105,7 +1158,7 @@ mwax_status mwax_correlate_host(mwax_plan_t plan, const void *voltages_host, int
             s.job.n_time, reinterpret_cast<int32_t *>(plan->stage_out[k]) + (int64_t)c * s.n_bl * 2,
             plan->sm_count, plan->stream));
     } else {
-      r = run_group(plan, s, plan->stage_in[k], 0, nc, plan->stage_out[k], plan->stream, use_pair);
+      r = run_group(plan, s, plan->stage_in[k], 0, nc, plan->stage_out[k], plan->stream, use_pair, true);
     }
     if (r != MWAX_OK) return r;
     e = cudaEventRecord(plan->ev_comp[k], plan->stream);
