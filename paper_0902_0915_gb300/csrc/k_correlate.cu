@@ -139,6 +139,9 @@ struct KParams {
   unsigned long long timeout_ns;
   int32_t n_jobs, stages, prefetch;
   int32_t withhold_seg;  // test hook: segment whose accumulator release the epilogue withholds (-1: none)
+  int32_t dependent, lets_start;  // as in TcLaunch
+  int32_t *clear;
+  unsigned long long *clear64;
 };
 
 struct KMaps {
@@ -377,7 +380,7 @@ __device__ __forceinline__ Item decode_item(const KParams &p, int64_t item) {
   Item it;
   it.job = j;
   const int cl = (int)(local / p.job[j].n_pairs);
-  it.c = p.chan_map ? __ldg(p.chan_map + cl) : cl;
+  it.c = p.chan_map ? __ldcg(p.chan_map + cl) : cl;
   pair_of((int)(local % p.job[j].n_pairs), it.I, it.J);
   return it;
 }
@@ -696,6 +699,7 @@ __device__ __forceinline__ bool drain_item(const KParams &p, const PairItem &it,
   named_bar_sync(1, EW * 32);
   if (!epi_flag[n_it & 1u]) return false;
   tc_fence_after();
+  if (it.n_split > 1) wait_for_predecessor();  // the output is zero
   const bool has = h == 0 || it.type != kItemOne;
   int c, I, J;
   if (it.type == kItemShared) {
@@ -899,6 +903,7 @@ __device__ __forceinline__ void pair_roles(const KMaps &maps, const KParams &p, 
         }
         ++n_it;
       }
+      if (p.lets_start) let_dependents_start();  // beside the last item's epilogue
       // no MMA may be in flight when tensor memory is freed
       tc_commit(drain);
       mbar_wait(drain, 0, nullptr, tmo);
@@ -1011,6 +1016,11 @@ __global__ void __launch_bounds__(Shape<MODE>::warps * 32, 1)
   const unsigned long long tmo = p.timeout_ns;
   const uint32_t smem_base = smem_u32(smem);
 
+  if (!PAIR && p.dependent) wait_for_predecessor();
+  if (PAIR && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (p.clear) *p.clear = 0;
+    if (p.clear64) *p.clear64 = 0;
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full(s), Sh::fill_arrivals);  // the TMA producer, or the converting warps
@@ -1333,10 +1343,12 @@ __global__ void __launch_bounds__(256) exact_check_kernel(const int32_t *out, in
                                                           unsigned long long *recomputed) {
   // recomputed[0]: running total for the caller, recomputed[1]: this call
   const int c = blockIdx.x;
+  let_dependents_start();
+  wait_for_predecessor();
   const int32_t *o = out + (int64_t)c * n_bl * 2;
   uint32_t m = 0;
   for (int i = threadIdx.x; i < n_inputs; i += blockDim.x)
-    m = max(m, (uint32_t)__ldg(o + 2 * ((int64_t)i * (i + 1) / 2 + i)));  // negative -> huge
+    m = max(m, (uint32_t)__ldcg(o + 2 * ((int64_t)i * (i + 1) / 2 + i)));  // negative -> huge
   m = __reduce_max_sync(0xffffffffu, m);
   __shared__ uint32_t wmax[8];
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
@@ -1372,6 +1384,11 @@ cudaError_t set_smem_attr(int bytes) {
                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
+__global__ void __launch_bounds__(256) zero_kernel(int32_t *out, int64_t n) {
+  let_dependents_start();
+  for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < n; k += (int64_t)gridDim.x * 256) out[k] = 0;
+}
+
 template <int MODE>
 cudaError_t prepare_shape(int sample_bits, int kind, int bytes) {
   if (sample_bits == 4) return set_smem_attr<4, MWAX_KIND_EXACT, MODE>(bytes);
@@ -1386,28 +1403,34 @@ cudaError_t prepare_fused(int sample_bits, int kind, int bytes) {
                                   : set_smem_attr<16, MWAX_KIND_EXACT, MODE>(bytes);
 }
 
-template <int MODE>
-void launch_fused(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
-                  const KParams &kp) {
-  const int threads = Shape<MODE>::warps * 32;
-  if (sample_bits == 4)
-    correlate_tc_kernel<4, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
-  else if (kind == MWAX_KIND_FP16)
-    correlate_tc_kernel<16, MWAX_KIND_FP16, MODE><<<grid, threads, smem, s>>>(maps, kp);
-  else
-    correlate_tc_kernel<16, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
+template <class K>
+cudaError_t launch_kernel(K kernel, int grid, int threads, int smem, cudaStream_t s, const KMaps &maps,
+                          const KParams &kp) {
+  if (kp.dependent) return launch_dependent(kernel, grid, threads, smem, s, maps, kp);
+  kernel<<<grid, threads, smem, s>>>(maps, kp);
+  return cudaGetLastError();
 }
 
 template <int MODE>
-void launch_shape(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
+cudaError_t launch_fused(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
                   const KParams &kp) {
   const int threads = Shape<MODE>::warps * 32;
   if (sample_bits == 4)
-    correlate_tc_kernel<4, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
-  else if (kind == MWAX_KIND_FP16)
-    correlate_tc_kernel<8, MWAX_KIND_FP16, MODE><<<grid, threads, smem, s>>>(maps, kp);
-  else
-    correlate_tc_kernel<8, MWAX_KIND_EXACT, MODE><<<grid, threads, smem, s>>>(maps, kp);
+    return launch_kernel(correlate_tc_kernel<4, MWAX_KIND_EXACT, MODE>, grid, threads, smem, s, maps, kp);
+  if (kind == MWAX_KIND_FP16)
+    return launch_kernel(correlate_tc_kernel<16, MWAX_KIND_FP16, MODE>, grid, threads, smem, s, maps, kp);
+  return launch_kernel(correlate_tc_kernel<16, MWAX_KIND_EXACT, MODE>, grid, threads, smem, s, maps, kp);
+}
+
+template <int MODE>
+cudaError_t launch_shape(int sample_bits, int kind, int grid, int smem, cudaStream_t s, const KMaps &maps,
+                  const KParams &kp) {
+  const int threads = Shape<MODE>::warps * 32;
+  if (sample_bits == 4)
+    return launch_kernel(correlate_tc_kernel<4, MWAX_KIND_EXACT, MODE>, grid, threads, smem, s, maps, kp);
+  if (kind == MWAX_KIND_FP16)
+    return launch_kernel(correlate_tc_kernel<8, MWAX_KIND_FP16, MODE>, grid, threads, smem, s, maps, kp);
+  return launch_kernel(correlate_tc_kernel<8, MWAX_KIND_EXACT, MODE>, grid, threads, smem, s, maps, kp);
 }
 
 int4 encode_item(int job, uint32_t type, int c0, int c1, int I0, int J0, int I1, int J1,
@@ -1450,9 +1473,14 @@ cudaError_t correlate_tc_prepare(int sample_bits, int kind, int stages, int mode
 
 cudaError_t launch_exact_check(const int32_t *out, int64_t n_bl, int n_inputs, int n_chan,
                                int32_t *bad, unsigned long long *recomputed, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int32_t), s);
-  if (e != cudaSuccess || n_chan <= 0) return e;
-  exact_check_kernel<<<n_chan, 256, 0, s>>>(out, n_bl, n_inputs, bad, recomputed);
+  if (n_chan <= 0) return cudaSuccess;
+  return launch_dependent(exact_check_kernel, n_chan, 256, 0, s, out, n_bl, n_inputs, bad, recomputed);
+}
+
+cudaError_t launch_zero(int32_t *out, int64_t n, int sm_count, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const int64_t ctas = std::min<int64_t>((n + 255) / 256, 8 * (int64_t)sm_count);
+  zero_kernel<<<(unsigned)ctas, 256, 0, s>>>(out, n);
   return cudaGetLastError();
 }
 
@@ -1605,20 +1633,21 @@ cudaError_t launch_correlate_tc(const TcJob *jobs, int n_jobs, const TcLaunch &c
   kp.stages = cfg.stages;
   kp.prefetch = cfg.prefetch;
   kp.withhold_seg = cfg.withhold_seg;
+  kp.dependent = cfg.dependent;
+  kp.lets_start = cfg.lets_start;
+  kp.clear = cfg.clear;
+  kp.clear64 = cfg.clear64;
   if (items <= 0) return cudaSuccess;
   const int grid = (int)(items < cfg.grid ? items : cfg.grid);
   const int smem = correlate_tc_smem_bytes(cfg.stages, cfg.mode);
   if (cfg.mode == kModeWide)
-    launch_shape<kModeWide>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else if (cfg.mode == kModePair)
-    launch_shape<kModePair>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else if (fused && words)
-    launch_fused<kModePairFusedWords>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else if (fused)
-    launch_fused<kModePairFused>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  else
-    launch_shape<kModeNarrow>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
-  return cudaGetLastError();
+    return launch_shape<kModeWide>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
+  if (cfg.mode == kModePair)
+    return launch_shape<kModePair>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
+  if (fused && words)
+    return launch_fused<kModePairFusedWords>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
+  if (fused) return launch_fused<kModePairFused>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
+  return launch_shape<kModeNarrow>(cfg.sample_bits, cfg.kind, grid, smem, s, maps, kp);
 }
 
 }  // namespace mwax

@@ -421,8 +421,12 @@ __global__ void __launch_bounds__(kTileThreads, 6)
   uint8_t *raw = sm + kTile * kRowBytes;  // 32 samples x 256 B
   __shared__ __align__(8) uint64_t bar;
   const uint32_t b = (uint32_t)__cvta_generic_to_shared(&bar);
-  if (MAPPED) n_chan = *n_chan_dev;
-  const auto chan_of = [&](int c) { return MAPPED ? __ldg(chan_map + c) : c; };
+  if (MAPPED) {  // a dependent of the kernel that made the list
+    let_dependents_start();
+    wait_for_predecessor();
+    n_chan = __ldcg(n_chan_dev);
+  }
+  const auto chan_of = [&](int c) { return MAPPED ? __ldcg(chan_map + c) : c; };
   const int n_rows = n_tiles * kTile;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
@@ -678,10 +682,10 @@ cudaError_t launch_unpack_tile(const uint8_t *volt, int sample_bits, int n_input
 #define MWAX_TILE_ARGS \
   in_map, out_map, volt, n_inputs, n_time, n_tiles, kb, chan0, n_chan, status, timeout_ns, chan_map, n_chan_dev
   if (chan_map && tma_in)
-    unpack8_tile_kernel<true, true><<<ctas, kTileThreads, smem, s>>>(MWAX_TILE_ARGS);
-  else if (chan_map)
-    unpack8_tile_kernel<false, true><<<ctas, kTileThreads, smem, s>>>(MWAX_TILE_ARGS);
-  else if (tma_in)
+    return launch_dependent(unpack8_tile_kernel<true, true>, ctas, kTileThreads, smem, s, MWAX_TILE_ARGS);
+  if (chan_map)
+    return launch_dependent(unpack8_tile_kernel<false, true>, ctas, kTileThreads, smem, s, MWAX_TILE_ARGS);
+  if (tma_in)
     unpack8_tile_kernel<true, false><<<ctas, kTileThreads, smem, s>>>(MWAX_TILE_ARGS);
   else
     unpack8_tile_kernel<false, false><<<ctas, kTileThreads, smem, s>>>(MWAX_TILE_ARGS);

@@ -91,6 +91,7 @@ struct mwax_plan_s {
   // [0]: channels recomputed since the caller last read the count; [1]: in
   // the current call (copied to recomp_host at the end of each call)
   unsigned long long *recomputed = nullptr;
+  bool clear_count = false;  // the next pair pass sets recomputed[1] to 0
   // adaptivity: after a call in which more than a quarter of the channels
   // had to be recomputed, the next kNarrowCalls calls run the narrow shape
   // directly, then the pair pass is tried again
@@ -425,6 +426,7 @@ bool checked_call_uses_pair(mwax_plan_s *p) {
     --p->narrow_calls_left;
     return false;
   }
+  p->clear_count = true;  // by the first group's correlation
   return true;
 }
 
@@ -433,7 +435,6 @@ bool checked_call_uses_pair(mwax_plan_s *p) {
 cudaError_t checked_call_done(mwax_plan_s *p, cudaStream_t st) {
   cudaError_t e = cudaMemcpyAsync(p->recomp_host, p->recomputed + 1, sizeof(unsigned long long),
                                   cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->recomputed + 1, 0, sizeof(unsigned long long), st);
   if (e == cudaSuccess) e = cudaEventRecord(p->ev_recomp, st);
   if (e == cudaSuccess) p->recomp_pending = true;
   return e;
@@ -448,6 +449,10 @@ cudaError_t unpack_rows(mwax_plan_s *p, const JobState &s, const uint8_t *rows, 
                             s.n_tiles, s.kb, 0, nc, p->scratch, p->sm_count * kTileCtasPerSm, p->status,
                             p->timeout_ns, st, chan_map, n_chan_dev);
 }
+
+// Output that a zeroing kernel covers, so that the correlation can start beside
+// it; larger ones take the driver's memset, which is faster by itself.
+constexpr int64_t kZeroKernelBytes = int64_t(8) << 20;
 
 mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op, int nc,
                             void *out_c0, cudaStream_t st, bool use_pair = true, bool host = false) {
@@ -471,8 +476,18 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
   }
   TimedLaunch tc(p, 1, st);
   cudaError_t e = cudaSuccess;
-  if (pair_like(p->mode) && s.k_split > 1)  // the time ranges' partial sums are added into it
-    e = cudaMemsetAsync(out_c0, 0, (size_t)(nc * s.out_chan_bytes), st);
+  if (pair_like(p->mode) && s.k_split > 1) {  // the time ranges' partial sums are added into it
+    const int64_t bytes = nc * s.out_chan_bytes;
+    cfg.dependent = bytes <= kZeroKernelBytes;
+    e = cfg.dependent ? launch_zero(reinterpret_cast<int32_t *>(out_c0), bytes / 4, p->sm_count, st)
+                      : cudaMemsetAsync(out_c0, 0, (size_t)bytes, st);
+  }
+  if (p->checked) {
+    cfg.lets_start = true;
+    cfg.clear = p->bad;
+    cfg.clear64 = p->clear_count ? p->recomputed + 1 : nullptr;
+    p->clear_count = false;
+  }
   if (e == cudaSuccess) e = launch_correlate_tc(&tj, 1, cfg, st);
   if (e == cudaSuccess && p->checked) {
     e = launch_exact_check(reinterpret_cast<const int32_t *>(out_c0), s.n_bl, s.job.n_inputs, nc,
@@ -491,6 +506,7 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
       fc.withhold_seg = -1;
       fc.chan_map = p->bad + 1;
       fc.n_chan_dev = p->bad;
+      fc.dependent = true;
       if (e == cudaSuccess) e = launch_correlate_tc(&fj, 1, fc, st);
     }
   }

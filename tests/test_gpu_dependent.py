@@ -1,0 +1,53 @@
+"""Launches that start beside their predecessor: time ranges added into an output
+that a kernel zeroes (up to 8 MB) or the driver's memset does, called again and
+again over a dirty output, directly and from a captured graph.  Integer results: equal to the oracle's."""
+import pytest
+import torch
+
+import synth
+from gpu_util import assert_exact, device_volt, oracle_for
+from test_gpu_correlate import mw  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def calls(mw, spec, **kw):  # noqa: F811
+    p = mw.Plan(spec.n_inputs, spec.n_chan, spec.n_time, spec.sample_bits, **kw)
+    volt = device_volt(spec)
+    ref = oracle_for(spec, range(spec.n_chan))
+    out = p.correlate(volt)
+    assert p.status() == 0
+    assert_exact(out.cpu().numpy(), ref, "first")
+    for _ in range(3):
+        out.fill_(-7)
+        p.correlate(volt, out)
+        p.correlate(volt, out)
+    assert_exact(out.cpu().numpy(), ref, "again")
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    q = mw.Plan(spec.n_inputs, spec.n_chan, spec.n_time, spec.sample_bits, stream=s, **kw)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        q.correlate(volt, out)
+        s.synchronize()
+        with torch.cuda.graph(g, stream=s):
+            q.correlate(volt, out)
+        out.fill_(-7)
+        g.replay()
+        g.replay()
+    torch.cuda.synchronize()
+    assert p.status() == 0 and q.status() == 0
+    assert_exact(out.cpu().numpy(), ref, "graph")
+    q.close()
+    p.close()
+
+
+@pytest.mark.parametrize("bits,N,C,T", [
+    (4, 64, 5, 700), (4, 100, 3, 900), (8, 48, 4, 300), (8, 250, 3, 290),
+    (4, 512, 7, 257),  # 7.4 MB of output
+    (4, 512, 8, 257),  # 8.4 MB
+])
+@pytest.mark.parametrize("shape", [0, 3])
+def test_time_ranges(mw, bits, N, C, T, shape):  # noqa: F811
+    spec = synth.Spec("dep", N, C, T, bits, seed=N + T, sigma=2 if bits == 4 else 20, tone_amp=0.3)
+    calls(mw, spec, mma_shape=shape, k_split=2)
