@@ -51,3 +51,23 @@ def calls(mw, spec, **kw):  # noqa: F811
 def test_time_ranges(mw, bits, N, C, T, shape):  # noqa: F811
     spec = synth.Spec("dep", N, C, T, bits, seed=N + T, sigma=2 if bits == 4 else 20, tone_amp=0.3)
     calls(mw, spec, mma_shape=shape, k_split=2)
+
+
+@pytest.mark.parametrize("gains", ["input", "chan", "jones"])
+@pytest.mark.parametrize("N,C", [(4, 1), (64, 3), (100, 70), (256, 40)])
+def test_sweeps_in_one_call_and_in_several(mw, gains, N, C):  # noqa: F811
+    """Every pair of sweeps runs the same kernels: equal bit for bit."""
+    gen = torch.Generator(device="cuda").manual_seed(N + C)
+    size = {"input": (N,), "chan": (C, N), "jones": (N // 2, 2, 2)}[gains]
+    solve = {"input": mw.calib_solve, "chan": mw.calib_chan_solve, "jones": mw.calib_jones_solve}[gains]
+    cplx = lambda *s: torch.randn(*s, dtype=torch.complex64, device="cuda", generator=gen)  # noqa: E731
+    V, M = cplx(C, N * (N + 1) // 2), cplx(C, N * (N + 1) // 2)
+    g0 = cplx(*size) + (2 * torch.eye(2, device="cuda") if gains == "jones" else 2)
+    whole, losses = solve(V, M, g0, 12)
+    g, parts = g0, []
+    for _ in range(6):
+        g, h = solve(V, M, g, 2)
+        torch.cuda.synchronize()
+        parts.append(h)
+    assert torch.isfinite(torch.view_as_real(whole)).all()
+    assert torch.equal(whole, g) and torch.equal(losses, torch.cat(parts))
