@@ -1125,12 +1125,11 @@ def main():
         # a checked-segment correlate launch is followed by the check kernel and
         # the (usually empty) recompute launch inside the same timed record (in the
         # fused pair mode also the unpack of the channels to recompute)
-        # (time ranges per item: a kernel zeroes an output of up to 8 MB first)
+        # (time ranges per item: a kernel zeroes the output first)
         "gpu_launches": int(tim.unpack_launches
                             + tim.correlate_launches * (1 if not info.checked_segment
                                                         else 4 if info.mma_shape == 4 else 3)
-                            + (tim.correlate_launches if info.k_split > 1 and info.chan_group
-                               * rspec.n_inputs * (rspec.n_inputs + 1) * 4 <= 8 << 20 else 0)),
+                            + (tim.correlate_launches if info.k_split > 1 else 0)),
         "clocks": clk,
     }
 

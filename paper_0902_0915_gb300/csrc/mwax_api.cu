@@ -450,10 +450,6 @@ cudaError_t unpack_rows(mwax_plan_s *p, const JobState &s, const uint8_t *rows, 
                             p->timeout_ns, st, chan_map, n_chan_dev);
 }
 
-// Output that a zeroing kernel covers, so that the correlation can start beside
-// it; larger ones take the driver's memset, which is faster by itself.
-constexpr int64_t kZeroKernelBytes = int64_t(8) << 20;
-
 mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op, int nc,
                             void *out_c0, cudaStream_t st, bool use_pair = true, bool host = false) {
   TcJob tj = tc_job(s, op, out_c0, nc);
@@ -477,10 +473,8 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
   TimedLaunch tc(p, 1, st);
   cudaError_t e = cudaSuccess;
   if (pair_like(p->mode) && s.k_split > 1) {  // the time ranges' partial sums are added into it
-    const int64_t bytes = nc * s.out_chan_bytes;
-    cfg.dependent = bytes <= kZeroKernelBytes;
-    e = cfg.dependent ? launch_zero(reinterpret_cast<int32_t *>(out_c0), bytes / 4, p->sm_count, st)
-                      : cudaMemsetAsync(out_c0, 0, (size_t)bytes, st);
+    e = launch_zero(reinterpret_cast<int32_t *>(out_c0), nc * s.out_chan_bytes / 4, p->sm_count, st);
+    cfg.dependent = true;
   }
   if (p->checked) {
     cfg.lets_start = true;

@@ -149,7 +149,9 @@ void build_pair_items(const TcJob *jobs, int n_jobs, std::vector<int4> &items);
 cudaError_t launch_exact_check(const int32_t *out, int64_t n_bl, int n_inputs, int n_chan,
                                int32_t *bad, unsigned long long *recomputed, cudaStream_t s);
 
-// out[0 .. n) = 0, a kernel whose successor may be a dependent.
+// out[0 .. n) = 0, a kernel whose successor may be a dependent (against a memset and
+// an ordinary launch: 512 inputs x 2000 samples of 4 bits, two time ranges, 1 MB of
+// output 31.4 / 33.4 us a call, 16 MB 56.0 / 60.1, 256 MB 516 / 528).
 cudaError_t launch_zero(int32_t *out, int64_t n, int sm_count, cudaStream_t s);
 
 #ifdef __CUDACC__

@@ -1,6 +1,7 @@
 """Launches that start beside their predecessor: time ranges added into an output
-that a kernel zeroes (up to 8 MB) or the driver's memset does, called again and
-again over a dirty output, directly and from a captured graph.  Integer results: equal to the oracle's."""
+that a kernel zeroes beside them, called again and again over a dirty output,
+directly and from a captured graph (integer results: equal to the oracle's); a
+solve's sweeps in one call and in several."""
 import pytest
 import torch
 
@@ -44,8 +45,8 @@ def calls(mw, spec, **kw):  # noqa: F811
 
 @pytest.mark.parametrize("bits,N,C,T", [
     (4, 64, 5, 700), (4, 100, 3, 900), (8, 48, 4, 300), (8, 250, 3, 290),
-    (4, 512, 7, 257),  # 7.4 MB of output
-    (4, 512, 8, 257),  # 8.4 MB
+    (4, 512, 7, 257),
+    (4, 512, 8, 257),  # more words than the zeroing kernel has threads
 ])
 @pytest.mark.parametrize("shape", [0, 3])
 def test_time_ranges(mw, bits, N, C, T, shape):  # noqa: F811
