@@ -102,6 +102,14 @@ __device__ __forceinline__ Support point_support(const GridGeom &g, int64_t k) {
     p.y = (double)g.Ng - p.y;
   }
   const double half = 0.5 * g.W;
+  // A point that is not within W cells of the grid, or not finite, reaches no cell:
+  // an empty support, whose bounds need no conversion (which would leave an int).
+  const double near = g.Ng + (double)g.W;
+  if (!(p.x > -(double)g.W && p.x < near && p.y > -(double)g.W && p.y < near)) {
+    p.s_lo = p.r_lo = 0;
+    p.s_hi = p.r_hi = -1;
+    return p;
+  }
   // cells strictly within half the support: the smallest integer above x - W/2
   // and the largest below x + W/2
   p.s_lo = (int)floor(p.x - half) + 1;
