@@ -36,6 +36,7 @@
 
 #include "mwax_internal.h"
 #include "mwax_nib4.h"
+#include "mwax_rows.h"
 
 namespace mwax {
 namespace {
@@ -258,13 +259,20 @@ __global__ void __launch_bounds__(256) unpack4_mn_kernel(const uint8_t *__restri
 // For the fused pair mode, whose warps read whole 16-byte units: rows of N
 // bytes (N not a multiple of 16) copied to rows of P = N rounded up.  A thread
 // makes one 16-byte unit of a row from the one or two aligned units of the input
-// that hold it (an aligned unit is only read when at least one of its bytes is
-// wanted, so no read leaves the last unit of the buffer) by selecting words and
-// funnel shifts.  The P - N bytes past a row's end are whatever follows it: they
-// are operand rows past the last input, whose products are never stored.
+// that hold it (read only where one of its bytes is wanted, and byte by byte where
+// the samples end inside it: nothing past them is read) by selecting words and
+// funnel shifts.  The P - N bytes past a row's end are the next row's, or zeros:
+// they are operand rows past the last input, whose products are never stored.
 // HBM-bound, twice the sample bytes (the unpack moves three times as many, and
 // its operands are read twice as wide).
 constexpr int kRepackRows = 4;  // rows in flight per thread
+struct LoadGlobal {
+  static __device__ __forceinline__ Unit16 unit(const uint8_t *p) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+    return Unit16{{v.x, v.y, v.z, v.w}};
+  }
+  static __device__ __forceinline__ uint8_t byte(const uint8_t *p) { return __ldg(p); }
+};
 __global__ void __launch_bounds__(256) repack_kernel(const uint8_t *__restrict__ volt,
                                                       uint8_t *__restrict__ out, int N, int P,
                                                       int64_t rows) {
@@ -276,22 +284,22 @@ __global__ void __launch_bounds__(256) repack_kernel(const uint8_t *__restrict__
   const int gstep = long_rows ? (int)blockDim.x : upr;
   if (r_off >= rpb) return;
   const int64_t rstride = (int64_t)gridDim.x * rpb;
+  // rows after which at least 15 more bytes follow (the others, at the end, test every unit)
+  const uint8_t *end = volt + rows * N;
+  const int64_t whole = rows - 1 - 14 / N;
   for (int64_t r = (int64_t)blockIdx.x * rpb + r_off; r < rows; r += rstride * kRepackRows) {
     for (int g = g0; g < upr; g += gstep) {
-      uint4 a[kRepackRows], b[kRepackRows];
+      Unit16 a[kRepackRows], b[kRepackRows];
       int s[kRepackRows];
 #pragma unroll
       for (int k = 0; k < kRepackRows; ++k) {
         const int64_t rk = r + k * rstride;
-        a[k] = b[k] = make_uint4(0, 0, 0, 0);
-        s[k] = 0;
-        if (rk < rows) {
-          const uint8_t *at = volt + rk * N + 16 * g;
-          s[k] = (int)(reinterpret_cast<uintptr_t>(at) & 15);
-          const uint4 *src = reinterpret_cast<const uint4 *>(at - s[k]);
-          a[k] = __ldg(src);
-          if (s[k] + min(16, N - 16 * g) > 16) b[k] = __ldg(src + 1);
-        }
+        const uint8_t *at = volt + rk * N + 16 * g;
+        const int n = min(16, N - 16 * g);
+        if (rk < whole)
+          s[k] = units_of<true>(at, n, end, LoadGlobal(), a[k], b[k]);
+        else if (rk < rows)
+          s[k] = units_of<false>(at, n, end, LoadGlobal(), a[k], b[k]);
       }
 #pragma unroll
       for (int k = 0; k < kRepackRows; ++k) {
@@ -299,8 +307,9 @@ __global__ void __launch_bounds__(256) repack_kernel(const uint8_t *__restrict__
         if (rk >= rows) break;
         // words w[s/4 ..] of the eight, then the byte shift
         const bool w2 = s[k] & 8, w1 = s[k] & 4;
-        const uint32_t x0 = w2 ? a[k].z : a[k].x, x1 = w2 ? a[k].w : a[k].y, x2 = w2 ? b[k].x : a[k].z,
-                       x3 = w2 ? b[k].y : a[k].w, x4 = w2 ? b[k].z : b[k].x, x5 = w2 ? b[k].w : b[k].y;
+        const uint32_t *p = a[k].w, *q = b[k].w;
+        const uint32_t x0 = w2 ? p[2] : p[0], x1 = w2 ? p[3] : p[1], x2 = w2 ? q[0] : p[2], x3 = w2 ? q[1] : p[3],
+                       x4 = w2 ? q[2] : q[0], x5 = w2 ? q[3] : q[1];
         const uint32_t y0 = w1 ? x1 : x0, y1 = w1 ? x2 : x1, y2 = w1 ? x3 : x2, y3 = w1 ? x4 : x3, y4 = w1 ? x5 : x4;
         const int sh = 8 * (s[k] & 3);
         *reinterpret_cast<uint4 *>(out + rk * P + 16 * (int64_t)g) =
