@@ -62,15 +62,23 @@ int max_chan_groups(int n_chan) { return n_chan < kMaxChanGroups ? n_chan : kMax
 // group's channels, `ctas` of them resident per SM: the count that leaves the
 // fewest channels to the busiest warp of the last round, rounds of CTAs times
 // channels per warp (of equal counts the largest that gives every warp a
-// channel).  At 1024 inputs that is 12 groups for 768 channels, as measured
-// best; 256 channels take 11 for the Jones pass (5 rounds of 3 channels, against
-// 6 of 3 with 12).
+// channel).  Only counts that give no warp more channels than the most groups
+// would: what a lane adds plainly (the Jones sums of a row pair or a column, the
+// gain solve's weights) is as many terms as its warp has channels, and few groups
+// would make those sums less exact (Jones gradient of 1024 inputs x 300 channels,
+// rms error against 64 bits: 3.3e-8 with the 2 groups of least cost, 2.7e-8 so; four
+// sweeps 1761 and 1857 us, 2074 with a fixed 12).  At 1024 inputs that is 12 groups for 768
+// channels, as measured best; 256 channels take 11 for the Jones pass (5 rounds
+// of 3 channels, against 6 of 3 with 12).
 int chan_groups(int tiles, int n_chan, int ctas) {
   const int64_t slots = 152 * (int64_t)ctas;
-  int best = 1;
+  const auto per_warp = [&](int n) { return (n_chan + 8 * n - 1) / (8 * n); };
+  const int most = max_chan_groups(n_chan);
+  int best = most;
   int64_t best_cost = INT64_MAX;
-  for (int n = 1; n <= max_chan_groups(n_chan) && n <= (n_chan + 7) / 8; ++n) {
-    const int64_t cost = (((int64_t)tiles * n + slots - 1) / slots) * ((n_chan + 8 * n - 1) / (8 * n));
+  for (int n = 1; n <= most && n <= (n_chan + 7) / 8; ++n) {
+    if (per_warp(n) > per_warp(most)) continue;
+    const int64_t cost = (((int64_t)tiles * n + slots - 1) / slots) * per_warp(n);
     if (cost <= best_cost) {
       best = n;
       best_cost = cost;

@@ -1,0 +1,27 @@
+"""The sums of the calibration passes at shapes with few channel groups."""
+import pytest
+import torch
+
+from test_gpu_calib import mw  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,C", [(1472, 100), (1024, 196), (768, 116)])
+def test_jones_sums_take_no_longer_chains(mw, N, C):  # noqa: F811
+    """Equal terms x of 17 bits: n of them add up exactly in FP32 while n is at
+    most 128, and with a systematic error of about 5e-6 at 416.  A lane's
+    uncompensated sum over the rows of a calibration tile and its warp's channels
+    has 2 x 32 to 3 x 32 terms when twelve groups share the channels, so it is
+    exact; what follows rounds at most 7 times (the warps' partials) and then
+    adds compensated: 12 x 2^-24 of the sum of equal signs in all."""
+    x = 127071 / 2 ** 17
+    B = N * (N + 1) // 2
+    M = torch.ones(C, B, dtype=torch.complex64, device="cuda")
+    V = torch.full((C, B), 1 - x, dtype=torch.complex64, device="cuda")
+    J = torch.eye(2, dtype=torch.complex64, device="cuda").repeat(N // 2, 1, 1)
+    _, grad = mw.calib_jones_loss_grad(V, M, J)
+    # G = sum over the other tiles and channels of R B^H (or R^H A) = 2 x in every entry
+    want = 2 * 2 * x * (N // 2 - 1) * C
+    err = (torch.view_as_real(grad).double() / want - torch.tensor([1.0, 0.0], device="cuda").double()).abs().max()
+    assert err.item() <= 12 * 2.0 ** -24, err.item() * 2 ** 24
