@@ -1,8 +1,10 @@
 """The sums of the calibration passes at shapes with few channel groups."""
+import numpy as np
 import pytest
 import torch
 
-from test_gpu_calib import mw  # noqa: F401
+import oracle
+from test_gpu_calib import mw, problem  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -25,3 +27,21 @@ def test_jones_sums_take_no_longer_chains(mw, N, C):  # noqa: F811
     want = 2 * 2 * x * (N // 2 - 1) * C
     err = (torch.view_as_real(grad).double() / want - torch.tensor([1.0, 0.0], device="cuda").double()).abs().max()
     assert err.item() <= 12 * 2.0 ** -24, err.item() * 2 ** 24
+
+
+@pytest.mark.parametrize("N", [2, 32, 33, 479, 480, 481, 512, 513, 545])
+def test_channel_gather_edges(mw, N):  # noqa: F811
+    """One to eighteen blocks of 32 inputs: contributions around whole batches of sixteen.
+    (1e-4 of the largest value, as in the other tests.)"""
+    C = 3
+    V, M, g = problem(N, C, seed=N)
+    G = np.stack([g * np.exp(0.1j * c) for c in range(C)]).astype(np.complex64)
+    Vd, Md, Gd = (torch.from_numpy(a).cuda() for a in (V, M, G))
+    _, grad = mw.calib_chan_loss_grad(Vd, Md, Gd)
+    new, _ = mw.calib_chan_solve(Vd, Md, Gd, 1)
+    for c in range(C):
+        v, m, g64 = (a.astype(np.complex128) for a in (V[c:c + 1], M[c:c + 1], G[c]))
+        want = oracle.calib_grad(v, m, g64)
+        assert np.abs(grad[c].cpu().numpy() - want).max() <= 1e-4 * np.abs(want).max()
+        h, _ = oracle.calib_solve(v, m, g64, 1)
+        assert np.abs(new[c].cpu().numpy() - h).max() <= 1e-4 * np.abs(h).max()
