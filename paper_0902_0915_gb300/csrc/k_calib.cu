@@ -58,8 +58,17 @@ struct Kahan {
 // Most channel groups of a shape (the workspaces are sized for them).
 int max_chan_groups(int n_chan) { return n_chan < kMaxChanGroups ? n_chan : kMaxChanGroups; }
 
+// SMs of the current device.
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  return n;
+}
+
 // Channel groups of a launch of `tiles` x groups CTAs whose eight warps share a
-// group's channels, `ctas` of them resident per SM: the count that leaves the
+// group's channels, `ctas` of them resident on each of `sms` SMs: the count that leaves the
 // fewest channels to the busiest warp of the last round, rounds of CTAs times
 // channels per warp (of equal counts the largest that gives every warp a
 // channel).  Only counts that give no warp more channels than the most groups
@@ -70,8 +79,8 @@ int max_chan_groups(int n_chan) { return n_chan < kMaxChanGroups ? n_chan : kMax
 // sweeps 1761 and 1857 us, 2074 with a fixed 12).  At 1024 inputs that is 12 groups for 768
 // channels, as measured best; 256 channels take 11 for the Jones pass (5 rounds
 // of 3 channels, against 6 of 3 with 12).
-int chan_groups(int tiles, int n_chan, int ctas) {
-  const int64_t slots = 152 * (int64_t)ctas;
+int chan_groups(int tiles, int n_chan, int ctas, int sms) {
+  const int64_t slots = sms * (int64_t)ctas;
   const auto per_warp = [&](int n) { return (n_chan + 8 * n - 1) / (8 * n); };
   const int most = max_chan_groups(n_chan);
   int best = most;
@@ -1094,7 +1103,7 @@ mwax_status mwax_calib_loss_grad(const float *V, const float *M, const float *g,
   if ((loss && !dev_ptr(loss)) || (grad && !dev_ptr(grad))) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas);
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count());
   Ws w = carve(workspace, nb, n_cg, false);
   launch(calib_tile_kernel<false>, false, dim3(tiles, n_cg), kCalThreads, 0, stream,
          reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M),
@@ -1124,7 +1133,7 @@ mwax_status mwax_calib_solve(const float *V, const float *M, float *g, int n_inp
   if (loss_hist && !dev_ptr(loss_hist)) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas);
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count());
   Ws w = carve(workspace, nb, n_cg, true);
   float2 *g2 = reinterpret_cast<float2 *>(g);
   for (int t = 1; t <= n_iter; ++t) {
@@ -1206,7 +1215,7 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
   const int n_tiles = n_inputs / 2;
   const int n_jt = (n_tiles + kJT - 1) / kJT;
   const int tiles = n_jt * (n_jt + 1) / 2;
-  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas);
+  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas, sm_count());
   const int64_t slots = (int64_t)tiles * n_cg;
   float *prow = reinterpret_cast<float *>(workspace);
   float *pcol = prow + slots * kJT * kJQ;
