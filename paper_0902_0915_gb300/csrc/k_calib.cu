@@ -71,22 +71,22 @@ int sm_count() {
 // group's channels, `ctas` of them resident on each of `sms` SMs: the count that leaves the
 // fewest channels to the busiest warp of the last round, rounds of CTAs times
 // channels per warp (of equal counts the largest that gives every warp a
-// channel).  Only counts that give no warp more channels than the most groups
-// would: what a lane adds plainly (the Jones sums of a row pair or a column, the
-// gain solve's weights) is as many terms as its warp has channels, and few groups
-// would make those sums less exact (Jones gradient of 1024 inputs x 300 channels,
+// channel).  plain: the pass adds some sums over a warp's channels without
+// compensation (the Jones sums of a row pair or a column, the gain solve's
+// weights), and few groups would make them less exact; then only counts that give
+// no warp more channels than the most groups would (Jones gradient of 1024 inputs x 300 channels,
 // rms error against 64 bits: 3.3e-8 with the 2 groups of least cost, 2.7e-8 so; four
 // sweeps 1761 and 1857 us, 2074 with a fixed 12).  At 1024 inputs that is 12 groups for 768
 // channels, as measured best; 256 channels take 11 for the Jones pass (5 rounds
 // of 3 channels, against 6 of 3 with 12).
-int chan_groups(int tiles, int n_chan, int ctas, int sms) {
+int chan_groups(int tiles, int n_chan, int ctas, int sms, bool plain) {
   const int64_t slots = sms * (int64_t)ctas;
   const auto per_warp = [&](int n) { return (n_chan + 8 * n - 1) / (8 * n); };
   const int most = max_chan_groups(n_chan);
   int best = most;
   int64_t best_cost = INT64_MAX;
   for (int n = 1; n <= most && n <= (n_chan + 7) / 8; ++n) {
-    if (per_warp(n) > per_warp(most)) continue;
+    if (plain && per_warp(n) > per_warp(most)) continue;
     const int64_t cost = (((int64_t)tiles * n + slots - 1) / slots) * per_warp(n);
     if (cost <= best_cost) {
       best = n;
@@ -1120,7 +1120,7 @@ mwax_status mwax_calib_loss_grad(const float *V, const float *M, const float *g,
   if ((loss && !dev_ptr(loss)) || (grad && !dev_ptr(grad))) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count());
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count(), false);
   Ws w = carve(workspace, nb, n_cg, false);
   launch(calib_tile_kernel<false>, false, dim3(tiles, n_cg), kCalThreads, 0, stream,
          reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M),
@@ -1150,7 +1150,7 @@ mwax_status mwax_calib_solve(const float *V, const float *M, float *g, int n_inp
   if (loss_hist && !dev_ptr(loss_hist)) return MWAX_ERR_INVALID_ARG;
   const int nb = (n_inputs + kCT - 1) / kCT;
   const int tiles = nb * (nb + 1) / 2;
-  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count());
+  const int n_cg = chan_groups(tiles, n_chan, kCalibCtas, sm_count(), true);
   Ws w = carve(workspace, nb, n_cg, true);
   float2 *g2 = reinterpret_cast<float2 *>(g);
   for (int t = 1; t <= n_iter; ++t) {
@@ -1234,7 +1234,7 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
   const int n_jt = (n_tiles + kJT - 1) / kJT;
   const int tiles = n_jt * (n_jt + 1) / 2;
   const int sms = sm_count();
-  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas, sms);
+  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas, sms, true);
   const int64_t slots = (int64_t)tiles * n_cg;
   float *prow = reinterpret_cast<float *>(workspace);
   float *pcol = prow + slots * kJT * kJQ;
