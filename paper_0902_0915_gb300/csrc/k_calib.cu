@@ -1075,16 +1075,18 @@ int64_t jones_ws_bytes(int n_inputs, int n_chan) {
 // Started beside it, its CTAs find the gather's on some SMs and crowd on the others,
 // and stay there.  That costs more than the launch where the gather holds over half
 // of the SMs and an ordinary launch would spread evenly: the pass's last CTA per SM
-// goes to most of the SMs, and they have room for another (`per_sm` resident on
-// each).  Measured, six sweeps as dependent / ordinary launches: Jones, 256 inputs x
-// 768 channels (120 CTAs after 80) 1057 / 680 us, 320 x 64 (120 after 96) 213 / 154;
-// per channel, 64 x 768 (288 after 288) 97 / 78, 128 x 200 (250 after 125) 83 / 78,
-// 320 x 64 (440 after 88) 105 / 93.  On the other side: Jones, 256 x 64 (80 after 80)
-// 142 / 152, 320 x 768 (180 after 96) 1152 / 1161; per channel, 192 x 64 (168 after
-// 56) 67 / 78, 224 x 90 (336 after 84) 87 / 90, 96 x 768 (576 after 384) 112 / 127.
-bool pass_waits(int64_t pass_ctas, int64_t gather_ctas, int per_sm, int sms) {
+// goes to over three fifths of the SMs, which have room for another (`per_sm` resident
+// on each), and all its warps have a channel.  Measured, six sweeps as dependent /
+// ordinary launches: Jones, 256 inputs x 768 channels (120 CTAs after 80) 1057 / 680
+// us, 320 x 64 (120 after 96) 213 / 154; per channel, 64 x 768 (288 after 288) 97 /
+// 78, 320 x 64 (440 after 88) 105 / 93.  On the other side: Jones, 256 x 64 (80 after
+// 80) 142 / 152, 320 x 768 (180 after 96) 1152 / 1161, 1024 x 1 (136 after 272, four
+// sweeps) 79 / 86; per channel, 192 x 64 (168 after 56) 67 / 78, 224 x 90 (336 after
+// 84) 87 / 90, 96 x 768 (576 after 384) 112 / 127.
+bool pass_waits(int64_t pass_ctas, int64_t gather_ctas, int cta_chans, int per_sm, int sms) {
   const int64_t last = (pass_ctas - 1) % sms + 1;
-  return 2 * gather_ctas > sms && 5 * last > 3 * sms && pass_ctas <= (per_sm - 1) * (int64_t)sms;
+  return 2 * gather_ctas > sms && 5 * last > 3 * sms && pass_ctas <= (per_sm - 1) * (int64_t)sms &&
+         cta_chans >= kCalThreads / 32;
 }
 
 template <typename... P, typename... A>
@@ -1208,7 +1210,8 @@ mwax_status mwax_calib_chan_solve(const float *V, const float *M, float *g, int 
   const int n_cy = (n_chan + kChanPerCta - 1) / kChanPerCta;
   ChanWs w = chan_carve(workspace, nb, n_chan, n_cy, true);
   float2 *g2 = reinterpret_cast<float2 *>(g);
-  const bool waits = pass_waits((int64_t)tiles * n_cy, (int64_t)(nb + 1) * n_cy, kCalibChanCtas, sm_count());
+  const bool waits = pass_waits((int64_t)tiles * n_cy, (int64_t)(nb + 1) * n_cy, (n_chan + n_cy - 1) / n_cy,
+                                kCalibChanCtas, sm_count());
   for (int t = 1; t <= n_iter; ++t) {
     launch(calib_chan_tile_kernel<true>, t > 1 && !waits, dim3(tiles, n_cy), kCalThreads, 0, stream,
            reinterpret_cast<const float2 *>(V), reinterpret_cast<const float2 *>(M), g2, n_inputs, n_chan,
@@ -1264,7 +1267,8 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
            0);
     return cudaGetLastError() == cudaSuccess ? MWAX_OK : MWAX_ERR_CUDA;
   }
-  const bool waits = pass_waits(slots, (int64_t)(n_jt + 1) * (kJT / 2), kJonesCtas, sms);
+  const bool waits =
+      pass_waits(slots, (int64_t)(n_jt + 1) * (kJT / 2), (n_chan + n_cg - 1) / n_cg, kJonesCtas, sms);
   for (int t = 1; t <= n_iter; ++t) {
     tile_pass(true, t % 2 == 0, t > 1 && !waits);
     if (cudaGetLastError() != cudaSuccess) return MWAX_ERR_CUDA;
