@@ -1237,7 +1237,11 @@ static mwax_status jones_run(const float *V, const float *M, float *J, int n_inp
   const int n_jt = (n_tiles + kJT - 1) / kJT;
   const int tiles = n_jt * (n_jt + 1) / 2;
   const int sms = sm_count();
-  const int n_cg = chan_groups(tiles, n_chan, kJonesCtas, sms, true);
+  // launches that leave half of the SMs idle even with the most groups take those: the
+  // pass is bound by issue, and its warps then share an SM with fewer others (four
+  // sweeps of 64 inputs x 24 channels 71 us, with 3 groups 89)
+  const int most = max_chan_groups(n_chan);
+  const int n_cg = 2 * tiles * most <= sms ? most : chan_groups(tiles, n_chan, kJonesCtas, sms, true);
   const int64_t slots = (int64_t)tiles * n_cg;
   float *prow = reinterpret_cast<float *>(workspace);
   float *pcol = prow + slots * kJT * kJQ;
