@@ -45,3 +45,27 @@ def test_channel_gather_edges(mw, N):  # noqa: F811
         assert np.abs(grad[c].cpu().numpy() - want).max() <= 1e-4 * np.abs(want).max()
         h, _ = oracle.calib_solve(v, m, g64, 1)
         assert np.abs(new[c].cpu().numpy() - h).max() <= 1e-4 * np.abs(h).max()
+
+
+@pytest.mark.parametrize("N,C", [(512, 96), (510, 90)])
+def test_jones_gather_loses_nothing(mw, N, C):  # noqa: F811
+    """Whole residuals below 2^14 and a model of ones: every partial sum of the pass
+    (at most 8 warps x 32 rows x 2 terms) is below 2^24 and exact, so what the gather
+    rounds is all there is.  It carries what its additions lose: the nearest FP32
+    number, where sixteen rounded sums miss it in every tenth entry."""
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    n, B = N // 2, N * (N + 1) // 2
+    R = torch.randint(1, 2 ** 14, (C, B), generator=gen, device="cuda")
+    M = torch.ones(C, B, dtype=torch.complex64, device="cuda")
+    J = torch.eye(2, dtype=torch.complex64, device="cuda").repeat(n, 1, 1)
+    # M J^H = J M has 1 in every entry, and a model block of ones is J_a M J_b^H
+    _, grad = mw.calib_jones_loss_grad((1 - R).to(torch.complex64), M, J)
+    a, b = torch.tril_indices(n, n, -1, device="cuda")
+    row = a * (2 * a + 1) + 2 * b
+    r = R.sum(0).double()
+    blk = torch.stack([r[row], r[row + 1], r[row + 2 * a + 1], r[row + 2 * a + 2]], 1).view(-1, 2, 2)
+    G = torch.zeros(n, 2, dtype=torch.float64, device="cuda")
+    G.index_add_(0, a, blk.sum(2))  # R B^H: row sums, the same in both columns
+    G.index_add_(0, b, blk.sum(1))  # R^H A: column sums
+    want = (2 * G).float()[:, :, None].expand(n, 2, 2)
+    assert (grad.real == want).all().item() and (grad.imag == 0).all().item()
