@@ -31,6 +31,8 @@
 // Salvini & Wijnholds 2014, which keeps the simultaneous update from
 // oscillating).  Working from the residual keeps the FP32 update accurate
 // near convergence, where num and g den nearly cancel.
+#include <float.h>
+
 #include <mutex>
 
 #include "mwax_internal.h"
@@ -52,6 +54,12 @@ struct Kahan {
     const float t = s + y;
     c = (t - s) - y;
     s = t;
+  }
+  // For sums that may overflow: an infinite one stays infinite (its compensation,
+  // inf - inf, would make the next sum NaN).
+  __device__ __forceinline__ void add_or_inf(float x) {
+    add(x);
+    if (!(fabsf(s) <= FLT_MAX)) c = 0.f;
   }
 };
 
@@ -239,7 +247,7 @@ __global__ void __launch_bounds__(kCalThreads, kCalibCtas) calib_tile_kernel(
   for (int nu = cg + n_cg * w; nu < C; nu += n_cg * kWarps) {
     const TileSums t = tile_channel<DEN>(V + (int64_t)nu * B, M + (int64_t)nu * B, sgi, gj, I, j,
                                                N, lane);
-    loss.add(t.loss);
+    loss.add_or_inf(t.loss);
     rre.add(t.rre);
     rim.add(t.rim);
     cre.add(t.cre);
@@ -323,7 +331,7 @@ __device__ __forceinline__ void sum_losses(const float *__restrict__ part, int64
       v[u] = i < n ? __ldcg(part + i) : 0.f;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc.add(v[u]);
+    for (int u = 0; u < 4; ++u) acc.add_or_inf(v[u]);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float s = acc.s, e = -acc.c;
@@ -338,7 +346,7 @@ __device__ __forceinline__ void sum_losses(const float *__restrict__ part, int64
     s = has ? red[2 * lane] : 0.f;
     e = has ? red[2 * lane + 1] : 0.f;
     warp_sum2(s, e);
-    if (lane == 0) *loss = s + e;
+    if (lane == 0) *loss = fabsf(s) <= FLT_MAX ? s + e : s;  // (an infinite s makes e NaN)
   }
 }
 
@@ -848,7 +856,7 @@ __global__ void __launch_bounds__(kCalThreads, kJonesCtas) calib_jones_tile2_ker
         row[m][1] += v[1];
         row[m][2] += v[2];
       }
-      loss.add(lq);
+      loss.add_or_inf(lq);
     }
   cp_async_wait<0>();
   __syncthreads();  // every warp is done with the ring
