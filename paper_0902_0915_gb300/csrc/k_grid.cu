@@ -34,10 +34,9 @@
 //      support a rectangle, so an entry stores its W column and up to 7 row
 //      factors (computed in FP64, kept in FP32, 0 outside the support) and its
 //      first column: 64 bytes up to W = 7;
-//   4. the units of work: a strip of 4 columns by 32 rows (fewer on small
-//      grids) is one warp's; strips that hold more entries than a quarter of a
+//   4. the units of work: a strip of 4 columns by 8, 16 or 32 rows is one warp's; strips that hold more entries than a quarter of a
 //      warp's even share (the centre of the uv plane) take a CTA of 4 warps,
-//      sparse ones are joined to strips of 32 columns by 16 rows.
+//      sparse ones are joined to strips of 32 columns by 8 rows.
 // Grid call (per integration): one kernel gathers the four polarisation values
 // of every baseline and channel from the int32 correlator output into its
 // entries; then each warp walks its strip row of bins by row of bins.  The
@@ -270,18 +269,45 @@ __global__ void __launch_bounds__(256) grid_weights_kernel(GridGeom g,
 // r0 + i of the bin table and reaches the unit's rows i - off .. i; row i - off
 // is complete after it.
 constexpr int kCols = 4;
-constexpr int kUnitRows = 32;
+constexpr int kUnitRows = 32;  // at most (see unit_rows)
 // Wide units: 32 columns, one entry a step, no sums across groups: a bin row costs
 // its steps alone, while each of eight narrow strips pays about 100 instructions
-// for it.  But the steps follow one another, so only strips of few entries (96 per
-// 32 rows) are joined, and the longest are handed out first.  Measured a call, up
-// to 400 entries in any order / up to 96, longest first: 69 tiles x 21 channels on
+// for it.  But the steps follow one another, so only strips of few entries a row are
+// joined, and the longest are handed out first.  Measured a call, joined up to 12
+// entries a row in any order / up to 3, longest first: 69 tiles x 21 channels on
 // 1466^2 cells, W = 7: 55 / 38 us (narrow strips alone: 63); 17 x 328 on 1420^2,
 // W = 6: 63 / 34; 100 x 200 on 2000^2, W = 5: 206 / 183; 128 x 768 on 2048^2,
-// W = 7, of which little is sparse: 548 / 541.
-constexpr int kWideCols = 32, kWideRows = 16, kWideEntries = 96;
+// W = 7, of which little is sparse: 548 / 541.  In pieces of 8 rows instead of 16, the
+// first 38 -> 35, 33 x 17 on 632^2 (units of 16 rows) 19.3 -> 19.5, 27 x 64 on
+// 1076^2 22.5 -> 21.2.
+constexpr int kWideCols = 32, kWideRows = 8, kWidePerRow = 3;
 constexpr int kWideFlag = 1 << 30;
+constexpr int kApplyWarps = 4, kApplyCtas = 4;  // of a CTA; CTAs per SM: 16 warps at up to 128 registers
 constexpr int kMaxBinRows = 40;  // >= kUnitRows + 6
+
+// Rows of a plan's units, from the half plane's rows, its column blocks, the entries
+// and the SMs.  A unit of r rows walks r + 6 bin rows, so short units cost more work,
+// and long ones leave a call with few units to wait for the longest.
+// Measured a call, in us, units of 32 / 16 / 8 rows: 128 tiles x 64 channels on 2048^2
+// cells, W = 7: 166 / 138 / 156; 92 x 24 on 932^2, W = 6: 47 / 34 / 36; 33 x 17 on
+// 632^2, W = 7: 25 / 19 / 16; 24 x 357 on 294^2, W = 5: 49 / 31 / 24.  So 16 rows, with
+// these exceptions (u units of 16 rows):
+//   8 rows under three units a warp (16 / 8: 35 x 85 on 410^2 22.7 / 21.6, 100 x 24 on
+//     800^2 39 / 35, 92 x 24 on 932^2, 2.9 a warp, 34 / 36);
+//   32 rows where most strips are joined ones anyhow (8 entries a unit and many units:
+//     69 x 21 on 1466^2 34.8, with 16 rows 38.9; 49 x 22 on 1994^2 41.0 and 44.2);
+//   32 rows above 40 entries a unit (16 or 8 to give every warp half a unit), where more
+//     of the strips are then heavy and summed in 32 parts: in 16 rows 128 x 768 on 2048^2
+//     takes 533 instead of 538 us and 128 x 256 264 instead of 288, with errors against
+//     64 bits 7 and 2 % larger.
+int unit_rows(int n_rows, int n_cb, int64_t n_ent, int sms) {
+  const auto units = [&](int r) { return (int64_t)((n_rows + r - 1) / r) * n_cb; };
+  const int64_t u = units(16), warps = (int64_t)sms * kApplyCtas * kApplyWarps;
+  if (2 * u < warps) return 8;
+  if (n_ent > 40 * u) return 2 * units(32) < warps ? 16 : 32;
+  if (u < 3 * warps) return 8;
+  return u >= 4 * warps && n_ent <= 8 * u ? 32 : 16;
+}
 
 // entries of every unit of `rows` rows and `cols` columns (unit = row segment * n_cb +
 // column block)
@@ -315,6 +341,7 @@ __global__ void __launch_bounds__(256) grid_values_kernel(const int2 *__restrict
                                                           const int2 *__restrict__ vis,
                                                           float4 *__restrict__ vals,
                                                           int *__restrict__ next) {
+  let_dependents_start();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *next = 0;  // step 2's unit counter
   const int tbl = blockIdx.x * blockDim.x + threadIdx.x;
   if (tbl >= n_tbl) return;
@@ -343,7 +370,6 @@ __global__ void __launch_bounds__(256) grid_values_kernel(const int2 *__restrict
 // zeros.  One step is G entries, one per group of 32 / G lanes.
 constexpr int kSlots = 2;
 constexpr int kChunk = 32, kRing = kSlots * kChunk;
-constexpr int kApplyWarps = 4;
 __host__ __device__ constexpr int apply_warp_bytes(int f4) {
   return kRing * (32 + 16 * f4) + (3 * kMaxBinRows + 4) * 4;
 }
@@ -545,7 +571,6 @@ __device__ __forceinline__ void strip_walk(const ApplyArgs &A, int s0, int n_bin
 constexpr int apply_smem_bytes(int f4) {
   return kApplyWarps * apply_warp_bytes(f4) + kApplyWarps * kUnitRows * 32 * 4;
 }
-constexpr int kApplyCtas = 4;  // per SM: 16 warps at up to 128 registers
 
 // Bound by instruction issue (70 % of the slots, 59 % of the instructions on the
 // FMA pipe): 56 multiply-adds, 8 multiplies and about 20 other instructions per
@@ -571,6 +596,7 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
   float *part = reinterpret_cast<float *>(sm_all + kApplyWarps * apply_warp_bytes(f4));
   const int comp = lane >> 2;
   int h = blockIdx.x;
+  wait_for_predecessor();
   while (true) {
     const bool heavy = h < A.n_heavy;
     int u = h;
@@ -585,9 +611,9 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
     const int s0 = (unit.x & ~kWideFlag) * kCols, r0 = unit.y >> 8, n_rows = unit.y & 255;
     const int c1 = min(s0 + (wide ? kWideCols : kCols) + A.W - 1, A.nbw);
     const int n_bins = n_rows + off;
-    int carry = 0;
+    int steps = 0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const int i = 32 * k + lane;
       int lo = 0, n = 0;
       if (i < n_bins) {
@@ -609,15 +635,15 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) grid_apply_kerne
       if (i < n_bins) {
         rows.q[i] = lo;
         rows.n[i] = n;
-        rows.s[i + 1] = carry + x;
+        rows.s[i + 1] = steps + x;
       }
-      carry += __shfl_sync(0xffffffffu, x, 31);
+      steps += __shfl_sync(0xffffffffu, x, 31);
     }
     if (lane == 0) rows.s[0] = 0;
     __syncwarp();
     const int s = s0 + (wide ? lane : lane & 3);
     RowOut out(A, r0, s, wide ? 0 : comp);
-    if (carry == 0 && !heavy) {
+    if (steps == 0 && !heavy) {
       const float zero[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       for (int r = 0; r < n_rows; ++r) {
         if (wide)
@@ -663,6 +689,12 @@ cudaError_t apply_one(const ApplyArgs &A, int sms, cudaStream_t s) {
     return cudaFuncSetAttribute(grid_apply_kernel<WN, F4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 apply_smem_bytes(F4 ? F4 : kMaxF4));
   const int ctas = std::min(kApplyCtas * sms, A.n_heavy + (A.n_light + kApplyWarps - 1) / kApplyWarps);
+  // beside the values kernel, whose CTAs would set how this kernel's lie on the SMs: no
+  // matter for the light units, which are handed out, but a heavy unit's CTA is fixed,
+  // and neighbouring ones are alike (95 tiles x 562 channels on 388^2 cells: 348 us, as a
+  // dependent 437; 33 x 17 on 632^2, no heavy units: 17 as an ordinary launch, 15 so)
+  if (A.n_heavy <= sms)
+    return launch_dependent(grid_apply_kernel<WN, F4>, ctas, 32 * kApplyWarps, apply_smem_bytes(A.f4), s, A);
   grid_apply_kernel<WN, F4><<<ctas, 32 * kApplyWarps, apply_smem_bytes(A.f4), s>>>(A);
   return cudaGetLastError();
 }
@@ -810,12 +842,9 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
           g, ids, n_ent, 1.0 / (2.0 * sigma * sigma), fx, n_pts, p->wts, p->slot);
     e = cudaGetLastError();
   }
-  // units: 32 rows, or fewer where that would leave CTAs without a unit; a unit
-  // of r rows walks r + 6 bin rows, so short ones cost more
   const int n_cb = Ng / kCols + 1;  // the last block holds column Ng alone
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
-  int rows = kUnitRows;
-  while (rows > 8 && (n_rows + rows - 1) / rows * n_cb < 2 * p->sms * kApplyCtas) rows /= 2;
+  const int rows = unit_rows(n_rows, n_cb, n_ent, p->sms);
   const int n_seg = (n_rows + rows - 1) / rows, per_wide = kWideCols / kCols, n_wcb = (n_cb + per_wide - 1) / per_wide;
   const int n_u = n_seg * n_cb, n_wu = n_seg * n_wcb;
   std::vector<int> cnt(n_u + n_wu);
@@ -840,7 +869,7 @@ mwax_status mwax_grid_plan(mwax_grid_plan_t *out, const double *tile_xy, int n_t
       const int r0 = seg * rows, nr = std::min(rows, n_rows - r0);
       for (int wb = 0; wb < n_wcb; ++wb) {
         const int n_wide = cnt[n_u + seg * n_wcb + wb];
-        if (n_wide <= kWideEntries * rows / kUnitRows) {
+        if (n_wide <= kWidePerRow * rows) {
           for (int r = 0; r < nr; r += kWideRows)
             wide.push_back({n_wide, make_int2(wb * per_wide | kWideFlag, (r0 + r) << 8 | std::min(kWideRows, nr - r))});
           continue;
