@@ -114,11 +114,13 @@ typedef struct {
                               least 8 + n_tiles^2 / 2 time blocks (rows that are not whole
                               16-byte units: 16 MB at least, 8 bits at most 384 inputs unless
                               odd; batch plans: where this holds for most of the
-                              operand bytes), else 3 where it applies, else 1             */
+                              operand bytes; with pipeline 2 only for 4-bit jobs of
+                              n_inputs <= 256 in whole 16-byte rows), else 3 where it
+                              applies, else 1                                             */
   int32_t pipeline;        /* tuning: 1 = unpack then correlate each channel group on the
                               plan's stream, 2 = unpack the next group (second stream,
                               second scratch buffer) while the current group correlates,
-                              see unpack_sms; 0 = auto (1)                               */
+                              see unpack_sms (mma_shape 4 unpacks nothing: 1); 0 = auto (1) */
   int32_t timeout_ms;      /* limit of every device-side wait, ms (0 = 2000)              */
   int32_t test_fault;      /* failure-detection tests only, 0 = off: with k > 0 the
                               epilogue of the tensor correlator withholds the release of

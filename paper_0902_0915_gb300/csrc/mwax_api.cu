@@ -319,12 +319,15 @@ bool fused_pays(const TcJob &j, int sample_bits) {
 // of the launch's operands, else the pair mode where every job integrates in one
 // exact segment, else narrow); -1 when an explicit pair or fused pair request
 // cannot be served (an explicit fused request takes 4-bit samples in whole-unit
-// rows only).
-int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int sample_bits) {
+// rows only).  overlap: the caller asks for an unpack beside the correlation
+// (pipeline 2), which the fused mode has none of: it is then the automatic choice
+// only for 4-bit samples in whole units of up to two tiles.
+int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int sample_bits, bool overlap) {
   const bool pair_ok = pair_mode_supported(tj.data(), (int)tj.size());
-  bool whole = true;
+  bool whole = true, small = true;
   int64_t all = 0, pays = 0;
   for (const TcJob &j : tj) {
+    small = small && j.n_tiles <= kFusedTiles;
     whole = whole && j.packed_row % 16 == 0 && sample_bits == 4;
     all += operand_bytes(j);
     if (fused_pays(j, sample_bits)) pays += operand_bytes(j);
@@ -332,7 +335,7 @@ int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int 
   if (mma_shape == 4) return pair_ok && fused_ok && whole ? 3 : -1;
   if (mma_shape == 3) return pair_ok ? 2 : -1;
   if (mma_shape == 1 || mma_shape == 2) return mma_shape - 1;
-  if (pair_ok && fused_ok && 2 * pays > all) return 3;
+  if (pair_ok && fused_ok && 2 * pays > all && !(overlap && !(whole && small))) return 3;
   return pair_ok ? 2 : 0;
 }
 
@@ -741,7 +744,7 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
                  s.n_tiles <= 255;
     if (p->checked) full[0].flush_blocks = s.kb;
     const bool fused_ok = fused_pair_supported(full.data(), 1) && !(p->checked && job->sample_bits == 4);
-    p->mode = choose_mode(job->mma_shape, full, fused_ok, job->sample_bits);
+    p->mode = choose_mode(job->mma_shape, full, fused_ok, job->sample_bits, job->pipeline == 2);
     if (p->mode < 0) {
       free_plan(p);
       return MWAX_ERR_UNSUPPORTED;
@@ -859,7 +862,7 @@ mwax_status mwax_plan_batch(mwax_plan_t *plan, const mwax_job *jobs, int n_jobs,
   // the fused pair mode (the correlate then reads each job's voltages itself: no
   // operand buffers, and an unpack graph only for the padded copies of ragged rows)
   const bool fused_ok = fused_pair_supported(tj.data(), n_jobs);
-  p->mode = choose_mode(jobs[0].mma_shape, tj, fused_ok, jobs[0].sample_bits);
+  p->mode = choose_mode(jobs[0].mma_shape, tj, fused_ok, jobs[0].sample_bits, false);
   if (p->mode < 0) {
     free_plan(p);
     return MWAX_ERR_UNSUPPORTED;
