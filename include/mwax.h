@@ -105,11 +105,11 @@ typedef struct {
                               read the packed samples and write the operand tiles into
                               shared memory, so no operand buffer and no unpack pass
                               (4-bit exact samples in one exact segment with n_inputs a
-                              multiple of 16 -- every job of a batch plan --, else
-                              MWAX_ERR_UNSUPPORTED); 0 = auto: 4 (also with 8-bit samples,
-                              the FP16 kind, a checked segment and any n_inputs, whose rows
-                              are copied to padded ones first where they are not whole
-                              4-byte words) for 4-bit jobs of n_inputs <= 256 and where the
+                              multiple of 16 -- every job of a batch plan --, and the
+                              jobs for which 0 chooses it, else MWAX_ERR_UNSUPPORTED);
+                              0 = auto: 4 (also with 8-bit samples, the FP16 kind, a checked
+                              segment and any n_inputs, whose rows are copied to padded
+                              ones first where they are not whole 4-byte words) for 4-bit jobs of n_inputs <= 256 and where the
                               operand tiles would exceed 64 MB and the integration has at
                               least 8 + n_tiles^2 / 2 time blocks (rows that are not whole
                               16-byte units: 16 MB at least, 8 bits at most 384 inputs unless
@@ -155,7 +155,8 @@ typedef struct {
   int32_t grid;              /* persistent CTAs of the correlate kernel                */
   int32_t stages;            /* shared-memory pipeline stages                          */
   int32_t prefetch;          /* K-blocks of L2 prefetch ahead of the TMA loads         */
-  int32_t mma_shape;         /* 1 = N128, 2 = N256 [Re | Im], 3 = two pairs per item   */
+  int32_t mma_shape;         /* 1 = N128, 2 = N256 [Re | Im], 3 = two pairs per item,
+                                4 = 3 with the unpack folded in                        */
   int32_t pipeline;          /* 1 = sequential, 2 = overlapped unpack/correlate        */
   int64_t scratch_bytes;     /* device scratch owned by the plan                       */
   int64_t work_items;        /* work items per call: (job, channel, tile pair), or the
@@ -171,8 +172,8 @@ typedef struct {
                                 the output is exact either way.  After a call that
                                 recomputed more than a quarter of its channels, the
                                 next 8 calls run the narrow shape directly.  Chosen
-                                when kind is exact and mma_shape and flush_blocks are
-                                auto (0) or mma_shape is 3.  0 otherwise.               */
+                                when kind is exact, flush_blocks is auto (0) and mma_shape
+                                auto, 3 or 4.  0 otherwise.                             */
   int32_t k_split;           /* time ranges per pair-mode item (largest over the jobs) */
 } mwax_plan_info;
 

@@ -319,7 +319,8 @@ bool fused_pays(const TcJob &j, int sample_bits) {
 // of the launch's operands, else the pair mode where every job integrates in one
 // exact segment, else narrow); -1 when an explicit pair or fused pair request
 // cannot be served (an explicit fused request takes 4-bit samples in whole-unit
-// rows only).  overlap: the caller asks for an unpack beside the correlation
+// rows, and whatever the automatic choice fuses, so that a plan's reported shape can
+// be asked for).  overlap: the caller asks for an unpack beside the correlation
 // (pipeline 2), which the fused mode has none of: it is then the automatic choice
 // only for 4-bit samples in whole units of up to two tiles.
 int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int sample_bits, bool overlap) {
@@ -332,7 +333,7 @@ int choose_mode(int mma_shape, const std::vector<TcJob> &tj, bool fused_ok, int 
     all += operand_bytes(j);
     if (fused_pays(j, sample_bits)) pays += operand_bytes(j);
   }
-  if (mma_shape == 4) return pair_ok && fused_ok && whole ? 3 : -1;
+  if (mma_shape == 4) return pair_ok && fused_ok && (whole || 2 * pays > all) ? 3 : -1;
   if (mma_shape == 3) return pair_ok ? 2 : -1;
   if (mma_shape == 1 || mma_shape == 2) return mma_shape - 1;
   if (pair_ok && fused_ok && 2 * pays > all && !(overlap && !(whole && small))) return 3;
@@ -740,7 +741,7 @@ mwax_status mwax_plan(mwax_plan_t *plan, const mwax_job *job, cudaStream_t strea
     // exact jobs longer than one exact segment, shape and segments left to the
     // plan: one checked optimistic segment per pair-mode item
     p->checked = job->kind == MWAX_KIND_EXACT && job->flush_blocks == 0 &&
-                 (job->mma_shape == 0 || job->mma_shape == 3) && s.flush_blocks < s.kb &&
+                 (job->mma_shape == 0 || job->mma_shape >= 3) && s.flush_blocks < s.kb &&
                  s.n_tiles <= 255;
     if (p->checked) full[0].flush_blocks = s.kb;
     const bool fused_ok = fused_pair_supported(full.data(), 1) && !(p->checked && job->sample_bits == 4);

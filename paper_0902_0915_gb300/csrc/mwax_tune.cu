@@ -194,7 +194,7 @@ mwax_status mwax_autotune(mwax_job *job, const void *voltages, void *out, cudaSt
   // Pair-mode candidates with time ranges per item fail to plan (and are
   // skipped) where the job cannot take them (FP16 kind, too few time blocks),
   // and so do the fused pair mode's (mma_shape 4) outside 4-bit exact jobs of
-  // whole 16-input sample rows.
+  // whole 16-input sample rows and the jobs for which it is the default.
   const std::vector<Cand> cands = {
       {0, 0, 0, 0, 0, 0},  {3, 0, -1, 1, 0, 1}, {3, 0, -1, 1, 0, 2}, {3, 0, -1, 1, 0, 4},
       {3, 0, -1, 1, 0, 8}, {4, 0, -1, 1, 0, 1}, {4, 0, -1, 1, 0, 2}, {4, 0, -1, 1, 0, 4},
@@ -230,7 +230,8 @@ mwax_status mwax_autotune_batch(mwax_job *jobs, int n_jobs, const void *const *v
   memset(&rep, 0, sizeof(rep));
   std::vector<mwax_job> base(jobs, jobs + n_jobs);
   // candidate 0: the batch plan's own default (all fields automatic); the
-  // fused pair mode (4) fails to plan, and is skipped, unless every job allows it
+  // fused pair mode (4) fails to plan, and is skipped, unless every job allows it or it
+  // is that default
   const std::vector<Cand> cands = {{0, 0, 0, 0, 0, 0}, {3, 0, -1, 0, 0, 0}, {4, 0, -1, 0, 0, 0},
                                    {1, 2, -1, 0, 0, 0}, {1, 2, 8, 0, 0, 0},  {2, 4, -1, 0, 0, 0},
                                    {2, 3, -1, 0, 0, 0}};
