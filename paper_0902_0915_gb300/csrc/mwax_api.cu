@@ -468,10 +468,11 @@ mwax_status correlate_group(mwax_plan_s *p, const JobState &s, const uint8_t *op
   }
   if (pair_like(p->mode)) {
     const bool full = nc == s.chan_group;  // (host path: s is its own JobState)
-    const int4 *items = host ? p->host_items : p->items;
-    const int64_t n_full = host ? p->n_host_full : p->n_items_full;
+    const bool own = host && p->host_items;
+    const int4 *items = own ? p->host_items : p->items;
+    const int64_t n_full = own ? p->n_host_full : p->n_items_full;
     cfg.items = full ? items : items + n_full;
-    cfg.n_items = full ? n_full : host ? p->n_host_last : p->n_items_last;
+    cfg.n_items = full ? n_full : own ? p->n_host_last : p->n_items_last;
     if (p->checked) tj.flush_blocks = s.kb;  // one optimistic segment per item
   }
   TimedLaunch tc(p, 1, st);
@@ -606,7 +607,7 @@ cudaError_t prepare_host_groups(mwax_plan_s *p) {
   }
   p->host_group = (int)g;
   p->host_split = s.k_split;
-  if (!pair_like(p->mode)) return cudaSuccess;
+  if (!pair_like(p->mode) || g == s.chan_group) return cudaSuccess;  // the plan's own lists serve
   std::vector<TcJob> full = {tc_job(s, nullptr, nullptr, (int)g)}, tail;
   if (p->checked) full[0].flush_blocks = s.kb;
   if (s.job.k_split == 0) {
