@@ -89,7 +89,9 @@ typedef struct {
   int32_t flush_blocks;    /* tuning: K-blocks per exact FP32 segment (0 = largest safe) */
   int32_t chan_group;      /* tuning: channels unpacked per pass (0 = auto)              */
   int32_t stages;          /* tuning: shared-memory stages: 2 narrow (3 K blocks each),
-                              2..4 wide, 2 pair (2 K blocks each) (0 = auto)               */
+                              2..4 wide, 2 pair (2 K blocks each, 3 in items of two
+                              tiles where the fused mode or a job of up to two tiles
+                              runs them) (0 = auto)                                       */
   int32_t prefetch;        /* tuning: K-blocks of L2 prefetch ahead, 1..64 (0 = auto,
                               which is none; -1 = none); narrow and wide shapes only      */
   int32_t mma_shape;       /* tuning: 1 = M128xN128 MMAs (Re, Im separately), 2 = M128xN256

@@ -285,13 +285,14 @@ int resolve_split(const mwax_job &job, int mode, int kb, int64_t base_items, int
 // conversion stops during an item's drain.  So: always for 4-bit samples of up
 // to two tiles; else when the launch's operands take over half of the L2 (64 MB)
 // and an item has enough blocks to hide the drain, the more the less each block
-// saves (8 + n_tiles^2 / 2).  Measured, fused against unpack + pair, in
-// microseconds, 4 bits: 256 inputs x 768 channels x 20,000 samples 1821 / 3449,
-// 384 x 512 x 20,000 2652 / 4004, 512 x 64 x 1000 73 / 76, 768 x 256 x 20,000 4490
-// / 5228, 1024 x 192 x 20,000 5644 / 6188, 1024 x 64 x 3000 374 / 379; 8 bits: 128 x
-// 300 x 5000 152 / 332, 512 x 96 x 10,000 929 / 1233, 1024 x 384 x 10,000 11,186 /
-// 12,069, 1024 x 64 x 2000 481 / 515; on the other side 512 x 32 x 1000 (4 bits, 33
-// MB) 50 / 47, 768 x 32 x 1000 76 / 73, 1024 x 64 x 1000 209 / 181, 1024 x 128 x 1000
+// saves (8 + n_tiles^2 / 2).  Measured back to back in one run (a call by itself, on
+// a warm chip, takes up to 8 % longer), fused against unpack + pair, in microseconds, 4
+// bits: 256 inputs x 768 channels x 20,000 samples 1729 / 3353, 384 x 512 x 20,000
+// 2517 / 3993, 512 x 64 x 1000 68 / 76, 768 x 256 x 20,000 4146 / 5165, 1024 x 192 x
+// 20,000 5164 / 6067, 1024 x 64 x 3000 356 / 378; 8 bits: 128 x 300 x 5000 139 / 328,
+// 512 x 96 x 10,000 884 / 1240, 1024 x 384 x 10,000 10,554 / 12,240, 1024 x 64 x 2000
+// 444 / 495; on the other side 512 x 32 x 1000 (4 bits, 33 MB) 47 / 48, 768 x 32 x
+// 1000 72 / 72, 1024 x 64 x 1000 197 / 181, and in an earlier run 1024 x 128 x 1000
 // (8 bits, 32 blocks) 609 / 568.
 constexpr int kFusedTiles = 2;
 constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
@@ -301,8 +302,9 @@ constexpr int64_t kFusedOperandBytes = int64_t(64) << 20;
 // wide); the extra launch needs operands of 16 MB to pay, and rows of words take
 // the same line.  8-bit rows of words leave the fused mode above three tiles, where
 // their four-byte stores cost more than the unpack (in microseconds, fused / unpack
-// + pair: 250 x 384 x 4001 484 / 748, 334 x 128 x 3000 313 / 370, 500 x 64 x 4000 423 /
-// 409, 998 x 64 x 4000 1154 / 939; odd N, copied: 999 x 64 x 4000 986 / 1192).
+// + pair: 250 x 384 x 4001 475 / 698, 334 x 128 x 3000 298 / 344; in an earlier run 500
+// x 64 x 4000 423 / 409, 998 x 64 x 4000 1154 / 939; odd N, copied: 999 x 64 x 4000
+// 971 / 1183).
 constexpr int64_t kRaggedOperandBytes = int64_t(16) << 20;
 
 int64_t operand_bytes(const TcJob &j) { return (int64_t)j.n_chan * j.n_tiles * j.kb * kTile * kRowBytes; }
