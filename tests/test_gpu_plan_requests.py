@@ -33,3 +33,34 @@ def test_overlapped_pipeline_keeps_small_arrays_fused(mw):  # noqa: F811
     p = mw.Plan(256, 8, 2000, 4, chan_group=2, pipeline=2)
     assert p.info().mma_shape == 4 and p.info().pipeline == 1
     p.close()
+
+
+@pytest.mark.parametrize("bits,N,C,blocks,shape", [
+    (4, 640, 41, 20, 4), (4, 640, 40, 20, 3), (4, 640, 60, 19, 3),  # 5 tiles: 64 MB and 8 + 25 / 2 blocks
+    (8, 896, 18, 32, 3), (8, 896, 18, 33, 4), (8, 896, 19, 32, 4),  # 7 tiles: 64 MB and 32 blocks
+    (8, 896, 40, 31, 3),
+    (4, 252, 65, 8, 4), (4, 252, 64, 8, 3),   # rows of words, two tiles: 16 MB
+    (8, 372, 110, 13, 4), (8, 500, 200, 16, 3), (8, 501, 130, 16, 4),  # 8-bit rows of words: up to three tiles
+])
+def test_fused_lines(mw, bits, N, C, blocks, shape):  # noqa: F811
+    """Both sides of each line of the automatic choice (a tile's block is 16 KB)."""
+    p = mw.Plan(N, C, blocks * (64 if bits == 4 else 32), bits)
+    assert p.info().mma_shape == shape
+    p.close()
+
+
+@pytest.mark.parametrize("N,T,C", [(256, 4000, 40), (250, 3000, 60), (255, 2500, 60)])
+def test_fused_fp16_rounds_as_the_pair_mode(mw, N, T, C):  # noqa: F811
+    """Full-scale samples, whose FP32 sums round: the same sums in the same order."""
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    v = (torch.randint(0, 2, (C * T * N * 2,), generator=gen, device="cuda") * 254 - 127).to(torch.int8).view(torch.uint8)
+    p = mw.Plan(N, C, T, 8, kind=mw.KIND_FP16)
+    q = mw.Plan(N, C, T, 8, kind=mw.KIND_FP16, mma_shape=3)
+    assert p.info().mma_shape == 4 and q.info().mma_shape == 3
+    a, b = p.correlate(v), q.correlate(v)
+    assert p.status() == 0 and q.status() == 0
+    assert a.max().item() > 2 ** 24 and torch.equal(a, b)
+    p.close()
+    q.close()
