@@ -1084,8 +1084,9 @@ int64_t jones_ws_bytes(int n_inputs, int n_chan) {
 // of all, then lets its successor start, whose launch costs nothing that way.  The
 // first one of a call is an ordinary launch.  Gains and partial sums are read
 // past L1 (__ldcg), which another kernel may have filled before they were written.
-// Measured, ten sweeps of 256 inputs x 768 channels with a gain per channel:
-// 799 us, as ordinary launches 827; four Jones sweeps of 1024 x 256: 1561, 1565.
+// Measured, ten sweeps of 256 inputs x 768 channels with a gain per channel: 799 us,
+// as ordinary launches 827 (790 now, with the gather's loads in flight together); four
+// Jones sweeps of 1024 x 256: 1561, 1565.
 // A sweep's pass is an ordinary launch where pass_waits says so.
 // Whether a sweep's pass is better launched once the gather before it has ended.
 // Started beside it, its CTAs find the gather's on some SMs and crowd on the others,
